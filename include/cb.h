@@ -428,7 +428,7 @@ int cb_topk(const double *S, uint32_t n, uint32_t k, uint32_t *idx, double *val,
  * allocation, or a latency-critical loop where an allocation might stall.
  *   Arguments, order and tie rule as cb_topk.  k <= CB_MAX_TOPK (4096);
  *   a larger k is rejected with CB_ERR_ARG and a message naming the limit.
- *   Scratch: one fixed array of about 65 KB in device memory per GPU that
+ *   Scratch: one fixed array of about 90 KB in device memory per GPU that
  *   loads the library, held until the process exits.  The first call in a
  *   CUDA context looks up that array's device address in the context
  *   (cudaGetSymbolAddress) and caches it under the context's unique id, so

@@ -2,39 +2,50 @@
 // algorithm": the recovered target is the k nodes of largest summed EBTC).
 //
 // The paper sorts all n scores (Introsort, O(n log n)).  Only the k largest
-// are needed, so this selects them by most-significant-digit radix select
-// and sorts just those k:
+// are needed, so one kernel selects a few candidates and sorts those:
 //
-//  * each score maps to an order-preserving 64-bit key (NaN lowest, -0 = +0)
-//    and the key is extended by the complemented node index, so the 96-bit
-//    composite keys are distinct and larger composite = larger score, ties
-//    to the smaller index;
-//  * pass L (L = 0..11) histograms byte L of the composite key over the
-//    elements whose bytes 0..L-1 equal the prefix found so far; the last CTA
-//    to finish picks the byte where the count from the top reaches the
-//    number still needed, and stops the passes as soon as the whole bucket
-//    is needed;
-//  * one pass collects the k elements at or above the prefix, one CTA sorts
-//    them (bitonic) and writes indices and values.
-// Up to 4096 scores, one CTA sorts them all instead (one launch).
+//  * each score maps to an order-preserving 64-bit key (NaN lowest, -0 = +0),
+//    extended by the complemented node index: the 96-bit composite keys are
+//    distinct and larger composite = larger score, ties to the smaller index;
+//  * every thread takes the largest key of its own elements.  The k-th largest
+//    of these maxima bounds the k-th largest element from below, so a radix
+//    select over one key per thread (11 bits a pass, histograms merged over
+//    the grid) gives a threshold that at least k and usually few more elements
+//    reach: the scores are read twice in all, whatever their digits;
+//  * the elements at or above the threshold are collected and sorted by one
+//    CTA (bitonic).  If more than kCand reach it (ties), or k is too large for
+//    the maxima to bound it well, the radix select runs over the composite
+//    keys of all elements instead, until at most kCand remain.
 //
-// Every pass is launched unconditionally and returns at once when the
-// selection is complete, so the sequence needs no host round trip.
+// The passes are separated by grid barriers of one cooperative launch (up to
+// one CTA per SM; a single CTA with everything in shared memory for small n).
+// Up to 4096 scores one bitonic sort of all took 17 us at n = 500 and 100 us
+// at n = 4000 (now 12 and 16 us), and above that 12 histogram passes with a
+// launch each 67 us at n = 1e5 and 250 us at n = 1e7 (now 17 and 93 us): the
+// launches, and in the first passes, where all scores share a digit, the
+// histogram's same-address atomics.
+#include <algorithm>
+
+#include "cb_grid.cuh"
 #include "cb_internal.cuh"
 
 namespace cb {
 
 namespace {
 
+constexpr uint32_t kTopkThreads = 1024;
+constexpr uint32_t kBins = 2048;   // 11-bit digits
+constexpr uint32_t kLevels = 9;    // 64 key bits as 5 x 11 + 9, then 32 index bits as 11 + 11 + 10
+constexpr uint32_t kKeyLevels = 6;
+constexpr uint32_t kCand = CB_MAX_TOPK;  // most candidates one CTA sorts
+constexpr uint32_t kFew = 1024;          // candidates after which no further pass pays
+constexpr uint32_t kOneCta = 4096;       // up to this many scores: one CTA
+
 struct TopkState {
-  unsigned long long phi;  // prefix of the 64-bit score key (unfixed bits zero)
-  uint32_t plo;            // prefix of the complemented index
-  uint32_t level;          // bytes fixed so far (0..12)
-  uint32_t krem;           // elements still needed inside the prefix bucket
-  uint32_t done;
-  uint32_t arrive;
-  uint32_t ncol;
-  uint32_t hist[256];
+  uint32_t bar;      // grid barrier
+  uint32_t ncol;     // candidates collected
+  uint32_t pad[62];
+  uint32_t hist[3][kBins];  // pass p adds into hist[p % 3]; cleared two barriers later
 };
 
 struct Cand {
@@ -43,96 +54,37 @@ struct Cand {
   uint32_t pad;
 };
 
+// order-preserving key, integer arithmetic only (FP64 compares are scarce)
 __device__ __forceinline__ unsigned long long order_key(double v) {
-  if (v != v) return 0ull;  // NaN ranks below every number
-  if (v == 0.0) v = 0.0;    // -0.0 -> +0.0
   const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned long long mag = b & 0x7fffffffffffffffull;
+  if (mag > 0x7ff0000000000000ull) return 0ull;        // NaN ranks below every number
+  if (mag == 0ull) return 0x8000000000000000ull;       // -0.0 -> +0.0
   return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
 }
 
+// bits fixed before level L, and the digit of level L
+__device__ __forceinline__ uint32_t bits_before(uint32_t L) {
+  return L <= 5 ? 11 * L : (L == 6 ? 64u : (L == 7 ? 75u : (L == 8 ? 86u : 96u)));
+}
 __device__ __forceinline__ unsigned long long mask_hi(uint32_t L) {
-  return L == 0 ? 0ull : (L >= 8 ? ~0ull : (~0ull << (64 - 8 * L)));
+  const uint32_t b = bits_before(L);
+  return b == 0 ? 0ull : (b >= 64 ? ~0ull : (~0ull << (64 - b)));
 }
 __device__ __forceinline__ uint32_t mask_lo(uint32_t L) {
-  return L <= 8 ? 0u : (L >= 12 ? ~0u : (~0u << (32 - 8 * (L - 8))));
+  const uint32_t b = bits_before(L);
+  return b <= 64 ? 0u : (b >= 96 ? ~0u : (~0u << (96 - b)));
 }
 __device__ __forceinline__ uint32_t digit(unsigned long long hi, uint32_t lo, uint32_t L) {
-  return L < 8 ? (uint32_t)((hi >> (56 - 8 * L)) & 255ull) : ((lo >> (24 - 8 * (L - 8))) & 255u);
+  if (L < 5) return (uint32_t)(hi >> (53 - 11 * L)) & 2047u;
+  if (L == 5) return (uint32_t)hi & 511u;
+  return L == 6 ? lo >> 21 : (L == 7 ? (lo >> 10) & 2047u : lo & 1023u);
 }
-
-__global__ void topk_init(TopkState *st, uint32_t k) {
-  for (int d = threadIdx.x; d < 256; d += blockDim.x) st->hist[d] = 0;
-  if (threadIdx.x == 0) {
-    st->phi = 0ull;
-    st->plo = 0u;
-    st->level = 0u;
-    st->krem = k;
-    st->done = 0u;
-    st->arrive = 0u;
-    st->ncol = 0u;
-  }
+__device__ __forceinline__ unsigned long long put_hi(uint32_t d, uint32_t L) {
+  return L < 5 ? (unsigned long long)d << (53 - 11 * L) : (L == 5 ? (unsigned long long)d : 0ull);
 }
-
-__global__ void __launch_bounds__(256) topk_pass(const double *__restrict__ S, uint32_t n,
-                                                 TopkState *st, uint32_t L) {
-  __shared__ uint32_t sh[256];
-  __shared__ int s_last;
-  if (st->done) return;
-  const unsigned long long phi = st->phi, mh = mask_hi(L);
-  const uint32_t plo = st->plo, ml = mask_lo(L);
-  sh[threadIdx.x] = 0;
-  __syncthreads();
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const unsigned long long key = order_key(__ldg(S + i));
-    const uint32_t lo = ~i;
-    if ((key & mh) == phi && (lo & ml) == plo) atomicAdd(&sh[digit(key, lo, L)], 1u);
-  }
-  __syncthreads();
-  if (sh[threadIdx.x]) atomicAdd(&st->hist[threadIdx.x], sh[threadIdx.x]);
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = (atomicAdd(&st->arrive, 1u) == gridDim.x - 1);
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  if (threadIdx.x == 0) {
-    const uint32_t krem = st->krem;
-    uint32_t cum = 0, dstar = 0, hstar = 0;
-    for (int d = 255; d >= 0; --d) {
-      const uint32_t hd = __ldcg(&st->hist[d]);
-      if (cum + hd >= krem) {
-        dstar = (uint32_t)d;
-        hstar = hd;
-        break;
-      }
-      cum += hd;
-    }
-    if (L < 8) st->phi = phi | ((unsigned long long)dstar << (56 - 8 * L));
-    else st->plo = plo | (dstar << (24 - 8 * (L - 8)));
-    const uint32_t left = krem - cum;
-    st->krem = left;
-    st->level = L + 1;
-    if (hstar == left || L + 1 >= 12) st->done = 1u;
-    st->arrive = 0u;
-  }
-  __syncthreads();
-  st->hist[threadIdx.x] = 0u;
-}
-
-__global__ void __launch_bounds__(256) topk_collect(const double *__restrict__ S, uint32_t n,
-                                                    TopkState *st, Cand *buf, uint32_t k) {
-  const uint32_t L = st->level;
-  const unsigned long long mh = mask_hi(L), phi = st->phi;
-  const uint32_t ml = mask_lo(L), plo = st->plo;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const unsigned long long key = order_key(__ldg(S + i));
-    const uint32_t lo = ~i;
-    const unsigned long long kh = key & mh;
-    if (kh > phi || (kh == phi && (lo & ml) >= plo)) {
-      const uint32_t pos = atomicAdd(&st->ncol, 1u);
-      if (pos < k) buf[pos] = Cand{key, i, 0u};
-    }
-  }
+__device__ __forceinline__ uint32_t put_lo(uint32_t d, uint32_t L) {
+  return L < 6 ? 0u : (L == 6 ? d << 21 : (L == 7 ? d << 10 : d));
 }
 
 // (key desc, idx asc) ordering: a goes before b
@@ -141,117 +93,267 @@ __device__ __forceinline__ bool before(unsigned long long ka, uint32_t ia, unsig
   return ka > kb || (ka == kb && ia < ib);
 }
 
-__global__ void __launch_bounds__(1024) topk_sort(const double *__restrict__ S, const Cand *buf,
-                                                  uint32_t k, uint32_t P, uint32_t *idx,
-                                                  double *val) {
-  extern __shared__ unsigned char s_raw[];
+// The prefix found so far and what is still needed inside it.
+struct Select {
+  unsigned long long phi;
+  uint32_t plo, krem, above;  // above: elements in higher buckets (taken already)
+};
+
+// What the passes share within a CTA.
+struct TopkShared {
+  uint32_t hist[kBins];
+  uint32_t warp[kTopkThreads / 32];
+  uint32_t digit, need, bucket, ncol;
+};
+
+// End of pass L: the histograms of the grid merged, the digit where the count
+// from the top reaches sel.krem chosen, the prefix extended.  Returns the
+// elements of the chosen bucket.  pass: passes done so far (selects the merged
+// histogram).  *ok turns false when a barrier gave up.
+__device__ uint32_t pass_end(TopkShared &sh, TopkState *st, Select &sel, uint32_t L, uint32_t &pass,
+                             uint32_t &epoch, bool *ok) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __syncthreads();
+  uint32_t h0 = sh.hist[kBins - 1 - 2 * tid], h1 = sh.hist[kBins - 2 - 2 * tid];  // from the top
+  if (gridDim.x > 1) {
+    uint32_t *g = st->hist[pass % 3];
+    if (h0) atomicAdd(&g[kBins - 1 - 2 * tid], h0);
+    if (h1) atomicAdd(&g[kBins - 2 - 2 * tid], h1);
+    if (!grid_sync(&st->bar, epoch)) *ok = false;
+    h0 = __ldcg(&g[kBins - 1 - 2 * tid]);
+    h1 = __ldcg(&g[kBins - 2 - 2 * tid]);
+    // the buffer of the previous pass: every CTA read it before this barrier,
+    // and its next use is two passes on
+    if (pass > 0)
+      for (uint32_t q = blockIdx.x * kTopkThreads + tid; q < kBins; q += gridDim.x * kTopkThreads)
+        st->hist[(pass - 1) % 3][q] = 0u;
+  }
+  ++pass;
+  const uint32_t mine = h0 + h1;
+  uint32_t incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= (uint32_t)o) incl += y;
+  }
+  if (lane == 31) sh.warp[warp] = incl;
+  __syncthreads();
+  uint32_t base = 0;
+  for (uint32_t w = 0; w < warp; ++w) base += sh.warp[w];
+  const uint32_t c0 = base + incl - mine;  // count in higher bins
+  if (c0 < sel.krem && c0 + mine >= sel.krem) {  // exactly one thread
+    const bool first = c0 + h0 >= sel.krem;
+    sh.digit = kBins - 1 - 2 * tid - (first ? 0u : 1u);
+    sh.need = sel.krem - (first ? c0 : c0 + h0);
+    sh.bucket = first ? h0 : h1;
+  }
+  __syncthreads();
+  sel.phi |= put_hi(sh.digit, L);
+  sel.plo |= put_lo(sh.digit, L);
+  sel.above += sel.krem - sh.need;
+  sel.krem = sh.need;
+  const uint32_t bucket = sh.bucket;
+  __syncthreads();
+  sh.hist[2 * tid] = sh.hist[2 * tid + 1] = 0u;
+  __syncthreads();
+  return bucket;
+}
+
+// Elements whose composite key reaches the prefix (phi, plo) go to buf, in any
+// order; their number (which may exceed kCand) is returned.
+__device__ uint32_t collect(const double *__restrict__ S, uint32_t n, unsigned long long phi,
+                            uint32_t plo, TopkShared &sh, TopkState *st, Cand *buf, uint32_t &epoch,
+                            bool *ok) {
+  uint32_t *ctr = gridDim.x > 1 ? &st->ncol : &sh.ncol;
+  const uint64_t stride = (uint64_t)gridDim.x * kTopkThreads;
+  uint64_t i = blockIdx.x * kTopkThreads + threadIdx.x;
+  auto take = [&](double v, uint32_t at) {
+    const unsigned long long key = order_key(v);
+    if (key > phi || (key == phi && ~at >= plo)) {
+      const uint32_t pos = atomicAdd(ctr, 1u);
+      if (pos < kCand) buf[pos] = Cand{key, at, 0u};
+    }
+  };
+  for (; i + 3 * stride < n; i += 4 * stride) {
+    double v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = __ldg(S + i + u * stride);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) take(v[u], (uint32_t)(i + u * stride));
+  }
+  for (; i < n; i += stride) take(__ldg(S + i), (uint32_t)i);
+  if (!grid_sync(&st->bar, epoch)) *ok = false;
+  const uint32_t c = gridDim.x > 1 ? __ldcg(&st->ncol) : sh.ncol;
+  __syncthreads();  // a second collection clears the count
+  return c;
+}
+
+// buf[0, C) sorted, the first k out.  One CTA.
+__device__ void sort_out(const double *__restrict__ S, const Cand *buf, uint32_t C, uint32_t k,
+                         unsigned char *s_raw, uint32_t *idx, double *val) {
+  uint32_t P = 32;
+  while (P < C) P <<= 1;
   unsigned long long *sk = reinterpret_cast<unsigned long long *>(s_raw);
   uint32_t *si = reinterpret_cast<uint32_t *>(sk + P);
-  for (uint32_t q = threadIdx.x; q < P; q += blockDim.x) {
-    if (q < k) { sk[q] = buf[q].key; si[q] = buf[q].idx; }
-    else { sk[q] = 0ull; si[q] = 0xffffffffu; }
+  const uint32_t q = threadIdx.x;
+  if (P <= kTopkThreads) {  // one element per thread: strides below 32 by shuffle
+    unsigned long long key = 0ull;
+    uint32_t ix = 0xffffffffu;  // after every element, NaN included
+    if (q < C) {
+      key = buf[q].key;
+      ix = buf[q].idx;
+    }
+    for (uint32_t size = 2; size <= P; size <<= 1) {
+      for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
+        unsigned long long ok2;
+        uint32_t oi;
+        if (stride >= 32) {
+          __syncthreads();
+          if (q < P) { sk[q] = key; si[q] = ix; }
+          __syncthreads();
+          ok2 = q < P ? sk[q ^ stride] : 0ull;
+          oi = q < P ? si[q ^ stride] : 0u;
+        } else {
+          ok2 = __shfl_xor_sync(0xffffffffu, key, stride);
+          oi = __shfl_xor_sync(0xffffffffu, ix, stride);
+        }
+        const bool low = (q & stride) == 0, desc = (q & size) == 0;
+        if (before(ok2, oi, key, ix) == (low == desc)) { key = ok2; ix = oi; }
+      }
+    }
+    if (q < k) {
+      idx[q] = ix;
+      val[q] = S[ix];
+    }
+    return;
+  }
+  for (uint32_t p = q; p < P; p += kTopkThreads) {
+    if (p < C) { sk[p] = buf[p].key; si[p] = buf[p].idx; }
+    else { sk[p] = 0ull; si[p] = 0xffffffffu; }
   }
   __syncthreads();
   for (uint32_t size = 2; size <= P; size <<= 1) {
     for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
-      for (uint32_t q = threadIdx.x; q < P; q += blockDim.x) {
-        const uint32_t p = q ^ stride;
-        if (p > q) {
-          const bool desc = (q & size) == 0;  // first half of each block in final order
-          const bool swap = desc ? before(sk[p], si[p], sk[q], si[q])
-                                 : before(sk[q], si[q], sk[p], si[p]);
+      for (uint32_t a = q; a < P; a += kTopkThreads) {
+        const uint32_t p = a ^ stride;
+        if (p > a) {
+          const bool desc = (a & size) == 0;  // first half of each block in final order
+          const bool swap = desc ? before(sk[p], si[p], sk[a], si[a])
+                                 : before(sk[a], si[a], sk[p], si[p]);
           if (swap) {
-            const unsigned long long tk = sk[q]; sk[q] = sk[p]; sk[p] = tk;
-            const uint32_t ti = si[q]; si[q] = si[p]; si[p] = ti;
+            const unsigned long long tk = sk[a]; sk[a] = sk[p]; sk[p] = tk;
+            const uint32_t ti = si[a]; si[a] = si[p]; si[p] = ti;
           }
         }
       }
       __syncthreads();
     }
   }
-  for (uint32_t q = threadIdx.x; q < k; q += blockDim.x) {
-    idx[q] = si[q];
-    val[q] = S[si[q]];
+  for (uint32_t p = q; p < k; p += kTopkThreads) {
+    idx[p] = si[p];
+    val[p] = S[si[p]];
   }
 }
 
-// n <= kTopkSmallN: one CTA sorts all n composite keys (bitonic, in shared
-// memory, the same order as topk_sort) and writes the first k -- one launch
-// instead of the 15 of the radix select.
-constexpr uint32_t kTopkSmallN = 4096;
-
-__global__ void __launch_bounds__(1024) topk_small(const double *__restrict__ S, uint32_t n,
-                                                   uint32_t k, uint32_t P, uint32_t *idx,
-                                                   double *val) {
-  extern __shared__ unsigned char s_raw[];
-  unsigned long long *sk = reinterpret_cast<unsigned long long *>(s_raw);
-  uint32_t *si = reinterpret_cast<uint32_t *>(sk + P);
-  for (uint32_t q = threadIdx.x; q < P; q += blockDim.x) {
-    if (q < n) { sk[q] = order_key(S[q]); si[q] = q; }
-    else { sk[q] = 0ull; si[q] = 0xffffffffu; }  // after every element, NaN included
-  }
+// st and gbuf: the grid's scratch (st zeroed); unused by a single CTA, whose
+// candidates stay in shared memory (kCand of them fit beside the sort).
+__global__ void __launch_bounds__(kTopkThreads, 1) topk_kernel(const double *__restrict__ S, uint32_t n,
+                                                               uint32_t k, TopkState *st, Cand *gbuf,
+                                                               uint32_t *idx, double *val) {
+  extern __shared__ __align__(16) unsigned char s_raw[];
+  __shared__ TopkShared sh;
+  const uint32_t tid = threadIdx.x;
+  const uint64_t stride = (uint64_t)gridDim.x * kTopkThreads, i0 = blockIdx.x * kTopkThreads + tid;
+  Cand *buf = gridDim.x > 1 ? gbuf : reinterpret_cast<Cand *>(s_raw + kCand * 12);
+  uint32_t epoch = 0, pass = 0, C = kCand + 1;
+  bool ok = true;
+  sh.hist[2 * tid] = sh.hist[2 * tid + 1] = 0u;
+  if (tid == 0) sh.ncol = 0u;
   __syncthreads();
-  for (uint32_t size = 2; size <= P; size <<= 1) {
-    for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
-      for (uint32_t q = threadIdx.x; q < P; q += blockDim.x) {
-        const uint32_t p = q ^ stride;
-        if (p > q) {
-          const bool desc = (q & size) == 0;
-          const bool swap = desc ? before(sk[p], si[p], sk[q], si[q])
-                                 : before(sk[q], si[q], sk[p], si[p]);
-          if (swap) {
-            const unsigned long long tk = sk[q]; sk[q] = sk[p]; sk[p] = tk;
-            const uint32_t ti = si[q]; si[q] = si[p]; si[p] = ti;
-          }
-        }
-      }
-      __syncthreads();
+  const uint32_t maxima = (uint32_t)min((uint64_t)n, stride);  // threads that hold an element
+  if (k <= maxima / 4 || maxima == n) {
+    // threshold: the k-th largest of the threads' maxima, to kFew candidates
+    unsigned long long my = 0ull;
+    uint64_t i = i0;
+    for (; i + 3 * stride < n; i += 4 * stride) {
+      double v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = __ldg(S + i + u * stride);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) my = max(my, order_key(v[u]));
     }
+    for (; i < n; i += stride) my = max(my, order_key(__ldg(S + i)));
+    Select sel{0ull, 0u, k, 0u};
+    for (uint32_t L = 0; L < kKeyLevels && ok; ++L) {
+      if (i0 < n && (my & mask_hi(L)) == sel.phi) atomicAdd(&sh.hist[digit(my, 0u, L)], 1u);
+      const uint32_t bucket = pass_end(sh, st, sel, L, pass, epoch, &ok);
+      if (sel.above + bucket <= max(kFew, k) || sel.krem == bucket) break;
+    }
+    if (ok) C = collect(S, n, sel.phi, 0u, sh, st, buf, epoch, &ok);
   }
-  for (uint32_t q = threadIdx.x; q < k; q += blockDim.x) {
-    idx[q] = si[q];
-    val[q] = S[si[q]];
+  if (C > kCand && ok) {  // uniform over the grid: the composite keys of all elements
+    if (tid == 0) {
+      if (gridDim.x == 1) sh.ncol = 0u;
+    }
+    Select sel{0ull, 0u, k, 0u};
+    for (uint32_t L = 0; L < kLevels && ok; ++L) {
+      const unsigned long long mh = mask_hi(L);
+      const uint32_t ml = mask_lo(L);
+      for (uint64_t i = i0; i < n; i += stride) {
+        const unsigned long long key = order_key(__ldg(S + i));
+        const uint32_t lo = ~(uint32_t)i;
+        if ((key & mh) == sel.phi && (lo & ml) == sel.plo) atomicAdd(&sh.hist[digit(key, lo, L)], 1u);
+      }
+      // no CTA still reads the count of the first collection after the first barrier
+      const uint32_t bucket = pass_end(sh, st, sel, L, pass, epoch, &ok);
+      if (L == 0 && gridDim.x > 1 && blockIdx.x == 0 && tid == 0) st->ncol = 0u;
+      if (L > 0 && (sel.above + bucket <= max(kFew, k) || sel.krem == bucket)) break;
+    }
+    if (ok) C = collect(S, n, sel.phi, sel.plo, sh, st, buf, epoch, &ok);
   }
+  if (blockIdx.x != 0) return;
+  if (!ok || C > kCand || C < k) {  // a barrier gave up: no selection
+    for (uint32_t p = tid; p < k; p += kTopkThreads) {
+      idx[p] = 0xffffffffu;
+      val[p] = __longlong_as_double(0x7ff8000000000000ll);
+    }
+    return;
+  }
+  sort_out(S, buf, C, k, s_raw, idx, val);
 }
 
 }  // namespace
 
 int topk_launch(const double *S, uint32_t n, uint32_t k, uint32_t *idx, double *val,
                 void *scratch, cudaStream_t s) {
-  if (n <= kTopkSmallN) {
-    uint32_t P = 1;
-    while (P < n) P <<= 1;
-    const int tok = prof_begin(CB_K_TOPK, s);
-    topk_small<<<1, 1024, (size_t)P * (sizeof(unsigned long long) + sizeof(uint32_t)), s>>>(S, n, k, P,
-                                                                                          idx, val);
-    prof_end(tok, s);
-    return cuda_error(cudaGetLastError(), "topk launch");
-  }
-  TopkState *st = reinterpret_cast<TopkState *>(scratch);
-  Cand *buf = reinterpret_cast<Cand *>(reinterpret_cast<char *>(scratch) +
-                                       ((sizeof(TopkState) + 255) / 256) * 256);
-  uint32_t grid = (n + 256 * 8 - 1) / (256 * 8);
-  if (grid > 152 * 8) grid = 152 * 8;
-  if (grid == 0) grid = 1;
-  prefer_shared(topk_init);
-  prefer_shared(topk_pass);
-  prefer_shared(topk_collect);
-  prefer_shared(topk_sort);
+  // shared memory: the sort's arrays, and for a single CTA its candidates too
+  constexpr size_t kSort = (size_t)kCand * 12, kAll = kSort + (size_t)kCand * sizeof(Cand);
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAll);
+  if (e != cudaSuccess) return cuda_error(e, "topk launch");
   const int tok = prof_begin(CB_K_TOPK, s);
-  topk_init<<<1, 256, 0, s>>>(st, k);
-  for (uint32_t L = 0; L < 12; ++L) topk_pass<<<grid, 256, 0, s>>>(S, n, st, L);
-  topk_collect<<<grid, 256, 0, s>>>(S, n, st, buf, k);
-  uint32_t P = 1;
-  while (P < k) P <<= 1;
-  const size_t shm = (size_t)P * (sizeof(unsigned long long) + sizeof(uint32_t));
-  topk_sort<<<1, 1024, shm, s>>>(S, buf, k, P, idx, val);
+  if (n <= kOneCta) {
+    topk_kernel<<<1, kTopkThreads, kAll, s>>>(S, n, k, nullptr, nullptr, idx, val);
+  } else {
+    TopkState *st = reinterpret_cast<TopkState *>(scratch);
+    Cand *buf = reinterpret_cast<Cand *>(st + 1);
+    // four scores per thread up to one CTA per SM: a barrier over fewer CTAs is cheaper
+    const uint32_t grid = std::min<uint32_t>((uint32_t)sms, (n + 4 * kTopkThreads - 1) / (4 * kTopkThreads));
+    e = cudaMemsetAsync(st, 0, sizeof(TopkState), s);
+    void *args[] = {&S, &n, &k, &st, &buf, &idx, &val};
+    if (e == cudaSuccess)
+      e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(topk_kernel), dim3(grid),
+                                      dim3(kTopkThreads), args, kSort, s);
+  }
   prof_end(tok, s);
-  return cuda_error(cudaGetLastError(), "topk launch");
+  if (e == cudaSuccess) e = cudaGetLastError();
+  return cuda_error(e, "topk launch");
 }
 
-size_t topk_scratch_bytes(uint32_t k) {
-  return ((sizeof(TopkState) + 255) / 256) * 256 + (size_t)k * sizeof(Cand);
-}
+size_t topk_scratch_bytes(uint32_t /*k*/) { return sizeof(TopkState) + (size_t)kCand * sizeof(Cand); }
 
 }  // namespace cb
 
@@ -281,7 +383,7 @@ CB_API int cb_topk(const double *S, uint32_t n, uint32_t k, uint32_t *idx, doubl
 // / cudaMallocAsync, a plug-in whose host forbids CUDA allocation calls, or a
 // latency-critical loop where an allocation could stall on the device.  This
 // variant uses a fixed file-scope device array instead, sized for the
-// largest k the library accepts (CB_MAX_TOPK), about 65 KB per device.  It
+// largest k the library accepts (CB_MAX_TOPK), about 90 KB per device.  It
 // runs the same kernels as cb_topk.
 // ---------------------------------------------------------------------------
 #include <mutex>
@@ -289,8 +391,7 @@ CB_API int cb_topk(const double *S, uint32_t n, uint32_t k, uint32_t *idx, doubl
 namespace cb {
 namespace {
 
-constexpr size_t kNoAllocScratchBytes =
-    ((sizeof(TopkState) + 255) / 256) * 256 + (size_t)CB_MAX_TOPK * sizeof(Cand);
+constexpr size_t kNoAllocScratchBytes = sizeof(TopkState) + (size_t)kCand * sizeof(Cand);
 
 // Shared by every cb_topk_noalloc call on a device; resident until exit.
 __device__ __align__(256) unsigned char g_topk_noalloc_scratch[kNoAllocScratchBytes];
@@ -376,7 +477,7 @@ CB_API int cb_topk_noalloc(const double *S, uint32_t n, uint32_t k, uint32_t *id
   void *scratch = nullptr;
   int rc = noalloc_scratch(&scratch);
   if (rc != CB_OK) return rc;
-  // topk_launch's first kernel resets every counter and histogram in the
-  // scratch, so the previous call's contents need no clearing here.
+  // topk_launch clears every counter and histogram in the scratch first, so
+  // the previous call's contents need no clearing here.
   return topk_launch(S, n, k, idx, val, scratch, reinterpret_cast<cudaStream_t>(stream));
 }

@@ -67,61 +67,67 @@ static int ensure_backwork(cb_graph *h, uint32_t m, int prec, cudaStream_t s) {
   return cuda_error(cudaMemsetAsync(B.blob, 0, bytes, s), "adjoint workspace clear");
 }
 
-// One warp per realisation: theta_r and the coefficient matrix K_r = M_r.
-__global__ void __launch_bounds__(32) bw_tridiag_kernel(Scalars s1, Scalars sw,
+// Two warps per realisation: theta_r and the coefficient matrix K_r = M_r.
+// Warp 0 solves for the basis from w, warp 1 for the one from 1 (on sub-cores
+// of their own: each has its FP64 unit).
+__global__ void __launch_bounds__(64) bw_tridiag_kernel(Scalars s1, Scalars sw,
                                                         const InstDesc *inst, double *K,
                                                         uint32_t kdim, double *theta_out,
-                                                        uint32_t *cnt_out) {
+                                                        uint32_t *cnt_out, contour::Nodes nd) {
   using namespace contour;
-  __shared__ double s_a1[kMaxAdjM], s_b1[kMaxAdjM], s_aw[kMaxAdjM], s_bw[kMaxAdjM];
-  __shared__ cplx s_x[kHalf][kMaxAdjM], s_y[kHalf][kMaxAdjM];
-  __shared__ double s_th[2];
-  const uint32_t r = blockIdx.x, lane = threadIdx.x;
+  extern __shared__ double s_dyn[];
+  Solve *s_s = reinterpret_cast<Solve *>(s_dyn);  // [2]
+  __shared__ double s_al[2][kMaxAdjM], s_be[2][kMaxAdjM];
+  __shared__ double s_th[2], s_scale[2];
+  __shared__ cplx s_inv0[2][kHalf];
+  const uint32_t r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
   const int M1 = (int)s1.meff[r], Mw = (int)sw.meff[r];
   const bool ok = M1 > 0 && Mw > 0 && s1.status[r] == CB_OK && sw.status[r] == CB_OK;
   if (!ok) {
-    if (lane == 0) {
+    if (tid == 0) {
       theta_out[r] = -1e308;
       cnt_out[r] = 0;
     }
     return;
   }
-  for (int i = lane; i < M1; i += 32) {
-    s_a1[i] = s1.alpha[r * s1.ms + i];
-    s_b1[i] = s1.beta[r * s1.ms + i];
-  }
-  for (int i = lane; i < Mw; i += 32) {
-    s_aw[i] = sw.alpha[r * sw.ms + i];
-    s_bw[i] = sw.beta[r * sw.ms + i];
+  const Scalars &sc = wp ? s1 : sw;
+  const int M = wp ? M1 : Mw;
+  for (int i = lane; i < M; i += 32) {
+    s_al[wp][i] = sc.alpha[r * sc.ms + i];
+    s_be[wp][i] = sc.beta[r * sc.ms + i];
   }
   __syncwarp();
-  if (lane == 0) s_th[0] = lambda_max(s_a1, s_b1, M1);
-  if (lane == 1) s_th[1] = lambda_max(s_aw, s_bw, Mw);
-  __syncwarp();
+  const double th = lambda_max(s_al[wp], s_be[wp], M, reinterpret_cast<float *>(s_s[wp].phi));
+  if (lane == 0) s_th[wp] = th;
+  __syncthreads();
   const double theta = fmax(s_th[0], s_th[1]);
-  if (lane < kHalf) {
-    cplx z, w;
-    node((int)lane, &z, &w);
-    cplx cp[kMaxAdjM], x[kMaxAdjM];
-    thomas_e1(s_aw, s_bw, Mw, theta, z, cp, x);
-    for (int i = 0; i < Mw; ++i) s_x[lane][i] = cmul(w, x[i]);
-    thomas_e1(s_a1, s_b1, M1, theta, z, cp, x);
-    for (int i = 0; i < M1; ++i) s_y[lane][i] = x[i];
+  cplx inv0;
+  const double scale = continuants(s_al[wp], s_be[wp], M, theta, nd, s_s[wp], &inv0);
+  if (lane < kCols && !(lane & 1)) s_inv0[wp][lane >> 1] = inv0;
+  if (lane == 0) s_scale[wp] = scale;
+  __syncthreads();
+  // x_k of the basis from w in place of its continuants, with the node's weight
+  // and both 1 / phi_0 folded in
+  for (int t = tid; t < Mw * kHalf; t += 64) {
+    const int i = t / kHalf, k = t % kHalf;
+    double *x = s_s[0].phi + i * kCols + 2 * k;
+    const cplx v = cmul(cmul(cmul(nd.w[k], s_inv0[0][k]), s_inv0[1][k]), {x[0], x[1]});
+    x[0] = v.re;
+    x[1] = -v.im;  // the product below takes the real part
   }
-  __syncwarp();
+  __syncthreads();
   // ||w|| = 1 / scale_w[0], sqrt(n) = 1 / scale_1[0]
-  const double c = 1.0 / (sw.scale[r * sw.ms] * s1.scale[r * s1.ms]);
+  const double c = 2.0 * s_scale[0] * s_scale[1] / (sw.scale[r * sw.ms] * s1.scale[r * s1.ms]);
   double *Kr = K + (size_t)r * kdim * kdim;
-  for (int q = lane; q < Mw * M1; q += 32) {
+  for (int q = tid; q < Mw * M1; q += 64) {
     const int a = q / M1, b = q % M1;
+    const double *x = s_s[0].phi + a * kCols, *y = s_s[1].phi + b * kCols;
     double acc = 0.0;
-    for (int k = 0; k < kHalf; ++k) {
-      const cplx xa = s_x[k][a], yb = s_y[k][b];
-      acc += xa.re * yb.re - xa.im * yb.im;
-    }
-    Kr[a * kdim + b] = 2.0 * c * acc;
+#pragma unroll
+    for (int k = 0; k < kCols; ++k) acc = fma(x[k], y[k], acc);
+    Kr[a * kdim + b] = c * (s_s[0].B[a] * s_s[1].B[b]) * acc;
   }
-  if (lane == 0) {
+  if (tid == 0) {
     theta_out[r] = theta;
     const double sw0 = sw.scale[r * sw.ms];
     cnt_out[r] = (uint32_t)llrint(1.0 / (sw0 * sw0));
@@ -356,7 +362,10 @@ static int backward_t(cb_graph *h, uint32_t m, const uint32_t *idx, uint32_t k, 
   prefer_shared(bw_node_kernel<T>);
   prefer_shared(bw_edge_kernel<T>);
   const int tok = prof_begin(CB_K_BACKWARD, s);
-  bw_tridiag_kernel<<<N, 32, 0, s>>>(h->ws.sc, h->ws2.sc, h->d_inst, B.K, m, B.theta, B.cnt);
+  const size_t shm_tri = 2 * sizeof(contour::Solve);
+  cudaFuncSetAttribute(bw_tridiag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_tri);
+  bw_tridiag_kernel<<<N, 64, shm_tri, s>>>(h->ws.sc, h->ws2.sc, h->d_inst, B.K, m, B.theta, B.cnt,
+                                           contour::nodes());
   const size_t shm = (size_t)(m * m + 8 * m * 32) * sizeof(T);
   auto nk = bw_node_kernel<T>;
   if (shm > 48 * 1024) cudaFuncSetAttribute(nk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);

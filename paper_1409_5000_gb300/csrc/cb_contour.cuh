@@ -1,20 +1,18 @@
 // FP64 building blocks for functions of the small Lanczos tridiagonal T.
 //
-//  * lambda_max: the largest eigenvalue of T by Laguerre's iteration on
-//    det(xI - T), started above the Gershgorin bound.  For a polynomial
-//    with only real roots, Laguerre's method started above the largest root
-//    decreases monotonically to it and converges cubically.  f'/f and f''/f
-//    come from the ratio form of the three-term determinant recurrence
-//    (r_k = p_k / p_{k-1}), which cannot overflow.
+//  * lambda_max: the largest eigenvalue of T, bracketed in FP32 by a warp-wide
+//    multisection on the signs of the pivots of xI - T, then the FP64 Rayleigh
+//    quotient of an eigenvector from inverse iteration.
 //  * contour nodes: exp(x) on (-inf, 0] as the trapezoid rule for the
 //    Cauchy integral over the cotangent contour of Trefethen, Weideman &
 //    Schmelzer ("Talbot quadratures and rational approximations", BIT 46,
 //    2006): z(t) = N (a t cot(b t) - c + i d t), N = 24, error ~2e-14.
 //    Nodes come in conjugate pairs; only the 12 in the upper half plane are
 //    evaluated and the real result is 2 Re of their sum.
-//  * thomas_e1: (z I - (T - theta I))^{-1} e1 for complex z (Thomas
-//    algorithm; z I - S is complex symmetric tridiagonal).
+//  * continuants: (z I - (T - theta I))^{-1} e1 for the 12 nodes z at once.
 #pragma once
+
+#include <cmath>
 
 #include "cb_internal.cuh"
 
@@ -23,8 +21,7 @@ namespace contour {
 
 constexpr int kNodes = 24;
 constexpr int kHalf = kNodes / 2;
-constexpr double kA = 0.5017, kB = 0.6407, kC = 0.6122, kD = 0.2645;
-constexpr double kPi = 3.14159265358979323846;
+constexpr long double kA = 0.5017L, kB = 0.6407L, kC = 0.6122L, kD = 0.2645L;
 
 struct cplx {
   double re, im;
@@ -37,124 +34,287 @@ __device__ __forceinline__ cplx cinv(cplx a) {
   return {a.re * d, -a.im * d};
 }
 
-// f'/f and (f'/f)^2 - f''/f of f(x) = det(xI - T) via the ratios
-// r_k = p_k / p_{k-1} of the leading principal minors and their derivatives
-// (one reciprocal per k).  Returns false if some r_k <= 0, i.e. x is not
-// above every eigenvalue of every leading block.  R is float or double.
-template <typename R>
-__device__ inline bool laguerre_terms(const double *al, const double *be, int M, R x, R *G,
-                                      R *H) {
-  R r = x - (R)al[0], rd = R(1), rdd = R(0);
-  if (!(r > R(0))) return false;
-  R ir = R(1) / r;
-  R g = rd * ir;
-  R h = g * g - rdd * ir;
-  for (int k = 1; k < M; ++k) {
-    const R b2 = (R)be[k - 1] * (R)be[k - 1];
-    const R q = b2 * ir;
-    const R nr = (x - (R)al[k]) - q;
-    const R nrd = R(1) + q * ir * rd;
-    const R nrdd = q * ir * (rdd - R(2) * rd * rd * ir);
-    r = nr;
-    rd = nrd;
-    rdd = nrdd;
-    if (!(r > R(0))) return false;
-    ir = R(1) / r;
-    const R gk = rd * ir;
-    g += gk;
-    h += gk * gk - rdd * ir;
-  }
-  *G = g;
-  *H = h;
-  return true;
+// 1 / r for r in the normal FP32 range: an FP32 reciprocal refined by two
+// Newton-Raphson steps y <- y + y (1 - r y), which double the correct bits
+// each (23 -> 46 -> all).
+__device__ __forceinline__ double rcp_nr(double r) {
+  double y = (double)__frcp_rn((float)r);
+  y = fma(y, fma(-r, y, 1.0), y);
+  return fma(y, fma(-r, y, 1.0), y);
 }
 
-// One Laguerre step from x (above the largest root); false when x is not
-// above the spectrum or the step is not finite.
-template <typename R>
-__device__ inline bool laguerre_step(const double *al, const double *be, int M, R x, R *step) {
-  R G, H;
-  if (!laguerre_terms<R>(al, be, M, x, &G, &H)) return false;
-  const R disc = (R)(M - 1) * ((R)M * H - G * G);
-  const R den = G + sqrt(disc > R(0) ? disc : R(0));
-  if (!(den > R(0))) return false;
-  *step = (R)M / den;
-  return true;
-}
-
-// Largest eigenvalue of tridiag(be, al, be) (be[0..M-2] used).  Laguerre's
-// iteration from above the Gershgorin bound runs in FP32 until its step is
-// below 1e-6 relative (FP64 arithmetic is scarce on GB300), then two FP64
-// steps polish the result: the convergence is cubic, so the FP32 estimate
-// turns into an FP64-accurate one.  theta only has to lie within rounding
-// of lambda_max for the contour rule to keep its accuracy.
-__device__ inline double lambda_max(const double *al, const double *be, int M) {
+// Largest eigenvalue of tridiag(be, al, be) (be[0..M-2] used, positive), by
+// one full warp; every lane gets it.  al and be are in shared memory; f is
+// shared scratch of 5 M floats.
+//
+// An FP64 instruction of one warp occupies its sub-core's FP64 unit for about
+// 64 cycles whatever its active lanes (0.5 lanes per clock), so the serial
+// recurrences run in FP32 and FP64 only takes the few operations that set the
+// accuracy, spread over the lanes:
+//  1. FP32 multisection: x lies above the spectrum iff every pivot of xI - T
+//     is positive; the 32 lanes test 32 points of the bracket at once, so a
+//     round costs M dependent FP32 steps and gains a factor of 33; four
+//     rounds reach FP32 resolution, sigma just above lambda_max.
+//  2. two inverse iterations with sigma I - T (positive definite) in FP32.
+//  3. the Rayleigh quotient in FP64, as rho + v.(T - rho)v / v.v from rho =
+//     sigma, one correction of v from its FP64 residual by an FP32 solve, and
+//     the quotient again: the error of the quotient is the square of v's, which
+//     the correction takes from FP32 rounding to below 1e-9.  A cluster (the
+//     copies of lambda_max in an unreorthogonalised T) gives a value inside it.
+// tridiag_kernel with this and the continuants below: 79 -> 20 us at M = 20,
+// 131 -> 25 us at M = 30, 220 -> 34 us at M = 40 (before: one lane running
+// Laguerre's iteration in FP32 and twice in FP64, and a Thomas sweep with a
+// complex reciprocal per row and lane).
+__device__ inline double lambda_max(const double *al, const double *be, int M, float *f) {
   if (M == 1) return al[0];
-  double x0 = -1e300;
-  for (int i = 0; i < M; ++i) {
-    const double lo = i > 0 ? fabs(be[i - 1]) : 0.0;
-    const double hi = i < M - 1 ? fabs(be[i]) : 0.0;
-    x0 = fmax(x0, al[i] + lo + hi);
+  const int lane = threadIdx.x & 31;
+  float *fa = f, *fb = f + M, *fl = f + 2 * M, *fi = f + 3 * M, *fv = f + 4 * M;
+  float hi = -3.0e38f, lo = -3.0e38f, amax = 0.f;
+  for (int i = lane; i < M; i += 32) {
+    const float a = (float)al[i], b0 = i > 0 ? fabsf((float)be[i - 1]) : 0.f;
+    const float b1 = i < M - 1 ? fabsf((float)be[i]) : 0.f;
+    fa[i] = a;
+    fb[i] = b1;
+    hi = fmaxf(hi, a + b0 + b1);
+    lo = fmaxf(lo, a);
+    amax = fmaxf(amax, fabsf(a) + b0 + b1);
   }
-  x0 += 1e-3 * (fabs(x0) + 1.0);  // strictly above the spectrum, also in FP32
-  float xf = (float)x0;
-  if ((double)xf < x0) xf = nextafterf(xf, 3.0e38f);
-  float st;
-  if (laguerre_step<float>(al, be, M, xf, &st)) {
-    for (int it = 0; it < 40; ++it) {
-      const float nx = xf - st;
-      float st2;
-      if (!laguerre_step<float>(al, be, M, nx, &st2)) break;  // nx not above: keep xf
-      xf = nx;
-      st = st2;
-      if (st <= 1e-6f * (fabsf(xf) + 1.0f)) break;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    lo = fmaxf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+  }
+  __syncwarp();
+  auto next_pivot = [](float x, float a, float b, float r) {  // no contraction: the same in both uses
+    return __fsub_rn(__fsub_rn(x, a), __fdividef(__fmul_rn(b, b), r));
+  };
+  hi += 4e-6f * (amax + 1e-30f);  // Gershgorin: strictly above the spectrum, also in FP32
+  for (int round = 0; round < 4; ++round) {
+    const float x = lo + (hi - lo) * ((float)(lane + 1) * (1.0f / 33.0f));
+    float r = x - fa[0];
+    bool above = r > 0.f;
+#pragma unroll 4
+    for (int k = 1; k < M; ++k) {
+      r = next_pivot(x, fa[k], fb[k - 1], r);
+      above = above && r > 0.f;  // r is meaningless after the first r <= 0
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, above);
+    const int first = m ? __ffs(m) - 1 : 32;  // lowest point above the spectrum
+    const float xl = __shfl_sync(0xffffffffu, x, first > 0 ? first - 1 : 0);
+    const float xh = __shfl_sync(0xffffffffu, x, first < 32 ? first : 31);
+    if (first > 0) lo = xl;
+    if (first < 32) hi = xh;
+  }
+  // sigma I - T = L D L^T, sigma = hi: fl = -L's off-diagonal, fi = 1 / D; the
+  // pivots are those of the test that placed hi, so all are positive and the
+  // solves below stay bounded (every lane runs the serial loops; lane 0 writes)
+  float r = hi - fa[0];
+  for (int k = 0; k < M; ++k) {
+    if (k) r = next_pivot(hi, fa[k], fb[k - 1], r);
+    const float ir = __fdividef(1.0f, fmaxf(r, 1e-9f * amax + 1e-30f));
+    if (lane == 0) {
+      fi[k] = ir;
+      fl[k] = fb[k] * ir;
+      fv[k] = 1.0f;
     }
   }
-  double x = xf;
-  for (int it = 0; it < 2; ++it) {  // FP64 polish (a failed step leaves x above the root)
-    double sd;
-    if (!laguerre_step<double>(al, be, M, x, &sd)) break;
-    x -= sd;
+  __syncwarp();
+  // fv <- (sigma I - T)^{-1} fv, scaled to a largest entry of 1 when `unit`
+  auto solve = [&](bool unit) {
+    float y = 0.f;
+#pragma unroll 4
+    for (int k = 0; k < M; ++k) {
+      y = fmaf(k ? fl[k - 1] : 0.f, y, fv[k]);
+      __syncwarp();
+      if (lane == 0) fv[k] = y;
+    }
+    __syncwarp();
+    float x = 0.f, top = 0.f;
+#pragma unroll 4
+    for (int k = M - 1; k >= 0; --k) {
+      x = fmaf(fl[k], x, fv[k] * fi[k]);  // fl[M-1] = 0
+      top = fmaxf(top, fabsf(x));
+      __syncwarp();
+      if (lane == 0) fv[k] = x;
+    }
+    __syncwarp();
+    if (unit) {
+      const float sc = __fdividef(1.0f, fmaxf(top, 1e-30f));
+      for (int i = lane; i < M; i += 32) fv[i] *= sc;
+      __syncwarp();
+    }
+  };
+  solve(true);
+  solve(true);
+  // quotient, correction, quotient; up to 4 entries per lane (M <= 128)
+  double v[4], rho = (double)hi;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) v[e] = lane + 32 * e < M ? (double)fv[lane + 32 * e] : 0.0;
+  for (int it = 0; it < 2; ++it) {
+    double t[4], num = 0.0;
+    float den = 0.f;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      t[e] = 0.0;
+      if (32 * e < M) {  // uniform
+        const int i = lane + 32 * e;
+        double left = __shfl_up_sync(0xffffffffu, v[e], 1), right = __shfl_down_sync(0xffffffffu, v[e], 1);
+        const double lastp = e > 0 ? __shfl_sync(0xffffffffu, v[e > 0 ? e - 1 : 0], 31) : 0.0;
+        const double firstn = e < 3 ? __shfl_sync(0xffffffffu, v[e < 3 ? e + 1 : 3], 0) : 0.0;
+        if (lane == 0) left = lastp;
+        if (lane == 31) right = firstn;
+        if (i < M) {
+          t[e] = (al[i] - rho) * v[e];
+          if (i > 0) t[e] = fma(be[i - 1], left, t[e]);
+          if (i < M - 1) t[e] = fma(be[i], right, t[e]);
+          num = fma(v[e], t[e], num);
+          den = fmaf((float)v[e], (float)v[e], den);
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      num += __shfl_xor_sync(0xffffffffu, num, o);
+      den += __shfl_xor_sync(0xffffffffu, den, o);
+    }
+    // num is of the size of lambda_max - rho, 1e-6 and then 1e-12 of
+    // lambda_max, so FP32 suffices for the ratio
+    const float q = (float)num / den;
+    rho += (double)q;
+    if (it == 1) break;
+    __syncwarp();
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (lane + 32 * e < M) fv[lane + 32 * e] = (float)t[e] - q * (float)v[e];  // (T - rho) v
+    __syncwarp();
+    solve(false);  // (sigma - T)^{-1} (T - rho) v: minus the contamination of v
+    // the component along v itself would only rescale it: taken out, so that
+    // the correction stays small
+    float dot = 0.f;
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (lane + 32 * e < M) dot = fmaf(fv[lane + 32 * e], (float)v[e], dot);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+    dot /= den;
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (lane + 32 * e < M) v[e] += (double)(fv[lane + 32 * e] - dot * (float)v[e]);
   }
-  return x;
+  return rho;
 }
 
-// Node z and weight w = e^z z'(t) / (i N) of upper-half node q (0..kHalf-1).
-__device__ inline void node(int q, cplx *z, cplx *w) {
-  const int k = kHalf + q;
-  const double t = -kPi + (k + 0.5) * (2.0 * kPi / kNodes);
-  double sn, cs;
-  sincos(kB * t, &sn, &cs);
-  const double cot = cs / sn;
-  *z = {kNodes * (kA * t * cot - kC), kNodes * kD * t};
-  const cplx dz = {kNodes * (kA * cot - kA * kB * t / (sn * sn)), kNodes * kD};
-  double es, ec;
-  sincos(z->im, &es, &ec);
-  const double ez = exp(z->re);
-  const cplx ezdz = cmul({ez * ec, ez * es}, dz);
-  *w = {ezdz.im / kNodes, -ezdz.re / kNodes};
+// Node z and weight w = e^z z'(t) / (i N) of the upper-half nodes q =
+// 0..kHalf-1, evaluated once on the host and passed to the kernels by value.
+struct Nodes {
+  cplx z[kHalf], w[kHalf];
+};
+inline Nodes make_nodes() {
+  Nodes n;
+  long double re[kHalf], im[kHalf], at0 = 0.0L;
+  const long double pi = std::acos(-1.0L);
+  for (int q = 0; q < kHalf; ++q) {
+    const long double t = -pi + (kHalf + q + 0.5L) * (2.0L * pi / kNodes);
+    const long double sn = std::sin(kB * t), cot = std::cos(kB * t) / sn;
+    const long double zr = kNodes * (kA * t * cot - kC), zi = kNodes * kD * t;
+    const long double dr = kNodes * (kA * cot - kA * kB * t / (sn * sn)), di = kNodes * kD;
+    const long double ec = std::exp(zr) * std::cos(zi), es = std::exp(zr) * std::sin(zi);
+    re[q] = (ec * di + es * dr) / kNodes;
+    im[q] = -(ec * dr - es * di) / kNodes;
+    n.z[q] = {(double)zr, (double)zi};
+    at0 += 2.0L * (re[q] * zr + im[q] * zi) / (zr * zr + zi * zi);  // 2 Re(w / z)
+  }
+  // the rule's value at 0, where the dominant eigenvalue of T - theta lies, is
+  // e^0 = 1 up to its truncation error (1.7e-14): the weights make it exact
+  for (int q = 0; q < kHalf; ++q) n.w[q] = {(double)(re[q] / at0), (double)(im[q] / at0)};
+  return n;
+}
+inline const Nodes &nodes() {
+  static const Nodes n = make_nodes();
+  return n;
 }
 
-// x = (z I - (T - theta I))^{-1} e1; diag z - (al_i - theta), off-diagonal -be_i.
-// cp is scratch of length M.
-__device__ inline void thomas_e1(const double *al, const double *be, int M, double theta, cplx z,
-                                 cplx *cp, cplx *x) {
-  cplx den = {z.re - (al[0] - theta), z.im};
-  cplx inv = cinv(den);
-  const double b0 = M > 1 ? be[0] : 0.0;
-  cp[0] = {-b0 * inv.re, -b0 * inv.im};
-  x[0] = inv;
-  for (int i = 1; i < M; ++i) {
-    const double b = be[i - 1];
-    den = {z.re - (al[i] - theta) + b * cp[i - 1].re, z.im + b * cp[i - 1].im};
-    inv = cinv(den);
-    const double bn = (i < M - 1) ? be[i] : 0.0;
-    cp[i] = {-bn * inv.re, -bn * inv.im};
-    x[i] = cmul({b * x[i - 1].re, b * x[i - 1].im}, inv);
+// The contour solves x_k = (z_k I - (T - theta I))^{-1} e1 of one warp, by
+// continuants: with d_i = z - (al_i - theta),
+//   phi_M = 1, phi_i = d_i phi_{i+1} - be_i^2 phi_{i+2},
+//   x_i = be_0 .. be_{i-1} phi_{i+1} / phi_0,
+// no reciprocal per row, and the real and imaginary part of a node on two
+// lanes (24 of the warp): 4 FP64 instructions per row, where a pivoted sweep
+// takes 18 on 12 lanes.  T and z are scaled by a power of two so that |d_i|
+// is below 1 and no product leaves the FP64 range for M <= CB_MAX_M.
+constexpr int kCols = 2 * kHalf;
+struct Solve {                     // shared memory of one solve
+  double phi[CB_MAX_M * kCols];    // phi_{i+1} at row i, column 2 k + part
+  double d[CB_MAX_M], b2[CB_MAX_M], B[CB_MAX_M];  // scaled; B: the products of be
+};
+
+// Fills S; returns the scale (a power of two: x above is to be multiplied by
+// it) and, in both lanes of a node's pair, 1 / phi_0 of lane / 2.  al, be in
+// shared memory.
+__device__ inline double continuants(const double *al, const double *be, int M, double theta,
+                                     const Nodes &nd, Solve &S, cplx *inv_phi0) {
+  const int lane = threadIdx.x & 31, part = lane & 1, q = lane < kCols ? lane >> 1 : 0;
+  double lowest = theta;
+  for (int i = lane; i < M; i += 32) lowest = fmin(lowest, al[i]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) lowest = fmin(lowest, __shfl_xor_sync(0xffffffffu, lowest, o));
+  int ex;
+  frexpf((float)(theta - lowest) + 64.f, &ex);  // |z| < 40
+  const double s = __hiloint2double((1023 - ex) << 20, 0);  // 2^-ex
+  double run = 1.0;  // product of the chunks before this one
+  for (int c = 0; c < M; c += 32) {
+    const int i = c + lane;
+    const double b = i < M ? be[i] * s : 1.0;
+    if (i < M) {
+      S.d[i] = (theta - al[i]) * s;
+      S.b2[i] = i < M - 1 ? b * b : 0.0;
+    }
+    double p = b;  // inclusive prefix product
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double y = __shfl_up_sync(0xffffffffu, p, o);
+      if (lane >= o) p *= y;
+    }
+    const double ex1 = __shfl_up_sync(0xffffffffu, p, 1);
+    if (i < M) S.B[i] = run * (lane ? ex1 : 1.0);
+    run *= __shfl_sync(0xffffffffu, p, 31);
   }
-  for (int i = M - 2; i >= 0; --i) {
-    const cplx t2 = cmul(cp[i], x[i + 1]);
-    x[i] = {x[i].re - t2.re, x[i].im - t2.im};
+  __syncwarp();
+  const double zr = nd.z[q].re * s, zi = (part ? 1.0 : -1.0) * nd.z[q].im * s;
+  double own = part ? 0.0 : 1.0, own2 = 0.0;
+#pragma unroll 2
+  for (int i = M - 1; i >= 0; --i) {
+    if (lane < kCols) S.phi[i * kCols + lane] = own;
+    const double other = __shfl_xor_sync(0xffffffffu, own, 1);
+    const double nxt = fma(zr + S.d[i], own, fma(zi, other, -S.b2[i] * own2));
+    own2 = own;
+    own = nxt;
+  }
+  // 1 / phi_0, scaled to exponent 0 on the way (|phi_0|^2 may underflow)
+  const double other = __shfl_xor_sync(0xffffffffu, own, 1);
+  const double re = part ? other : own, im = part ? own : other;
+  const int e0 = max((__double2hiint(re) >> 20) & 0x7ff, (__double2hiint(im) >> 20) & 0x7ff);
+  const double k = __hiloint2double((2046 - e0) << 20, 0);  // 2^(1023 - e0)
+  const double rs = re * k, is = im * k, dd = rcp_nr(fma(rs, rs, is * is)) * k;
+  *inv_phi0 = {rs * dd, -is * dd};
+  __syncwarp();
+  return s;
+}
+
+// out(i, c_i) for the rows i < M: c_i = sum_k Re(p_k x_k,i), p (both lanes of
+// the pair) the node's factor times *inv_phi0.  Called by the warp.
+template <typename F>
+__device__ inline void real_sum(Solve &S, int M, double scale, cplx g, F out) {
+  const int lane = threadIdx.x & 31;
+  __shared__ double s_g[kCols];
+  if (lane < kCols) s_g[lane] = (lane & 1) ? -g.im * scale : g.re * scale;
+  __syncwarp();
+  for (int i = lane; i < M; i += 32) {
+    double c = 0.0;
+#pragma unroll
+    for (int q = 0; q < kCols; ++q) c = fma(s_g[q], S.phi[i * kCols + q], c);
+    out(i, c * S.B[i]);
   }
 }
 

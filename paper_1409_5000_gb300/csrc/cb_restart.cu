@@ -73,12 +73,11 @@ __device__ inline contour::cplx thomas_last(const double *al, const double *be, 
 // One warp per realisation: the shift, the combine weights gamma_j of the
 // current cycle's basis, and the state the next cycle starts from.
 __global__ void __launch_bounds__(32) restart_tridiag_kernel(Scalars sc, RState rs,
-                                                             const InstDesc *inst, uint32_t c) {
+                                                             const InstDesc *inst, uint32_t c,
+                                                             contour::Nodes nd) {
   using namespace contour;
   __shared__ double s_al[CB_MAX_M], s_be[CB_MAX_M];
-  __shared__ double s_c[kHalf][CB_MAX_M];
-  __shared__ double s_theta;
-  __shared__ int s_recompute;
+  __shared__ Solve s_s;
   const uint32_t r = blockIdx.x, lane = threadIdx.x, ms = sc.ms, m = rs.m;
   const bool active = c == 0 || rs.rscale[r] > 0.0;
   const int M = (int)sc.meff[r];
@@ -95,56 +94,51 @@ __global__ void __launch_bounds__(32) restart_tridiag_kernel(Scalars sc, RState 
     s_be[i] = sc.beta[r * ms + i];
   }
   __syncwarp();
-  if (lane == 0) {
-    const double tk = lambda_max(s_al, s_be, M);
-    const double told = rs.theta[r];
-    const double tn = c == 0 ? tk : fmax(told, tk);
-    rs.rho[r] = c == 0 ? 0.0 : exp(told - tn);
-    rs.theta[r] = tn;
-    s_theta = tn;
-    s_recompute = c > 0 && tn > told;
-  }
+  const double tk = lambda_max(s_al, s_be, M, reinterpret_cast<float *>(s_s.phi));
+  const double told = rs.theta[r];
+  const double theta = c == 0 ? tk : fmax(told, tk);
+  const bool recompute = c > 0 && theta > told;
   __syncwarp();
-  const double theta = s_theta;
+  if (lane == 0) {
+    rs.rho[r] = c == 0 ? 0.0 : exp(told - theta);
+    rs.theta[r] = theta;
+  }
   const bool more = M == (int)m && sc.scale[r * ms + m] > 0.0 && c + 1 < rs.cmax;
-  if (lane < kHalf) {
-    double *pq = rs.p + ((size_t)r * kHalf + lane) * 2;
-    cplx z, w;
-    node((int)lane, &z, &w);
-    cplx p = {1.0, 0.0};
-    if (s_recompute) {  // the shift moved: the products again from cycle 1
+  cplx inv0;
+  const double scale = continuants(s_al, s_be, M, theta, nd, s_s, &inv0);
+  cplx p = {1.0, 0.0}, w = {0.0, 0.0};  // both lanes of a node's pair
+  if (lane < kCols) {
+    const int q = lane >> 1;
+    double *pq = rs.p + ((size_t)r * kHalf + q) * 2;
+    w = nd.w[q];
+    if (recompute) {  // the shift moved: the products again from cycle 1
       for (uint32_t i = 0; i < c; ++i) {
         const size_t o = ((size_t)r * rs.cmax + i) * m;
-        const cplx xl = thomas_last(rs.hal + o, rs.hbe + o, (int)m, theta, z);
+        const cplx xl = thomas_last(rs.hal + o, rs.hbe + o, (int)m, theta, nd.z[q]);
         const double b = rs.couple[(size_t)r * rs.cmax + i];
         p = cmul(p, {b * xl.re, b * xl.im});
       }
     } else if (c > 0) {
       p = {pq[0], pq[1]};
     }
-    cplx cp[CB_MAX_M], x[CB_MAX_M];
-    thomas_e1(s_al, s_be, M, theta, z, cp, x);
-    const cplx wp = cmul(w, p);
-    for (int i = 0; i < M; ++i) s_c[lane][i] = 2.0 * (wp.re * x[i].re - wp.im * x[i].im);
-    if (more) {
-      const double b = sc.beta[r * ms + m - 1];
-      const cplx np = cmul(p, {b * x[m - 1].re, b * x[m - 1].im});
-      pq[0] = np.re;
-      pq[1] = np.im;
-    }
   }
   __syncwarp();
+  const cplx g = cmul(p, inv0);
+  if (more && lane < kCols && !(lane & 1)) {  // p_q b [x_q]_m: the last row, phi_M = 1
+    const double b = sc.beta[r * ms + m - 1] * scale * s_s.B[m - 1];
+    double *pq = rs.p + ((size_t)r * kHalf + (lane >> 1)) * 2;
+    pq[0] = b * g.re;
+    pq[1] = b * g.im;
+  }
   const double beta0 = sqrt((double)inst[r].n);
-  for (int i = lane; i < M; i += 32) {
-    double cc = 0.0;
-    for (int q = 0; q < kHalf; ++q) cc += s_c[q][i];
+  real_sum(s_s, M, 2.0 * scale, cmul(w, g), [&](int i, double cc) {
     sc.gamma[r * ms + i] = beta0 * cc * sc.scale[r * ms + i];
     if (more) {
       const size_t o = ((size_t)r * rs.cmax + c) * m + i;
       rs.hal[o] = s_al[i];
       rs.hbe[o] = s_be[i];
     }
-  }
+  });
   if (lane == 0) {
     rs.steps[r] += (uint32_t)M;
     rs.blast[r] = sc.beta[r * ms + M - 1];
@@ -227,7 +221,7 @@ int cycles_run(cb_graph *h, const RState &rs, double *Y, uint32_t m, uint32_t cy
     rc = lanczos_run(h, W, 0, h->n_inst, m, prec, s, nullptr, 0, false, c ? rs.rscale : nullptr);
     if (rc != CB_OK) break;
     int tok = prof_begin(CB_K_TRIDIAG, s);
-    restart_tridiag_kernel<<<h->n_inst, 32, 0, s>>>(W.sc, rs, h->d_inst, c);
+    restart_tridiag_kernel<<<h->n_inst, 32, 0, s>>>(W.sc, rs, h->d_inst, c, contour::nodes());
     prof_end(tok, s);
     tok = prof_begin(CB_K_COMBINE, s);
     if (h->total_fin)

@@ -21,11 +21,10 @@ namespace {
 
 // One warp per start node: theta_q = lambda_max(T), c0_q = [exp(T - theta) e1]_0
 // via the contour rule (theta in sc.theta[q], c0 in sc.gamma[q * ms]).
-__global__ void __launch_bounds__(32) sc_tridiag_kernel(Scalars sc) {
+__global__ void __launch_bounds__(32) sc_tridiag_kernel(Scalars sc, contour::Nodes nd) {
   using namespace contour;
   __shared__ double s_al[CB_MAX_M], s_be[CB_MAX_M];
-  __shared__ double s_c0[kHalf];
-  __shared__ double s_theta;
+  __shared__ Solve s_s;
   const uint32_t q = blockIdx.x, lane = threadIdx.x, ms = sc.ms;
   const int M = (int)sc.meff[q];
   if (sc.status[q] != CB_OK || M < 1) {
@@ -40,23 +39,14 @@ __global__ void __launch_bounds__(32) sc_tridiag_kernel(Scalars sc) {
     s_be[i] = sc.beta[q * ms + i];
   }
   __syncwarp();
-  if (lane == 0) s_theta = lambda_max(s_al, s_be, M);
+  const double theta = lambda_max(s_al, s_be, M, reinterpret_cast<float *>(s_s.phi));
   __syncwarp();
-  const double theta = s_theta;
-  if (lane < kHalf) {
-    cplx z, w;
-    node((int)lane, &z, &w);
-    cplx cp[CB_MAX_M], x[CB_MAX_M];
-    thomas_e1(s_al, s_be, M, theta, z, cp, x);
-    s_c0[lane] = 2.0 * (w.re * x[0].re - w.im * x[0].im);
-  }
-  __syncwarp();
-  if (lane == 0) {
-    double c0 = 0.0;
-    for (int t = 0; t < kHalf; ++t) c0 += s_c0[t];
+  cplx inv0;
+  const double scale = continuants(s_al, s_be, M, theta, nd, s_s, &inv0);
+  real_sum(s_s, 1, 2.0 * scale, cmul(nd.w[lane < kCols ? lane >> 1 : 0], inv0), [&](int, double c0) {
     sc.theta[q] = theta;
     sc.gamma[q * ms] = c0;
-  }
+  });
 }
 
 // Common shift theta* = max_q theta_q; out[q] = exp(theta_q - theta*) c0_q.
@@ -132,7 +122,7 @@ CB_API int cb_subgraph_centrality(cb_graph *h, uint32_t inst, uint32_t m, int pr
   rc = ensure_workspace(v, v->ws, m, prec, s);
   if (rc == CB_OK) rc = lanczos_run(v, v->ws, 0, k, m, prec, s, d_nodes, k, true);
   if (rc == CB_OK) {
-    sc_tridiag_kernel<<<k, 32, 0, s>>>(v->ws.sc);
+    sc_tridiag_kernel<<<k, 32, 0, s>>>(v->ws.sc, contour::nodes());
     sc_finish_kernel<<<1, 256, 0, s>>>(v->ws.sc, k, sc_scaled, log_scale);
     rc = cuda_error(cudaGetLastError(), "cb_subgraph_centrality: launch");
   }

@@ -1,0 +1,30 @@
+"""The small tridiagonal step at every kind of depth: one step, a breakdown,
+the deepest recurrence (needs a GB300)."""
+import numpy as np
+import pytest
+
+import oracle.communicability as oc
+from paper_1409_5000_gb300 import synth
+from tests import parity
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("m", [1, 2, 3, 31, 32, 33, 64, 128])
+def test_shift_and_scores_at_depth(m):
+    """theta is lambda_max of the oracle's T_m to FP64 rounding (1e-13 of its
+    size), and the scores meet the FP64 bar.  Reorthogonalised: T_m itself
+    agrees only then once the recurrence has converged."""
+    from paper_1409_5000_gb300 import binding as B
+
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for -m gpu tests")
+    graphs = [synth.er(3001, 9.0 / 3000, 11), synth.ws(700, 8, 0.1, 12), synth.ba(1200, 4, 13),
+              synth.from_edges(40, [(i, i + 1) for i in range(39)])]
+    with B.GraphSet(graphs) as gs:
+        for r, g in enumerate(graphs):
+            ls, y = B.communicability(gs, r, m, B.CB_FP64 | B.CB_REORTH)
+            th_o, y_o, _ = oc.krylov_expv(g.n, g.row_ptr, g.col, m)
+            assert abs(float(ls.item()) - th_o) <= 1e-13 * max(1.0, abs(th_o))
+            parity.assert_scores(float(ls.item()), y.cpu().numpy(), th_o, y_o, "fp64")

@@ -73,13 +73,15 @@ static int ensure_backwork(cb_graph *h, uint32_t m, int prec, cudaStream_t s) {
 __global__ void __launch_bounds__(64) bw_tridiag_kernel(Scalars s1, Scalars sw,
                                                         const InstDesc *inst, double *K,
                                                         uint32_t kdim, double *theta_out,
-                                                        uint32_t *cnt_out, contour::Nodes nd) {
+                                                        uint32_t *cnt_out, contour::Nodes nd,
+                                                        bool laguerre) {
   using namespace contour;
   extern __shared__ double s_dyn[];
   Solve *s_s = reinterpret_cast<Solve *>(s_dyn);  // [2]
   __shared__ double s_al[2][kMaxAdjM], s_be[2][kMaxAdjM];
   __shared__ double s_th[2], s_scale[2];
   __shared__ cplx s_inv0[2][kHalf];
+  __shared__ Spectrum s_sp[2];
   const uint32_t r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
   const int M1 = (int)s1.meff[r], Mw = (int)sw.meff[r];
   const bool ok = M1 > 0 && Mw > 0 && s1.status[r] == CB_OK && sw.status[r] == CB_OK;
@@ -97,7 +99,7 @@ __global__ void __launch_bounds__(64) bw_tridiag_kernel(Scalars s1, Scalars sw,
     s_be[wp][i] = sc.beta[r * sc.ms + i];
   }
   __syncwarp();
-  const double th = lambda_max(s_al[wp], s_be[wp], M, reinterpret_cast<float *>(s_s[wp].phi));
+  const double th = largest(s_al[wp], s_be[wp], M, s_sp[wp], laguerre);
   if (lane == 0) s_th[wp] = th;
   __syncthreads();
   const double theta = fmax(s_th[0], s_th[1]);
@@ -365,7 +367,7 @@ static int backward_t(cb_graph *h, uint32_t m, const uint32_t *idx, uint32_t k, 
   const size_t shm_tri = 2 * sizeof(contour::Solve);
   cudaFuncSetAttribute(bw_tridiag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_tri);
   bw_tridiag_kernel<<<N, 64, shm_tri, s>>>(h->ws.sc, h->ws2.sc, h->d_inst, B.K, m, B.theta, B.cnt,
-                                           contour::nodes());
+                                           contour::nodes(), sizeof(T) == 8 && !h->reorth);
   const size_t shm = (size_t)(m * m + 8 * m * 32) * sizeof(T);
   auto nk = bw_node_kernel<T>;
   if (shm > 48 * 1024) cudaFuncSetAttribute(nk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);

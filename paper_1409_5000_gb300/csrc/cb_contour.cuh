@@ -3,6 +3,10 @@
 //  * lambda_max: the largest eigenvalue of T, bracketed in FP32 by a warp-wide
 //    multisection on the signs of the pivots of xI - T, then the FP64 Rayleigh
 //    quotient of an eigenvector from inverse iteration.
+//  * lambda_max_laguerre: the same by Laguerre's iteration on det(xI - T),
+//    started above the Gershgorin bound.  For a polynomial with only real
+//    roots, Laguerre's method started above the largest root decreases
+//    monotonically to it and converges cubically.
 //  * contour nodes: exp(x) on (-inf, 0] as the trapezoid rule for the
 //    Cauchy integral over the cotangent contour of Trefethen, Weideman &
 //    Schmelzer ("Talbot quadratures and rational approximations", BIT 46,
@@ -43,9 +47,52 @@ __device__ __forceinline__ double rcp_nr(double r) {
   return fma(y, fma(-r, y, 1.0), y);
 }
 
+// 1 / sqrt(x) for x in the normal FP32 range, as rcp_nr: y <- y + y/2 (1 - x y^2).
+__device__ __forceinline__ double rsqrt_nr(double x) {
+  double y = (double)rsqrtf((float)x);
+  y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
+  return fma(0.5 * y, fma(-x * y, y, 1.0), y);
+}
+
+// FP32 Laguerre terms at x from f'/f and (f'/f)^2 - f''/f of f(x) = det(xI - T),
+// through the ratios r_k = p_k / p_{k-1} of the leading principal minors (one
+// reciprocal per k), which cannot overflow.  a: diagonal, b2: squared
+// off-diagonal.  False if some r_k <= 0, i.e. x is not above the spectrum.
+__device__ inline bool laguerre_f32(const float *a, const float *b2, int M, float x, float *step) {
+  float r = x - a[0], rd = 1.0f, rdd = 0.0f;
+  if (!(r > 0.0f)) return false;
+  float ir = 1.0f / r;
+  float g = rd * ir;
+  float h = g * g - rdd * ir;
+  for (int k = 1; k < M; ++k) {
+    const float q = b2[k - 1] * ir;
+    const float nr = (x - a[k]) - q;
+    const float nrd = 1.0f + q * ir * rd;
+    const float nrdd = q * ir * (rdd - 2.0f * rd * rd * ir);
+    r = nr;
+    rd = nrd;
+    rdd = nrdd;
+    if (!(r > 0.0f)) return false;
+    ir = 1.0f / r;
+    const float gk = rd * ir;
+    g += gk;
+    h += gk * gk - rdd * ir;
+  }
+  const float disc = (float)(M - 1) * ((float)M * h - g * g);
+  const float den = g + sqrtf(disc > 0.0f ? disc : 0.0f);
+  if (!(den > 0.0f)) return false;
+  *step = (float)M / den;
+  return true;
+}
+
+// Shared-memory scratch of the largest eigenvalue.
+struct Spectrum {
+  float f[5 * CB_MAX_M];
+  double as[CB_MAX_M], bs2[CB_MAX_M];
+};
+
 // Largest eigenvalue of tridiag(be, al, be) (be[0..M-2] used, positive), by
-// one full warp; every lane gets it.  al and be are in shared memory; f is
-// shared scratch of 5 M floats.
+// one full warp; every lane gets it.  al and be are in shared memory.
 //
 // An FP64 instruction of one warp occupies its sub-core's FP64 unit for about
 // 64 cycles whatever its active lanes (0.5 lanes per clock), so the serial
@@ -65,7 +112,8 @@ __device__ __forceinline__ double rcp_nr(double r) {
 // 131 -> 25 us at M = 30, 220 -> 34 us at M = 40 (before: one lane running
 // Laguerre's iteration in FP32 and twice in FP64, and a Thomas sweep with a
 // complex reciprocal per row and lane).
-__device__ inline double lambda_max(const double *al, const double *be, int M, float *f) {
+__device__ inline double lambda_max(const double *al, const double *be, int M, Spectrum &S) {
+  float *f = S.f;
   if (M == 1) return al[0];
   const int lane = threadIdx.x & 31;
   float *fa = f, *fb = f + M, *fl = f + 2 * M, *fi = f + 3 * M, *fv = f + 4 * M;
@@ -203,6 +251,93 @@ __device__ inline double lambda_max(const double *al, const double *be, int M, f
       if (lane + 32 * e < M) v[e] += (double)(fv[lane + 32 * e] - dot * (float)v[e]);
   }
   return rho;
+}
+
+// The same by Laguerre's iteration on det(xI - T), for FP64 recurrences
+// without reorthogonalisation: their T carries copies of lambda_max, over which
+// two FP64 steps stop up to about 1e-6 above it, and theta is a result that
+// callers compare and store in that precision.  (Elsewhere lambda_max is used:
+// 25 against 34 us at M = 30.)  The iteration from above the Gershgorin bound runs in FP32 until its step is
+// below 1e-6 relative, then two FP64 steps polish the result: the convergence
+// is cubic, so the FP32 estimate turns into an FP64-accurate one.
+//
+// T is converted once, in parallel, and the FP64 steps take f, f' and f'' from
+// p_k = (x - a_k) p_{k-1} - b_{k-1}^2 p_{k-2} and its derivatives on three
+// lanes at once: 4 FP64 instructions per row (the ratios above take 22).  T
+// and x are scaled by a power of two there, so that no product leaves the FP64
+// range for M <= CB_MAX_M.
+__device__ inline double lambda_max_laguerre(const double *al, const double *be, int M, Spectrum &S) {
+  if (M == 1) return al[0];
+  const int lane = threadIdx.x & 31;
+  float *fa = S.f, *fb2 = S.f + CB_MAX_M;
+  double x0 = -1e300, low = 1e300;
+  for (int i = lane; i < M; i += 32) {
+    const double lo = i > 0 ? fabs(be[i - 1]) : 0.0;
+    const double hi = i < M - 1 ? fabs(be[i]) : 0.0;
+    x0 = fmax(x0, al[i] + lo + hi);
+    low = fmin(low, al[i]);
+    const float fb = (float)be[i];
+    fa[i] = (float)al[i];
+    fb2[i] = fb * fb;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    x0 = fmax(x0, __shfl_xor_sync(0xffffffffu, x0, o));
+    low = fmin(low, __shfl_xor_sync(0xffffffffu, low, o));
+  }
+  x0 += 1e-3 * (fabs(x0) + 1.0);  // strictly above the spectrum, also in FP32
+  int ex;
+  frexpf((float)(x0 - low) + 1.0f, &ex);
+  const double s = __hiloint2double((1023 - ex) << 20, 0);  // 2^-ex: |x - a_k| < 2^ex
+  for (int i = lane; i < M; i += 32) {
+    const double b = be[i] * s;
+    S.as[i] = al[i] * s;
+    S.bs2[i] = b * b;
+  }
+  __syncwarp();
+  float xf = (float)x0;
+  if ((double)xf < x0) xf = nextafterf(xf, 3.0e38f);
+  float st;
+  if (laguerre_f32(fa, fb2, M, xf, &st)) {
+    for (int it = 0; it < 40; ++it) {
+      const float nx = xf - st;
+      float st2;
+      if (!laguerre_f32(fa, fb2, M, nx, &st2)) break;  // nx not above: keep xf
+      xf = nx;
+      st = st2;
+      if (st <= 1e-6f * (fabsf(xf) + 1.0f)) break;
+    }
+  }
+  double x = xf;
+  const double c = lane == 1 ? 1.0 : lane == 2 ? 2.0 : 0.0;  // lane d: the d-th derivative
+  for (int it = 0; it < 2; ++it) {  // FP64 polish (a failed step leaves x above the root)
+    const double xs = x * s;
+    double own2 = lane == 0 ? 1.0 : 0.0;                                 // p_0
+    double own = lane == 0 ? xs - S.as[0] : lane == 1 ? 1.0 : 0.0;       // p_1
+    bool above = lane != 0 || own > 0.0;
+#pragma unroll 2
+    for (int k = 1; k < M; ++k) {
+      const double below = __shfl_up_sync(0xffffffffu, own, 1);  // lane 0's c is 0
+      const double nxt = fma(xs - S.as[k], own, fma(c, below, -S.bs2[k - 1] * own2));
+      own2 = own;
+      own = nxt;
+      if (lane == 0) above = above && __double2hiint(own) > 0;  // own > 0, without an FP64 compare
+    }
+    if (!__all_sync(0xffffffffu, above)) break;
+    const double p = __shfl_sync(0xffffffffu, own, 0), p1 = __shfl_sync(0xffffffffu, own, 1);
+    const double p2 = __shfl_sync(0xffffffffu, own, 2);
+    // G = f'/f, H = G^2 - f''/f, times s and s^2
+    const double ip = 1.0 / p, G = p1 * ip, H = G * G - p2 * ip;
+    const double disc = (double)(M - 1) * ((double)M * H - G * G);
+    const double den = G + sqrt(disc > 0.0 ? disc : 0.0);
+    if (!(den > 0.0)) break;
+    x -= (double)M / (den * s);
+  }
+  return x;
+}
+
+__device__ inline double largest(const double *al, const double *be, int M, Spectrum &S, bool laguerre) {
+  return laguerre ? lambda_max_laguerre(al, be, M, S) : lambda_max(al, be, M, S);
 }
 
 // Node z and weight w = e^z z'(t) / (i N) of the upper-half nodes q =

@@ -74,10 +74,11 @@ __device__ inline contour::cplx thomas_last(const double *al, const double *be, 
 // current cycle's basis, and the state the next cycle starts from.
 __global__ void __launch_bounds__(32) restart_tridiag_kernel(Scalars sc, RState rs,
                                                              const InstDesc *inst, uint32_t c,
-                                                             contour::Nodes nd) {
+                                                             contour::Nodes nd, bool laguerre) {
   using namespace contour;
   __shared__ double s_al[CB_MAX_M], s_be[CB_MAX_M];
   __shared__ Solve s_s;
+  __shared__ Spectrum s_sp;
   const uint32_t r = blockIdx.x, lane = threadIdx.x, ms = sc.ms, m = rs.m;
   const bool active = c == 0 || rs.rscale[r] > 0.0;
   const int M = (int)sc.meff[r];
@@ -94,7 +95,7 @@ __global__ void __launch_bounds__(32) restart_tridiag_kernel(Scalars sc, RState 
     s_be[i] = sc.beta[r * ms + i];
   }
   __syncwarp();
-  const double tk = lambda_max(s_al, s_be, M, reinterpret_cast<float *>(s_s.phi));
+  const double tk = largest(s_al, s_be, M, s_sp, laguerre);
   const double told = rs.theta[r];
   const double theta = c == 0 ? tk : fmax(told, tk);
   const bool recompute = c > 0 && theta > told;
@@ -221,7 +222,8 @@ int cycles_run(cb_graph *h, const RState &rs, double *Y, uint32_t m, uint32_t cy
     rc = lanczos_run(h, W, 0, h->n_inst, m, prec, s, nullptr, 0, false, c ? rs.rscale : nullptr);
     if (rc != CB_OK) break;
     int tok = prof_begin(CB_K_TRIDIAG, s);
-    restart_tridiag_kernel<<<h->n_inst, 32, 0, s>>>(W.sc, rs, h->d_inst, c, contour::nodes());
+    restart_tridiag_kernel<<<h->n_inst, 32, 0, s>>>(W.sc, rs, h->d_inst, c, contour::nodes(),
+                                                     sizeof(T) == 8 && !h->reorth);
     prof_end(tok, s);
     tok = prof_begin(CB_K_COMBINE, s);
     if (h->total_fin)

@@ -21,10 +21,11 @@ namespace {
 
 // One warp per start node: theta_q = lambda_max(T), c0_q = [exp(T - theta) e1]_0
 // via the contour rule (theta in sc.theta[q], c0 in sc.gamma[q * ms]).
-__global__ void __launch_bounds__(32) sc_tridiag_kernel(Scalars sc, contour::Nodes nd) {
+__global__ void __launch_bounds__(32) sc_tridiag_kernel(Scalars sc, contour::Nodes nd, bool laguerre) {
   using namespace contour;
   __shared__ double s_al[CB_MAX_M], s_be[CB_MAX_M];
   __shared__ Solve s_s;
+  __shared__ Spectrum s_sp;
   const uint32_t q = blockIdx.x, lane = threadIdx.x, ms = sc.ms;
   const int M = (int)sc.meff[q];
   if (sc.status[q] != CB_OK || M < 1) {
@@ -39,7 +40,7 @@ __global__ void __launch_bounds__(32) sc_tridiag_kernel(Scalars sc, contour::Nod
     s_be[i] = sc.beta[q * ms + i];
   }
   __syncwarp();
-  const double theta = lambda_max(s_al, s_be, M, reinterpret_cast<float *>(s_s.phi));
+  const double theta = largest(s_al, s_be, M, s_sp, laguerre);
   __syncwarp();
   cplx inv0;
   const double scale = continuants(s_al, s_be, M, theta, nd, s_s, &inv0);
@@ -122,7 +123,7 @@ CB_API int cb_subgraph_centrality(cb_graph *h, uint32_t inst, uint32_t m, int pr
   rc = ensure_workspace(v, v->ws, m, prec, s);
   if (rc == CB_OK) rc = lanczos_run(v, v->ws, 0, k, m, prec, s, d_nodes, k, true);
   if (rc == CB_OK) {
-    sc_tridiag_kernel<<<k, 32, 0, s>>>(v->ws.sc, contour::nodes());
+    sc_tridiag_kernel<<<k, 32, 0, s>>>(v->ws.sc, contour::nodes(), prec == CB_FP64 && !reorth);
     sc_finish_kernel<<<1, 256, 0, s>>>(v->ws.sc, k, sc_scaled, log_scale);
     rc = cuda_error(cudaGetLastError(), "cb_subgraph_centrality: launch");
   }

@@ -18,10 +18,11 @@
 namespace cb {
 
 __global__ void __launch_bounds__(32) tridiag_kernel(Scalars sc, const InstDesc *inst,
-                                                     uint32_t r0, contour::Nodes nd) {
+                                                     uint32_t r0, contour::Nodes nd, bool laguerre) {
   using namespace contour;
   __shared__ double s_al[CB_MAX_M], s_be[CB_MAX_M];
   __shared__ Solve s_s;
+  __shared__ Spectrum s_sp;
   const uint32_t r = r0 + blockIdx.x;
   const uint32_t lane = threadIdx.x;
   const uint32_t ms = sc.ms;
@@ -35,7 +36,7 @@ __global__ void __launch_bounds__(32) tridiag_kernel(Scalars sc, const InstDesc 
     s_be[i] = sc.beta[r * ms + i];
   }
   __syncwarp();
-  const double theta = lambda_max(s_al, s_be, M, reinterpret_cast<float *>(s_s.phi));
+  const double theta = largest(s_al, s_be, M, s_sp, laguerre);
   __syncwarp();
   cplx inv0;
   const double scale = continuants(s_al, s_be, M, theta, nd, s_s, &inv0);
@@ -45,11 +46,12 @@ __global__ void __launch_bounds__(32) tridiag_kernel(Scalars sc, const InstDesc 
   if (lane == 0) sc.theta[r] = theta;
 }
 
-int tridiag_run(cb_graph *h, uint32_t r0, uint32_t r1, int /*prec*/, cudaStream_t s) {
+int tridiag_run(cb_graph *h, uint32_t r0, uint32_t r1, int prec, cudaStream_t s) {
   NvtxRange nvtx_range("tridiagonal exp");
   prefer_shared(tridiag_kernel);
   const int tok = prof_begin(CB_K_TRIDIAG, s);
-  tridiag_kernel<<<r1 - r0, 32, 0, s>>>(h->ws.sc, h->d_inst, r0, contour::nodes());
+  tridiag_kernel<<<r1 - r0, 32, 0, s>>>(h->ws.sc, h->d_inst, r0, contour::nodes(),
+                                     prec == CB_FP64 && !h->reorth);
   prof_end(tok, s);
   return cuda_error(cudaGetLastError(), "tridiag launch");
 }

@@ -546,6 +546,8 @@ CB_API int cb_scores_backward_budget(cb_graph *h, uint32_t m, int prec, const ui
     rc = cb_graph_upload(r1 - r0, vn.data(), nnz.data() + r0, vrp.data(), vcol.data(),
                          CB_DEVICE_PTRS, stream, &v);
     if (rc != CB_OK) break;
+    v->plan_of = h;
+    v->plan_r0 = r0;
     rc = cb_scores_backward(v, m, prec, topk_idx, k, grad + h->inst[r0].edge_base, d_ls + g, stream);
     if (rc == CB_OK) rc = cuda_error(cudaStreamSynchronize(s), "cb_scores_backward_budget");
     const int rf = cb_graph_free(v);

@@ -20,6 +20,7 @@
 #include <unordered_map>
 
 #include "cb_internal.cuh"
+#include "cb_team.cuh"
 
 namespace cb {
 
@@ -275,8 +276,10 @@ int ensure_workspace(cb_graph *h, Workspace &W, uint32_t m, int prec, cudaStream
   const size_t nheavy = std::max<size_t>(h->total_heavy, 1);
   // doubles first, then 32-bit words
   const size_t nfin = std::max<size_t>(h->total_fin, 1);
-  const size_t nd = 4 * (size_t)N * ms + N + nslots + ngroups + nchunks + nfin * ms + (size_t)N * ms;
-  const size_t nw = 2 * (size_t)N + ngroups + N + nheavy;
+  const size_t nxch = 2 * (size_t)kMaxTeamCtas, nxd = 2 * (size_t)kMaxTeamCtas * ms;
+  const size_t nd = 4 * (size_t)N * ms + N + nslots + ngroups + nchunks + nfin * ms + (size_t)N * ms +
+                    nxch + nxd;
+  const size_t nw = 2 * (size_t)N + ngroups + N + nheavy + kCtrStride * (kMaxTeams + 1);
   const size_t bytes = nd * sizeof(double) + nw * sizeof(uint32_t) + 256;
   e = dev_alloc(&W.blob, bytes);
   if (e != cudaSuccess) {
@@ -295,12 +298,15 @@ int ensure_workspace(cb_graph *h, Workspace &W, uint32_t m, int prec, cudaStream
   W.cpart = d; d += nchunks;
   W.rpart = d; d += nfin * ms;
   W.rh = d; d += (size_t)N * ms;
+  W.xd = d; d += nxd;
+  W.tparts = d; d += nxch;
   uint32_t *w = reinterpret_cast<uint32_t *>(d);
   W.sc.meff = w; w += N;
   W.sc.status = reinterpret_cast<int32_t *>(w); w += N;
   W.gcnt = w; w += ngroups;
   W.icnt = w; w += N;
   W.hcnt = w; w += nheavy;
+  W.tctr = w + (kCtrStride - (reinterpret_cast<uintptr_t>(w) / 4) % kCtrStride) % kCtrStride;
   W.sc.ms = ms;
   W.blob_bytes = bytes;
   W.m = m;
@@ -456,7 +462,7 @@ CB_API int cb_debug_violations(uint32_t *count, uint64_t *first, int reset) {
   *first = 0;
   if (cb_debug_build() && cudaDeviceSynchronize() != cudaSuccess)
     return set_error(CB_ERR_CUDA, "cb_debug_violations: device synchronize");
-  int (*readers[4])(uint32_t *, uint64_t *, bool) = {dbg_read_lanczos, dbg_read_blocked,
+  int (*readers[5])(uint32_t *, uint64_t *, bool) = {dbg_read_lanczos, dbg_read_team, dbg_read_blocked,
                                                      dbg_read_twophase, dbg_read_adjoint};
   for (auto rd : readers) {
     uint32_t c = 0;
@@ -892,8 +898,9 @@ CB_API int cb_graph_set_path(cb_graph *h, int path) {
   if (!h) return set_error(CB_ERR_ARG, "cb_graph_set_path: null handle");
   if (path != CB_PATH_AUTO && path != CB_PATH_FORMATS && path != CB_PATH_CSR)
     return set_error(CB_ERR_ARG, "cb_graph_set_path: unknown path");
-  if (h->path != path) {
+  if (h->path != path || h->tuned_auto) {
     h->path = path;
+    h->tuned_auto = false;
     drop_graphs(h);  // captured passes hold the old kernel choice
   }
   return CB_OK;
@@ -929,6 +936,8 @@ CB_API int cb_graph_tune(cb_graph *h, int prec, uint32_t *lanes_out, double *ms_
   cudaError_t e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
   const int keep_lanes = h->lanes, keep_path = h->path;
+  const bool keep_auto = h->tuned_auto;
+  h->tuned_auto = false;
   int best_lanes = keep_lanes, best_path = keep_path;
   double best_ms = 1e300;
   auto time_one = [&](int lanes, int path, int slot) {
@@ -943,7 +952,7 @@ CB_API int cb_graph_tune(cb_graph *h, int prec, uint32_t *lanes_out, double *ms_
     float ms = 0.f;
     if (rc == CB_OK && e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
     if (rc == CB_OK && e == cudaSuccess) {
-      if (ms_out) ms_out[slot] = ms / 2.0;
+      if (ms_out && slot >= 0) ms_out[slot] = ms / 2.0;
       if (ms < best_ms) {
         best_ms = ms;
         best_lanes = lanes;
@@ -955,17 +964,28 @@ CB_API int cb_graph_tune(cb_graph *h, int prec, uint32_t *lanes_out, double *ms_
   // the format path, with the best width for any tiled-CSR realisations left
   if (formats && e == cudaSuccess && rc == CB_OK) time_one(best_lanes, CB_PATH_FORMATS, 6);
   if (small && e == cudaSuccess && rc == CB_OK) time_one(best_lanes, CB_PATH_AUTO, 7);
-  // FP64 depends on the path only through the single launch of small handles
+  // FP64 depends on the path only through the single launch
   if (prec == CB_FP64 && !small) best_path = keep_path;
+  // other handles may run as one launch too: the path kept stays a per-step
+  // one, and the automatic choice is taken beside it where it is faster
+  if (!small && e == cudaSuccess && rc == CB_OK) {
+    const double per_step = best_ms;
+    const int l = best_lanes, p = best_path;
+    time_one(best_lanes, CB_PATH_AUTO, -1);
+    h->tuned_auto = best_ms < per_step;
+    best_lanes = l;
+    best_path = p;
+  }
   h->lanes = best_lanes;
   h->path = best_path;
-  if (best_lanes != keep_lanes || best_path != keep_path) drop_graphs(h);
+  if (keep_auto != h->tuned_auto || best_lanes != keep_lanes || best_path != keep_path) drop_graphs(h);
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   free_workspace(W);
   if (rc != CB_OK || e != cudaSuccess) {
     h->lanes = keep_lanes;
     h->path = keep_path;
+    h->tuned_auto = keep_auto;
     return rc != CB_OK ? rc : cuda_error(e, "cb_graph_tune");
   }
   if (lanes_out) *lanes_out = (uint32_t)best_lanes;

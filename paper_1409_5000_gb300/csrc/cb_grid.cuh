@@ -45,10 +45,8 @@ __device__ __forceinline__ bool grid_sync(uint32_t *ctr, uint32_t &epoch) {
   bool ok = true;
   __syncthreads();
   if (gridDim.x > 1 && threadIdx.x == 0) {
-    __threadfence();
-    red_release(ctr, 1u);
-    ok = grid_wait(ctr, epoch * gridDim.x);
-    __threadfence();
+    red_release(ctr, 1u);  // with the barrier above: after every store of the CTA
+    ok = grid_wait(ctr, epoch * gridDim.x);  // acquire; the barrier below passes it on
   }
   return __syncthreads_and(ok) != 0;
 }

@@ -28,8 +28,8 @@ constexpr uint32_t kHeavyDeg = 8192; // rows above this degree are split across 
 constexpr uint32_t kChunk = 4096;    // edges per heavy-row chunk
 constexpr uint32_t kLongDeg = 1024;  // rows above this (<= kHeavyDeg) use the whole CTA
 constexpr int kNodeAlign = 32;       // per-instance node offset alignment (elements)
-// Realisations of at most kSmallN nodes and kSmallNnz entries can run all
-// their Lanczos steps in one launch, one CTA each (lanczos_small_kernel).
+// Realisations up to this size are "small" to the tuner: their automatic path
+// is timed beside the per-step ones.
 constexpr uint32_t kSmallN = 8192;
 constexpr uint32_t kSmallNnz = 1u << 20;
 
@@ -152,6 +152,9 @@ struct Workspace {
   double *rpart = nullptr; // reorthogonalisation: per finalize tile, ms dot partials
   double *rh = nullptr;    // reorthogonalisation: per realisation, ms coefficients
   uint32_t *hcnt = nullptr;// heavy-row arrival counters
+  double *tparts = nullptr;  // team kernel: partials of the CTAs
+  uint32_t *tctr = nullptr;  // team kernel: barrier counters
+  double *xd = nullptr;    // team kernel: dot products of its Gram-Schmidt passes
   size_t blob_bytes = 0;
   void *blob = nullptr;    // single allocation backing sc/part/gpart/cnt
   uint64_t gen = 0;        // allocation generation (process-wide unique)
@@ -183,7 +186,13 @@ struct cb_graph {
   uint32_t total_slots = 0, total_groups = 0;
   int lanes = 8;  // lanes per row for short rows (1, 2, 4, 8, 16, 32)
   int path = CB_PATH_AUTO;  // FP32 SpMV path (cb_graph_set_path)
+  bool tuned_auto = false;  // the tuner found the automatic path fastest and kept a per-step one
+                            // beside it (cb_graph_tune)
   uint32_t n_sm = 1;        // SMs of the handle's device
+  // a group handle of the budgeted adjoint plans its teams as part of the
+  // whole handle, so that the groups' results are the whole's bit for bit
+  const cb_graph *plan_of = nullptr;
+  uint32_t plan_r0 = 0;
   bool owns_csr = true;     // false while an upload holds CSR arrays its caller still owns
   std::vector<cb::InstDesc> inst;        // host copy
   std::vector<cb::HeavyRow> heavy;       // host copy
@@ -320,6 +329,7 @@ int dbg_read_lanczos(uint32_t *count, uint64_t *first, bool reset);
 int dbg_read_blocked(uint32_t *count, uint64_t *first, bool reset);
 int dbg_read_twophase(uint32_t *count, uint64_t *first, bool reset);
 int dbg_read_adjoint(uint32_t *count, uint64_t *first, bool reset);
+int dbg_read_team(uint32_t *count, uint64_t *first, bool reset);
 
 // fn(i) for i in [0, n) on the host, spread over the hardware threads
 void parallel_for(uint32_t n, const std::function<void(uint32_t)> &fn);

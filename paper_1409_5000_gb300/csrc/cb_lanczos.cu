@@ -34,11 +34,12 @@
 // kHeavyDeg are cut into kChunk-edge chunks, one CTA per chunk, and the last
 // chunk to finish completes the row.  Column indices are streamed with an
 // evict-first hint; the gathered vector stays cache-resident.
-#include <cstdio>
+#include <algorithm>
 
 #include "cb_internal.cuh"
 #include "cb_reduce.cuh"
 #include "cb_step.cuh"
+#include "cb_team.cuh"
 
 namespace cb {
 
@@ -80,8 +81,12 @@ __global__ void __launch_bounds__(kThreads) init_indicator_kernel(LArgs a, uint3
 __global__ void __launch_bounds__(kThreads) init_scalars_kernel(LArgs a, uint32_t r0, uint32_t r1,
                                                                 uint32_t m, const uint32_t *idx,
                                                                 uint32_t k, bool per_inst,
-                                                                const double *rscale) {
+                                                                const double *rscale,
+                                                                uint32_t *tctr) {
   const uint32_t ms = a.sc.ms;
+  // the team kernel's barrier counters
+  if (blockIdx.x == 0)
+    for (uint32_t q = threadIdx.x; q < kMaxTeams; q += blockDim.x) tctr[q * kCtrStride] = 0u;
   const uint64_t total = (uint64_t)(r1 - r0) * ms;
   for (uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total;
        q += (uint64_t)gridDim.x * blockDim.x) {
@@ -613,8 +618,10 @@ __global__ void __launch_bounds__(kThreads) finalize_beta_kernel(LArgs a, uint32
 }
 
 // ---------------------------------------------------------------------------
-// Small realisations (n <= kSmallN, at most kSmallNnz entries): one CTA per
-// realisation runs all m Lanczos steps in one launch -- SpMV with the row
+// Small realisations (n <= kSmallN, at most kSmallNnz entries) in FP64 without
+// reorthogonalisation (the team kernel takes the others, cb_team.cu; here the
+// order of the sums stays, which decides the trailing part of T once
+// orthogonality is lost): one CTA per realisation runs all m Lanczos steps in one launch -- SpMV with the row
 // epilogue, alpha, the axpy w = u - alpha_j scale_j W_j, beta_j and the
 // breakdown test, the same arithmetic as spmv_kernel + finalize_kernel +
 // finalize_beta_kernel -- with W_j, W_{j-1} and the new vector resident in
@@ -979,28 +986,45 @@ static int run_t(cb_graph *h, Workspace &W, uint32_t r0, uint32_t r1, uint32_t m
                                                                       start_idx ? T(0) : T(1));
   if (start_idx && !rscale)
     init_indicator_kernel<T><<<r1 - r0, kThreads, 0, s>>>(a, r0, start_idx, k, per_inst);
+  // on-chip problems on the automatic path: the whole recurrence in one launch
+  TeamArgs ta;
+  uint32_t team_grid = 0;
+  bool team_coop = false;
+  const bool one_launch = (h->path == CB_PATH_AUTO || h->tuned_auto) && h->stall_btile == UINT32_MAX;
+  const cb_graph *hp = h->plan_of ? h->plan_of : h;  // a group handle decides as the whole one
+  const uint32_t p0 = h->plan_of ? 0u : r0, p1 = h->plan_of ? hp->n_inst : r1;
+  bool small = true;
+  for (uint32_t r = p0; r < p1 && small; ++r) small = hp->inst[r].n <= kSmallN && hp->inst[r].nnz <= kSmallNnz;
+  // a team sums in an order of its own: taken where that cannot show, FP64 with
+  // reorthogonalisation and FP32 ensembles and small graphs.  One larger graph in
+  // FP32 keeps the order of the per-step kernels (a planted clique's scores differ
+  // by less than FP32 rounding), as does FP64 without it (T's trailing part)
+  const bool team = one_launch &&
+                    (sizeof(T) == 8 ? h->reorth : !h->reorth && (small || p1 - p0 > 1)) &&
+                    team_plan(h, r0, r1, sizeof(T), h->reorth, &ta, &team_grid, &team_coop);
   const uint64_t nsc = (uint64_t)(r1 - r0) * W.sc.ms;
   init_scalars_kernel<<<(uint32_t)((nsc + kThreads - 1) / kThreads), kThreads, 0, s>>>(
-      a, r0, r1, m, start_idx, k, per_inst, rscale);
+      a, r0, r1, m, start_idx, k, per_inst, rscale, W.tctr);
   prof_end(tok, s);
-  // small realisations only (and the automatic path, no reorthogonalisation):
-  // the whole recurrence in one launch, one CTA per realisation
-  bool small = h->path == CB_PATH_AUTO && !h->reorth && h->stall_btile == UINT32_MAX;
-  for (uint32_t r = r0; r < r1 && small; ++r) small = h->inst[r].n <= kSmallN && h->inst[r].nnz <= kSmallNnz;
-  if (small) {
-    const size_t shm = 3 * (size_t)((nmax + 3) & ~3u) * sizeof(T);
-    static bool attr = false;
-    if (!attr) {
+  if (team) {
+    ta.parts = W.tparts;
+    ta.ctr = W.tctr;
+    ta.xd = W.xd;
+    tok = prof_begin(CB_K_SPMV, s);
+    const int rc = team_launch<T>(a, ta, r0, m, team_grid, team_coop, s);
+    prof_end(tok, s);
+    return rc;
+  }
+  if constexpr (sizeof(T) == 8) {
+    if (small && one_launch && !h->reorth) {
       cudaFuncSetAttribute(lanczos_small_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(3 * kSmallN * sizeof(double)));
-      cudaFuncSetAttribute(lanczos_small_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(3 * kSmallN * sizeof(double)));
-      attr = true;
+      tok = prof_begin(CB_K_SPMV, s);
+      lanczos_small_kernel<double><<<r1 - r0, kSmallThreads, 3 * (size_t)((nmax + 3) & ~3u) * sizeof(double), s>>>(
+          a, r0, m);
+      prof_end(tok, s);
+      return cuda_error(cudaGetLastError(), "lanczos launch");
     }
-    tok = prof_begin(CB_K_SPMV, s);
-    lanczos_small_kernel<T><<<r1 - r0, kSmallThreads, shm, s>>>(a, r0, m);
-    prof_end(tok, s);
-    return cuda_error(cudaGetLastError(), "lanczos launch");
   }
   for (uint32_t j = 0; j < m; ++j) {
     tok = prof_begin(CB_K_SPMV, s);

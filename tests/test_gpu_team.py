@@ -1,0 +1,66 @@
+"""The one-launch recurrence (teams of CTAs) at its edges, against the oracle:
+teams of one and of many, rows for a lane, a warp and the CTA, empty rows,
+16- and 32-bit columns, breakdowns, the most realisations (needs a GB300).
+
+Bars: the suite's (parity.py) against the oracle; with reorthogonalisation in
+FP64 the per-step kernels run the same scheme in another order of sums, so the
+scores of the two agree to 1e-12 (sums of at most 1e4 terms of relative rounding
+1.1e-16, and the head's scores are within 1e3 of each other)."""
+import numpy as np
+import pytest
+
+import oracle.communicability as oc
+from paper_1409_5000_gb300 import synth
+from tests import parity
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _hubs(n, hubs, seed):
+    """An ER graph with a few nodes joined to many others."""
+    rng = np.random.default_rng(seed)
+    e = [rng.integers(0, n, (3 * n, 2))]
+    for h, d in enumerate(hubs):
+        e.append(np.stack([np.full(d, h), rng.choice(np.arange(len(hubs), n), d, replace=False)], axis=1))
+    e = np.concatenate(e)
+    return synth.from_edges(n, e[e[:, 0] != e[:, 1]])
+
+
+def _sets():
+    er = lambda n, d, s: synth.er(n, d / max(n - 1, 1), s)  # noqa: E731
+    k7 = synth.from_edges(7, [(i, j) for i in range(7) for j in range(i)])
+    return {
+        "tiny": [synth.from_edges(1, np.zeros((0, 2))), synth.from_edges(2, [(0, 1)]), k7, er(33, 4, 1)],
+        "one": [er(8191, 6, 2)],
+        "uneven": [er(n, 9, n) for n in (500, 1023, 1025, 4097, 8192)],
+        "hubs": [_hubs(7001, (6000, 2049, 2048, 1025, 600, 300), 3), er(300, 5, 4)],
+        "large": [er(30_011, 12, 5), _hubs(20_003, (9000, 3000), 6)],
+        "wide": [er(70_001, 8, 7), er(66_000, 3, 8)],
+        "most": [er(200 + q, 6, q) for q in range(160)],
+        "beyond": [er(150 + q, 6, q) for q in range(161)],
+    }
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("name", sorted(_sets()))
+def test_matches_oracle(name, prec):
+    from paper_1409_5000_gb300 import binding as B
+
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for -m gpu tests")
+    graphs = _sets()[name]
+    m, p = 15, (B.CB_FP32 if prec == "fp32" else B.CB_FP64 | B.CB_REORTH)
+    th_o, S_o = oc.ensemble_scores([(g.n, g.row_ptr, g.col) for g in graphs], m)
+    with B.GraphSet(graphs) as gs:
+        ls, S, rep = B.ensemble_scores(gs, m, p, report=True)
+        parity.assert_scores(float(ls.item()), S.cpu().numpy(), th_o, S_o, prec)
+        if prec == "fp64":
+            with B.GraphSet(graphs, path=B.CB_PATH_CSR) as ref:
+                ls_r, S_r = B.ensemble_scores(ref, m, p)
+            e = parity.errors(float(ls.item()), S.cpu().numpy(), float(ls_r.item()), S_r.cpu().numpy())
+            assert e["head_rel"] <= 1e-12 and e["norm_rel"] <= 1e-12, e
+        if name == "tiny":  # breakdowns: an empty graph, K_2 and K_7 are spanned by 1
+            assert [r.m_eff for r in rep[:3]] == [1, 1, 1]
+        again = B.ensemble_scores(gs, m, p)[1]
+        assert torch.equal(S, again)

@@ -143,13 +143,18 @@ __global__ void __launch_bounds__(kThreads) spmv_kernel(LArgs a, uint32_t j, uin
   } else {
     tile = tile_off + (blockIdx.x - n_chunks);
     r = a.tile_inst[tile];
+    // the tile's row offsets, staged once (coalesced); fixed by the upload
+    const uint2 tr = a.tile_rows[tile];
+    const uint32_t *rp = a.row_ptr + a.inst[r].rp_base + tr.x;
+    for (uint32_t q = threadIdx.x; q <= tr.y - tr.x; q += kThreads) s_rp[q] = rp[q];
   }
+  dep_wait();
+  dep_trigger();
   if (j >= a.sc.meff[r]) return;  // realisation stopped (uniform per CTA)
   if (a.skip_blocked && a.inst[r].blocked) return;  // the column-blocked kernel owns it
   if (a.skip_pb && a.inst[r].pb) return;            // the two-phase kernels own it
 
   const InstDesc &I = a.inst[r];
-  const uint32_t *rp = a.row_ptr + I.rp_base;
   const uint32_t *col = a.col + I.edge_base;
   T *Vb = reinterpret_cast<T *>(a.V);
   const T *x = Vb + (uint64_t)j * a.vs + I.node_base;
@@ -168,9 +173,7 @@ __global__ void __launch_bounds__(kThreads) spmv_kernel(LArgs a, uint32_t j, uin
   const uint2 tr = a.tile_rows[tile];
   const uint32_t row0 = tr.x;
   const uint32_t nrows = tr.y - tr.x;  // <= kTileRows
-  // the tile's row offsets, staged once (coalesced)
-  for (uint32_t q = threadIdx.x; q <= nrows; q += kThreads) s_rp[q] = rp[row0 + q];
-  __syncthreads();
+  __syncthreads();  // s_rp
 
   T acc = T(0);
   const uint32_t lane_g = threadIdx.x % G;
@@ -345,6 +348,8 @@ __global__ void __launch_bounds__(kBThreads, 1) bspmv_kernel(LArgs a, uint32_t j
   __shared__ uint64_t s_seg[kBMaxBlocks + 1];     // stream offset of each column block's segment
   const uint32_t t = btile_off + blockIdx.x;
   const uint32_t r = a.btile_inst[t];
+  dep_wait();
+  dep_trigger();
   if (j >= a.sc.meff[r]) return;
   const InstDesc &I = a.inst[r];
   const uint32_t ms = a.sc.ms;
@@ -549,10 +554,10 @@ __global__ void __launch_bounds__(kThreads) finalize_kernel(LArgs a, uint32_t j,
   // CTA's latency chain is most of its lifetime); a finished realisation
   // only reads them
   T u[8], v[8];
-  if (full) {
-    Vec8<T>::load(out + i0, u);
-    Vec8<T>::load(x + i0, v);
-  }
+  if (full) Vec8<T>::load(x + i0, v);  // W_j: complete before the SpMV began
+  dep_wait();
+  dep_trigger();
+  if (full) Vec8<T>::load(out + i0, u);
   if (j >= a.sc.meff[r]) return;
   const T coef = (T)(a.sc.alpha[r * ms + j] * a.sc.scale[r * ms + j]);
   T acc = T(0);
@@ -584,8 +589,10 @@ __global__ void __launch_bounds__(kThreads) finalize_kernel(LArgs a, uint32_t j,
 __global__ void __launch_bounds__(kThreads) finalize_beta_kernel(LArgs a, uint32_t j, uint32_t r0) {
   __shared__ double s_red[kThreads / 32];
   const uint32_t r = r0 + blockIdx.x;
-  if (j >= a.sc.meff[r]) return;
   const RedPlan P = a.inst[r].fin;
+  dep_wait();
+  dep_trigger();
+  if (j >= a.sc.meff[r]) return;
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (uint32_t g = warp; g < P.n_groups; g += kThreads / 32) {
     const uint32_t gsize = min((uint32_t)kGroup, P.n_slots - g * kGroup);
@@ -880,7 +887,7 @@ template <typename T, int G>
 static void launch_spmv(const LArgs &a, uint32_t j, uint32_t chunk_off, uint32_t n_chunks,
                         uint32_t tile_off, uint32_t n_tiles, cudaStream_t s) {
   const uint32_t grid = n_chunks + n_tiles;
-  if (grid) spmv_kernel<T, G><<<grid, kThreads, 0, s>>>(a, j, chunk_off, n_chunks, tile_off);
+  if (grid) launch_dep(spmv_kernel<T, G>, grid, kThreads, 0, s, a, j, chunk_off, n_chunks, tile_off);
 }
 
 template <typename T>
@@ -1029,15 +1036,15 @@ static int run_t(cb_graph *h, Workspace &W, uint32_t r0, uint32_t r1, uint32_t m
   for (uint32_t j = 0; j < m; ++j) {
     tok = prof_begin(CB_K_SPMV, s);
     if (any_csr) launch_spmv_lanes<T>(h->lanes, a, j, chunk_off, n_chunks, tile_off, n_tiles, s);
-    if (n_btiles) bspmv_kernel<<<n_btiles, kBThreads, kBSmemBytes, s>>>(a, j, btile_off);
+    if (n_btiles) launch_dep(bspmv_kernel, n_btiles, kBThreads, kBSmemBytes, s, a, j, btile_off);
     if (any_pb)
       launch_twophase(a, h->lanes, j, ptile_lo, ptile_hi, pg_lo, pg_hi, chunk_off, n_chunks,
                       bin_off, n_bins, s);
     prof_end(tok, s);
     tok = prof_begin(CB_K_FINALIZE, s);
     if (n_fin) {
-      finalize_kernel<T><<<n_fin, kThreads, 0, s>>>(a, j, fin_off);
-      finalize_beta_kernel<<<r1 - r0, kThreads, 0, s>>>(a, j, r0);
+      launch_dep(finalize_kernel<T>, n_fin, kThreads, 0, s, a, j, fin_off);
+      launch_dep(finalize_beta_kernel, r1 - r0, kThreads, 0, s, a, j, r0);
     }
     if (n_fin && h->reorth)
       for (int pass = 0; pass < 2; ++pass) {

@@ -49,6 +49,38 @@ struct LArgs {
   uint32_t skip_pb;  // the tiled-CSR kernel leaves two-phase realisations alone
 };
 
+// ---------------------------------------------------------------------------
+// Dependent launch.  The kernels of a step follow each other on one stream and
+// each needs what the one before wrote, so a launch boundary (about 2 us: drain,
+// launch, first loads) sits between them several times a step.  launch_dep
+// lets a kernel's CTAs become resident, and load what no kernel of the
+// recurrence writes, while the kernel before still runs:
+//  * dep_wait: returns when the kernels before have completed and their writes
+//    are visible.  Every CTA of a kernel launched this way calls it, whatever it
+//    does afterwards, so that a kernel never completes before its predecessor;
+//  * dep_trigger, after dep_wait: once every CTA has called it (or ended), the
+//    next kernel's CTAs may be launched.  What that kernel reads before its own
+//    dep_wait was therefore complete two kernels before it.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline void launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t shm, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = shm;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);  // errors are picked up by cudaGetLastError
+}
+
 // Column indices are read once per step: streaming (evict-first) load.
 __device__ __forceinline__ uint32_t ld_stream(const uint32_t *p) { return __ldcs(p); }
 

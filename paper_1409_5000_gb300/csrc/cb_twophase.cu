@@ -432,6 +432,8 @@ __global__ void __launch_bounds__(kP1Threads, 1) pscatter_kernel(LArgs a, uint32
   __shared__ uint32_t s_tile, s_issued[kP1Bufs], s_used[kP1Bufs];
   __shared__ int s_go, s_fail;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  dep_wait();
+  dep_trigger();
   const uint64_t span = g_hi - g_lo;
   uint64_t gb = g_lo + span * blockIdx.x / gridDim.x;
   const uint64_t ge = g_lo + span * (blockIdx.x + 1) / gridDim.x;
@@ -609,6 +611,8 @@ __global__ void __launch_bounds__(kP2Threads, 2) pgather_kernel(LArgs a, uint32_
   __shared__ uint32_t s_done;
   __shared__ int s_fail;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  dep_wait();
+  dep_trigger();
 
   if (blockIdx.x < n_chunks) {  // one chunk of a heavy row of a two-phase realisation
     const uint32_t cidx = chunk_off + blockIdx.x;
@@ -760,8 +764,8 @@ void launch_p2(const LArgs &a, uint32_t j, uint32_t chunk_off, uint32_t n_chunks
     attr = true;
   }
   // prefetch distance: the CTAs resident at once (two per SM)
-  pgather_kernel<<<n_chunks + n_bins, kP2Threads, kP2SmemBytes, s>>>(a, j, chunk_off, n_chunks, bin_off,
-                                                                     n_bins, 2u * (uint32_t)n_sm);
+  launch_dep(pgather_kernel, n_chunks + n_bins, kP2Threads, kP2SmemBytes, s, a, j, chunk_off, n_chunks, bin_off,
+             n_bins, 2u * (uint32_t)n_sm);
 }
 
 template <typename P>
@@ -789,7 +793,7 @@ void launch_twophase(const LArgs &a, int lanes, uint32_t j, uint32_t tile_lo, ui
     // one CTA per SM, each at least 1024 groups
     const uint64_t want = (g_hi - g_lo + 1023) / 1024;
     const uint32_t grid = (uint32_t)std::min<uint64_t>((uint64_t)n_sm, want);
-    pscatter_kernel<<<grid, kP1Threads, kP1SmemBytes, s>>>(a, j, tile_lo, tile_hi, g_lo, g_hi);
+    launch_dep(pscatter_kernel, grid, kP1Threads, kP1SmemBytes, s, a, j, tile_lo, tile_hi, g_lo, g_hi);
   }
   if (n_chunks + n_bins) launch_p2(a, j, chunk_off, n_chunks, bin_off, n_bins, n_sm, s);
   (void)lanes;  // the sliced rows of phase 2 need no group width

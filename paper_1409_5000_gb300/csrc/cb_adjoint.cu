@@ -136,12 +136,37 @@ __global__ void __launch_bounds__(64) bw_tridiag_kernel(Scalars s1, Scalars sw,
   }
 }
 
+// 16 bytes of consecutive values
+__device__ __forceinline__ void ld16(const float *p, float (&v)[4]) {
+  const float4 x = *reinterpret_cast<const float4 *>(p);
+  v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+}
+__device__ __forceinline__ void ld16(const double *p, double (&v)[2]) {
+  const double2 x = *reinterpret_cast<const double2 *>(p);
+  v[0] = x.x; v[1] = x.y;
+}
+
+// B-byte asynchronous copy global -> shared (both addresses B-byte aligned)
+template <int B>
+__device__ __forceinline__ void cp_async(void *smem, const void *gmem) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem);
+  if constexpr (B == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(gmem), "n"(B) : "memory");
+}
+
 // Node-major P = exp(theta_r - theta*) V_w K_r and U = V_1 (scales applied).
-// One CTA per finalize tile (kFinRows nodes of one realisation), 4 warps;
-// each warp stages 32 nodes' basis values in shared memory and writes the
-// node-major rows with lanes over the row index (coalesced).  All per-node
-// arithmetic runs in T: the FP64 scalars are converted once per CTA (FP64
-// instructions are scarce on GB300).
+// One CTA per finalize tile (kFinRows nodes of one realisation), 4 warps.  A
+// warp copies 32 nodes' basis values to shared memory asynchronously (all 2 m
+// lines in flight; the scales go into K and into the stored U); lane b then holds
+// P_q,b of all 32 nodes q in registers, so that a step of the sum over a takes
+// one load of K and 32 values of V_w by 16-byte broadcasts for 32 products
+// (2.3 ms on 64 graphs of 1e5 nodes at m = 30 when every product loaded both of
+// its operands, and U was read back through one bank; now 0.72), and writes
+// the node-major rows with lanes over the row index (coalesced).  All
+// per-node arithmetic runs in T: the FP64 scalars are converted once per CTA
+// (FP64 instructions are scarce on GB300).
 template <typename T>
 __global__ void __launch_bounds__(128) bw_node_kernel(const T *V1, const T *Vw, uint64_t vs,
                                                       Scalars s1, Scalars sw,
@@ -150,11 +175,11 @@ __global__ void __launch_bounds__(128) bw_node_kernel(const T *V1, const T *Vw, 
                                                       uint32_t kdim, const double *theta_in,
                                                       uint32_t mpad, T *P, T *U,
                                                       double *log_scale) {
-  extern __shared__ unsigned char s_raw[];
-  T *sK = reinterpret_cast<T *>(s_raw);              // kdim * kdim
-  T *sV = sK + kdim * kdim;                          // 4 warps x kdim x 32 (V_w values)
-  T *sW = sV + 4 * kdim * 32;                        // 4 warps x kdim x 32 (V_1 values)
-  __shared__ T s_sc1[kMaxAdjM], s_scw[kMaxAdjM];
+  extern __shared__ float4 s_raw4[];
+  T *sV = reinterpret_cast<T *>(s_raw4);             // 4 warps x kdim x 32 (V_w values)
+  T *sW = sV + 4 * kdim * 32;                        // 4 warps x kdim x 33 (V_1 values)
+  T *sK = sW + 4 * kdim * 33;                        // kdim * kdim
+  __shared__ T s_sc1[kMaxAdjM];
   __shared__ double s_wmax[4];
   const uint32_t t = blockIdx.x;
   const uint32_t r = fin_inst[t];
@@ -169,54 +194,56 @@ __global__ void __launch_bounds__(128) bw_node_kernel(const T *V1, const T *Vw, 
   const bool active = th > -1e307;
   const int M1 = active ? (int)s1.meff[r] : 0, Mw = active ? (int)sw.meff[r] : 0;
   for (int q = threadIdx.x; q < M1; q += blockDim.x) s_sc1[q] = (T)s1.scale[r * s1.ms + q];
-  for (int q = threadIdx.x; q < Mw; q += blockDim.x) s_scw[q] = (T)sw.scale[r * sw.ms + q];
   __syncthreads();
   const double tmax = fmax(fmax(s_wmax[0], s_wmax[1]), fmax(s_wmax[2], s_wmax[3]));
   if (t == 0 && threadIdx.x == 0) *log_scale = tmax > -1e307 ? tmax : 0.0;
   const double f = active ? exp(th - tmax) : 0.0;
   for (uint32_t q = threadIdx.x; q < (uint32_t)(Mw * M1); q += blockDim.x) {
     const uint32_t a = q / M1, b = q % M1;
-    sK[a * kdim + b] = (T)(f * K[(size_t)r * kdim * kdim + a * kdim + b]);
+    sK[a * kdim + b] = (T)(f * sw.scale[r * sw.ms + a] * K[(size_t)r * kdim * kdim + a * kdim + b]);
   }
   __syncthreads();
-  T *myV = sV + warp * kdim * 32, *myW = sW + warp * kdim * 32;
+  T *myV = sV + warp * kdim * 32, *myW = sW + warp * kdim * 33;
   const uint32_t i0 = (t - I.fin_base) * kFinRows, i1 = min(i0 + kFinRows, I.n);
   for (uint32_t base = i0 + warp * 32; base < i1; base += 4 * 32) {
-    const uint32_t i = base + lane;
-    const bool valid = i < i1;
-    for (int a = 0; a < Mw; ++a)
-      myV[a * 32 + lane] = valid ? s_scw[a] * Vw[(uint64_t)a * vs + I.node_base + i] : T(0);
-    for (int b = 0; b < M1; ++b)
-      myW[b * 32 + lane] = valid ? s_sc1[b] * V1[(uint64_t)b * vs + I.node_base + i] : T(0);
+    // whole groups of 32 nodes: the node ranges are padded to them
+    const T *gw = Vw + I.node_base + base, *g1 = V1 + I.node_base + base + lane;
+    constexpr uint32_t kV = 16 / sizeof(T), kParts = 32 / kV;  // 16-byte parts of a vector's 32 values
+    for (uint32_t q = lane; q < Mw * kParts; q += 32) {
+      const uint32_t a = q / kParts, part = (q % kParts) * kV;
+      cp_async<16>(myV + a * 32 + part, gw + (uint64_t)a * vs + part);
+    }
+    for (int b = 0; b < M1; ++b) cp_async<sizeof(T)>(myW + b * 33 + lane, g1 + (uint64_t)b * vs);
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncwarp();
     const uint32_t nn = min(32u, i1 - base);
-    for (uint32_t q = 0; q < nn; ++q) {
-      const uint64_t row = (I.node_base + base + q) * (uint64_t)mpad;
-      for (uint32_t b = lane; b < mpad; b += 32) {
-        T p = T(0), u = T(0);
-        if ((int)b < M1) {
-          for (int a = 0; a < Mw; ++a) p += myV[a * 32 + q] * sK[a * kdim + b];
-          u = myW[b * 32 + q];
+    for (uint32_t b = lane; b < ((mpad + 31) & ~31u); b += 32) {  // uniform trip count
+      const bool in = (int)b < M1;
+      T p[32];
+#pragma unroll
+      for (int q = 0; q < 32; ++q) p[q] = T(0);
+      for (int a = 0; a < Mw; ++a) {
+        const T k = in ? sK[a * kdim + b] : T(0);
+#pragma unroll
+        for (int q = 0; q < 32; q += (int)kV) {
+          T v[kV];
+          ld16(myV + a * 32 + q, v);
+#pragma unroll
+          for (int u = 0; u < (int)kV; ++u) p[q + u] += v[u] * k;
         }
-        P[row + b] = p;
-        U[row + b] = u;
+      }
+      if (b < mpad) {
+        T *Pr = P + (I.node_base + base) * (uint64_t)mpad + b, *Ur = U + (I.node_base + base) * (uint64_t)mpad + b;
+#pragma unroll
+        for (uint32_t q = 0; q < 32; ++q)
+          if (q < nn) {
+            Pr[(uint64_t)q * mpad] = p[q];
+            Ur[(uint64_t)q * mpad] = in ? s_sc1[b] * myW[b * 33 + q] : T(0);
+          }
       }
     }
     __syncwarp();
   }
-}
-
-// dot of 4 consecutive values of a with 4 of b (16- or 32-byte aligned)
-__device__ __forceinline__ float dot4(const float *a, const float *b) {
-  const float4 x = *reinterpret_cast<const float4 *>(a), y = *reinterpret_cast<const float4 *>(b);
-  return x.x * y.x + x.y * y.y + x.z * y.z + x.w * y.w;
-}
-__device__ __forceinline__ double dot4(const double *a, const double *b) {
-  const double2 x0 = *reinterpret_cast<const double2 *>(a);
-  const double2 x1 = *reinterpret_cast<const double2 *>(a + 2);
-  const double2 y0 = *reinterpret_cast<const double2 *>(b);
-  const double2 y1 = *reinterpret_cast<const double2 *>(b + 2);
-  return x0.x * y0.x + x0.y * y0.y + x1.x * y1.x + x1.y * y1.y;
 }
 
 // mirror[e] for every CSR entry e = (i, j) of one SpMV tile: the position of
@@ -256,16 +283,42 @@ __global__ void __launch_bounds__(256) bw_mirror_kernel(const InstDesc *inst,
   }
 }
 
+// 4 consecutive values (16- or 32-byte aligned)
+template <typename T>
+struct Quad {
+  T v[4];
+};
+__device__ __forceinline__ Quad<float> ld_quad(const float *p) {
+  const float4 x = *reinterpret_cast<const float4 *>(p);
+  return {{x.x, x.y, x.z, x.w}};
+}
+__device__ __forceinline__ Quad<double> ld_quad(const double *p) {
+  const double2 x = *reinterpret_cast<const double2 *>(p), y = *reinterpret_cast<const double2 *>(p + 2);
+  return {{x.x, x.y, y.x, y.y}};
+}
+template <typename T>
+__device__ __forceinline__ T dot4(const Quad<T> &a, const Quad<T> &b) {
+  return a.v[0] * b.v[0] + a.v[1] * b.v[1] + a.v[2] * b.v[2] + a.v[3] * b.v[3];
+}
+
 // The gradient is symmetric: g(i, j) = P_i . U_j + P_j . U_i = g(j, i).  Each
 // undirected edge is computed once, from its upper entry (j >= i, a suffix
 // of the sorted row i), and written to both CSR entries (the lower one
-// through mirror).  A group of kEdgeLanes lanes shares an edge: lane c takes
-// the 4-value chunks c, c + kEdgeLanes, ... of the four node-major rows, so
-// each row is read as whole 128-byte lines; the partials are summed across
-// the group with a shuffle tree.  Arithmetic in T (FP32 in CB_FP32 mode):
-// FP64 instructions are scarce on GB300 and would bound this kernel.
+// through mirror).  A warp takes an equal run of the tile's upper entries, 32
+// at a time: each lane finds the row, column and mirror of one entry, and the
+// result is stored by that lane; the dot products go four entries at a time,
+// kEdgeLanes lanes each, lane c reading the 4-value chunks c, c + kEdgeLanes of
+// the four node-major rows as whole 128-byte lines, two such steps in flight,
+// and a shuffle tree sums the partials.  Entries of one row meet in one load
+// instruction, so P_i and U_i cost little.  Latency bounds it (L2 at a quarter
+// of its throughput): 64 graphs of 1e5 nodes, 8e5 edges each, at m = 30 took
+// 3.62 ms with one dependent chain (row, column, rows, stores) per edge and
+// group, 3.98 ms with P_i and U_i kept in registers per group (few warps, groups
+// of a warp in rows of different lengths), 2.44 ms now.  Arithmetic in T (FP32
+// in CB_FP32 mode): FP64 instructions are scarce on GB300 and would bound this
+// kernel.
 constexpr uint32_t kEdgeLanes = 8;
-template <typename T>
+template <typename T, int NC>  // NC: chunks of a lane (rows of up to 32 NC values)
 __global__ void __launch_bounds__(256) bw_edge_kernel(const T *P, const T *U, uint32_t mpad,
                                                       const InstDesc *inst,
                                                       const uint32_t *tile_inst,
@@ -323,34 +376,63 @@ __global__ void __launch_bounds__(256) bw_edge_kernel(const T *P, const T *U, ui
   __syncthreads();
   const uint32_t nup = s_up[nrows];
   const bool active = theta_in[r] > -1e307;
-  const uint32_t nv = mpad / 4;
-  const uint32_t c0 = threadIdx.x % kEdgeLanes;
-  constexpr uint32_t kGroups = 256 / kEdgeLanes;
-  // the loop bound is uniform across each group, so the shuffles see all lanes
-  for (uint32_t ub = 0; ub < nup; ub += kGroups) {
-    const uint32_t u = ub + threadIdx.x / kEdgeLanes;
-    T g = T(0);
-    uint32_t e = 0;
-    if (u < nup) {
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t c0 = lane % kEdgeLanes, grp = lane / kEdgeLanes;
+  constexpr uint32_t kStep = 32 / kEdgeLanes;  // entries of a step
+  constexpr uint32_t kFly = NC == 1 && sizeof(T) == 4 ? 2 : 1;  // steps in flight
+  const uint32_t u1 = (uint32_t)((uint64_t)nup * (warp + 1) / 8);
+  for (uint32_t ub = (uint32_t)((uint64_t)nup * warp / 8); ub < u1; ub += 32) {
+    const uint32_t u = ub + lane;
+    uint32_t row = row0, j = row0, e = 0, mi = 0;
+    if (u < u1) {
       uint32_t lo = 0, hi = nrows;  // s_up[lo] <= u < s_up[hi]
       while (hi - lo > 1) {
         const uint32_t mid = (lo + hi) >> 1;
         if (s_up[mid] <= u) lo = mid; else hi = mid;
       }
       e = s_first[lo] + (u - s_up[lo]);
-      if (active && CB_DCHECK(__ldg(cl + e) < I.n, kDbgAdjointCol, __ldg(cl + e))) {
-        const uint64_t i = I.node_base + row0 + lo;
-        const uint64_t j = I.node_base + __ldg(cl + e);
-        const T *Pi = P + i * mpad, *Ui = U + i * mpad, *Pj = P + j * mpad, *Uj = U + j * mpad;
-        for (uint32_t c = c0; c < nv; c += kEdgeLanes)
-          g += dot4(Pi + 4 * c, Uj + 4 * c) + dot4(Pj + 4 * c, Ui + 4 * c);
+      row = row0 + lo;
+      j = __ldg(cl + e);
+      mi = __ldg(mirror + I.edge_base + e);
+      if (!CB_DCHECK(j < I.n, kDbgAdjointCol, j)) j = row;
+    }
+    T res = T(0);
+    const uint32_t cnt = min(32u, u1 - ub);
+    for (uint32_t k0 = 0; k0 * kStep < cnt; k0 += kFly) {  // uniform over the warp
+      Quad<T> x[kFly][NC][4];
+#pragma unroll
+      for (uint32_t f = 0; f < kFly; ++f) {
+        const uint32_t src = (k0 + f) * kStep + grp;  // lanes past the run: row0 with itself
+        const uint64_t oi = (I.node_base + __shfl_sync(0xffffffffu, row, src)) * (uint64_t)mpad;
+        const uint64_t oj = (I.node_base + __shfl_sync(0xffffffffu, j, src)) * (uint64_t)mpad;
+#pragma unroll
+        for (int q = 0; q < NC; ++q) {
+          const uint32_t c = 4 * (c0 + q * kEdgeLanes);
+          if (c < mpad) {
+            x[f][q][0] = ld_quad(P + oi + c);
+            x[f][q][1] = ld_quad(U + oj + c);
+            x[f][q][2] = ld_quad(P + oj + c);
+            x[f][q][3] = ld_quad(U + oi + c);
+          } else {
+            x[f][q][0] = x[f][q][1] = x[f][q][2] = x[f][q][3] = Quad<T>{};
+          }
+        }
+      }
+#pragma unroll
+      for (uint32_t f = 0; f < kFly; ++f) {
+        T g = T(0);
+#pragma unroll
+        for (int q = 0; q < NC; ++q) g += dot4(x[f][q][0], x[f][q][1]) + dot4(x[f][q][2], x[f][q][3]);
+#pragma unroll
+        for (uint32_t off = kEdgeLanes / 2; off > 0; off >>= 1) g += __shfl_xor_sync(0xffffffffu, g, off, kEdgeLanes);
+        const T mine = __shfl_sync(0xffffffffu, g, (lane % kStep) * kEdgeLanes);
+        if (lane / kStep == k0 + f) res = mine;
       }
     }
-    for (uint32_t off = kEdgeLanes / 2; off > 0; off >>= 1)
-      g += __shfl_xor_sync(0xffffffffu, g, off, kEdgeLanes);
-    if (c0 == 0 && u < nup) {
-      grad[I.edge_base + e] = (float)g;
-      grad[I.edge_base + mirror[I.edge_base + e]] = (float)g;
+    if (u < u1) {
+      const float v = active ? (float)res : 0.f;
+      grad[I.edge_base + e] = v;
+      grad[I.edge_base + mi] = v;
     }
   }
 }
@@ -362,22 +444,22 @@ static int backward_t(cb_graph *h, uint32_t m, const uint32_t *idx, uint32_t k, 
   const uint32_t N = h->n_inst;
   prefer_shared(bw_tridiag_kernel);
   prefer_shared(bw_node_kernel<T>);
-  prefer_shared(bw_edge_kernel<T>);
+  prefer_shared(bw_edge_kernel<T, 1>);
+  prefer_shared(bw_edge_kernel<T, 2>);
   const int tok = prof_begin(CB_K_BACKWARD, s);
   const size_t shm_tri = 2 * sizeof(contour::Solve);
   cudaFuncSetAttribute(bw_tridiag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_tri);
   bw_tridiag_kernel<<<N, 64, shm_tri, s>>>(h->ws.sc, h->ws2.sc, h->d_inst, B.K, m, B.theta, B.cnt,
                                            contour::nodes(), sizeof(T) == 8 && !h->reorth);
-  const size_t shm = (size_t)(m * m + 8 * m * 32) * sizeof(T);
+  const size_t shm = (size_t)(m * m + 4 * m * 65) * sizeof(T);
   auto nk = bw_node_kernel<T>;
   if (shm > 48 * 1024) cudaFuncSetAttribute(nk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
   nk<<<h->total_fin, 128, shm, s>>>((const T *)h->ws.V, (const T *)h->ws2.V, h->ws.vec_stride,
                                     h->ws.sc, h->ws2.sc, h->d_inst, h->d_fin_inst, N, B.K, m,
                                     B.theta, B.mpad, (T *)B.P, (T *)B.U, log_scale);
-  bw_edge_kernel<T><<<h->total_tiles, 256, 0, s>>>((const T *)B.P, (const T *)B.U, B.mpad,
-                                                   h->d_inst, h->d_tile_inst, h->d_tile_rows,
-                                                   h->row_ptr, h->col, h->d_mirror,
-                                                   B.theta, grad);
+  auto ek = B.mpad <= 4 * kEdgeLanes ? bw_edge_kernel<T, 1> : bw_edge_kernel<T, 2>;
+  ek<<<h->total_tiles, 256, 0, s>>>((const T *)B.P, (const T *)B.U, B.mpad, h->d_inst, h->d_tile_inst,
+                                    h->d_tile_rows, h->row_ptr, h->col, h->d_mirror, B.theta, grad);
   prof_end(tok, s);
   (void)idx;
   (void)k;

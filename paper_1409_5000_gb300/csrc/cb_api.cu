@@ -462,8 +462,8 @@ CB_API int cb_debug_violations(uint32_t *count, uint64_t *first, int reset) {
   *first = 0;
   if (cb_debug_build() && cudaDeviceSynchronize() != cudaSuccess)
     return set_error(CB_ERR_CUDA, "cb_debug_violations: device synchronize");
-  int (*readers[5])(uint32_t *, uint64_t *, bool) = {dbg_read_lanczos, dbg_read_team, dbg_read_blocked,
-                                                     dbg_read_twophase, dbg_read_adjoint};
+  int (*readers[6])(uint32_t *, uint64_t *, bool) = {dbg_read_lanczos, dbg_read_team, dbg_read_blocked,
+                                                     dbg_read_twophase, dbg_read_adjoint, dbg_read_subgraph};
   for (auto rd : readers) {
     uint32_t c = 0;
     uint64_t f = 0;

@@ -330,6 +330,7 @@ int dbg_read_blocked(uint32_t *count, uint64_t *first, bool reset);
 int dbg_read_twophase(uint32_t *count, uint64_t *first, bool reset);
 int dbg_read_adjoint(uint32_t *count, uint64_t *first, bool reset);
 int dbg_read_team(uint32_t *count, uint64_t *first, bool reset);
+int dbg_read_subgraph(uint32_t *count, uint64_t *first, bool reset);
 
 // fn(i) for i in [0, n) on the host, spread over the hardware threads
 void parallel_for(uint32_t n, const std::function<void(uint32_t)> &fn);

@@ -5,9 +5,9 @@
 // The format lets the SpMV stage a block of kBCol entries of v_j in shared
 // memory and gather only from there:
 //   * rows are tiled by kBTileRows; thread i of a tile owns rows
-//     i + kBThreads * k, k = 0..kBRowsPerThread-1 (row slot k), and its row
-//     sums sit in shared memory at k * kBThreads + i, so the sums of one
-//     warp's rows fall in bank (i mod 32) of the owning lane;
+//     i + kBThreads * k, k = 0..kBRowsPerThread-1 (row slot k), and a warp's
+//     row sums sit together in shared memory, [slot][lane], so each falls
+//     in bank (i mod 32) of the owning lane;
 //   * a tile's edges are grouped by column block b = col >> kBColBits into
 //     one segment per (tile, b), and within it per warp: the elements of the
 //     warp's 512 rows, taken lane by lane (each lane's rows in slot order,
@@ -19,9 +19,9 @@
 //     most two of one lane's rows (at most two-way bank conflicts on the
 //     sums), while the padding stays a few percent instead of the spread
 //     between the warp's fullest and emptiest lane;
-//   * an element is one u32: the local column (col & (kBCol-1)) and, above
-//     it, the offset of its row sum from the warp's base (k * kBThreads +
-//     owner lane); steps are stored in pairs, [step / 2][lane][2], so a lane
+//   * an element is one u32: the byte offset of its column in the staged
+//     block and, above it, that of its row sum from the warp's base
+//     (4 (32 k + owner lane)); steps are stored in pairs, [step / 2][lane][2], so a lane
 //     reads two elements per 8-byte load and a warp 256 contiguous bytes;
 //   * padding elements read column 0 into the executing lane's spare sum
 //     (slot kBRowsPerThread), which the epilogue never reads.
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kFillThreads) bfill_kernel(const InstDesc *ins
       for (uint32_t j = s_tot[b * W + wl] + lane; j < 32 * T; j += 32) {
         const uint32_t s = j % T, l = j / T;
         const uint32_t q = 64 * (s >> 1) + 2 * l + (s & 1);
-        const uint32_t el = kBPadOff(l) << kBColBits;
+        const uint32_t el = kBElem(0, 32 * kBPadSlot + l);
         if (staged) stage[base + q] = el; else belem[st + q] = el;
       }
     }
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kFillThreads) bfill_kernel(const InstDesc *ins
 #pragma unroll 1
     for (int k = 0; k < kBRowsPerThread; ++k) {
       const uint32_t e1 = s_re1[k * kFillThreads + tid];
-      const uint32_t off = (uint32_t)k * kBThreads + lane;  // row sum of (slot k, lane)
+      const uint32_t off = (uint32_t)k * 32 + lane;  // row sum of (slot k, lane)
       uint32_t e = s_ecur[k * kFillThreads + tid];
       bool more = e < e1;
       while (more) {  // kFillBatch columns per round of loads
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(kFillThreads) bfill_kernel(const InstDesc *ins
           s_next[b * kFillThreads + tid] = p;
           if (!CB_DCHECK(l < 32u && s < T, kDbgBlockedFill, p)) continue;
           const uint32_t q = 64 * (s >> 1) + 2 * l + (s & 1);
-          const uint32_t el = (c & (kBCol - 1)) | (off << kBColBits);
+          const uint32_t el = kBElem(c, off);
           if (staged) stage[s_sb[b * W + wl] + q] = el; else belem[s_start[b * W + wl] + q] = el;
         }
         e += taken;

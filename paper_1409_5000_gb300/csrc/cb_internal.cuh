@@ -43,9 +43,17 @@ constexpr int kBTileRows = kBThreads * kBRowsPerThread;  // 16384
 constexpr uint32_t kBColBits = 14;
 constexpr uint32_t kBCol = 1u << kBColBits;              // 16384 floats = 64 KB per buffer
 constexpr uint32_t kBBuf = kBCol + 4;                    // floats per staging buffer (16-byte multiple)
+// A warp's row sums lie together, [slot][lane], and a stream element holds two
+// byte offsets: the column's in the staged block (low 16 bits) and its row
+// sum's in the warp's (high 16 bits), so the SpMV adds them to two bases.
+constexpr uint32_t kBWarpSums = (kBRowsPerThread + 1) * 32;
+__host__ __device__ constexpr uint32_t kBElem(uint32_t col, uint32_t off) {
+  return ((col & (kBCol - 1)) << 2) | (off << 18);
+}
+static_assert(kBColBits == 14 && kBWarpSums <= 1u << 14, "two 16-bit byte offsets");
 // A padding element of lane l adds into the lane's spare row sum (slot
 // kBRowsPerThread), which no row reads.
-__host__ __device__ constexpr uint32_t kBPadOff(uint32_t l) { return kBRowsPerThread * kBThreads + l; }
+constexpr uint32_t kBPadSlot = kBRowsPerThread;
 constexpr uint32_t kBMaxBlocks = 32;                     // blocked when n <= 32 * kBCol
 constexpr uint32_t kBLongDeg = 512;                      // longer rows: whole-CTA global gathers
 
@@ -216,7 +224,7 @@ struct cb_graph {
   uint64_t *d_bwscan = nullptr;          // scratch of the prefix that makes d_bwstart
   uint32_t *d_bwlen = nullptr;           // per (segment, warp): steps T of its stream (even)
   uint16_t *d_bcnt = nullptr;            // per (segment, lane): its elements (format build)
-  uint32_t *d_belem = nullptr;           // stream elements: local column | row-sum offset << kBColBits
+  uint32_t *d_belem = nullptr;           // stream elements (kBElem)
   uint32_t *d_blong_ptr = nullptr;       // per blocked tile: range in d_blong_rows
   uint32_t *d_blong_rows = nullptr;      // local rows with degree > kBLongDeg, in row order
   // two-phase format (FP32 SpMV), for realisations with pb = 1

@@ -323,9 +323,17 @@ __global__ void __launch_bounds__(kThreads) spmv_kernel(LArgs a, uint32_t j, uin
 // blocks of its tile, double-buffering each block of W_j into shared memory
 // with one bulk copy (cp.async.bulk, completion on an mbarrier) while the
 // previous block is consumed.  Thread i owns rows
-// i + kBThreads k (k = 0..15) of the tile and accumulates them in shared memory
-// (slot-major, so the accumulator traffic is conflict-free); every row has a
-// single writer, so the result is deterministic.
+// i + kBThreads k (k = 0..15) of the tile and accumulates them in shared memory;
+// every row has a single writer, so the result is deterministic.
+//
+// Bound by the shared-memory pipe: a step of 32 elements is about 4.1
+// wavefronts for the gathers (32 random banks), 1.6 to read and 1.6 to write
+// the sums, 0.85 for its share of the staged blocks.  175 M entries in 40
+// graphs: 325 us with a round's gathers after the previous sums, elements
+// decoded by shifts (29 instructions a step, 56% of the pipe); 293 with byte
+// offsets and the gathers of a round together (18); 277 with the loads two
+// rounds ahead; 263 with the prologue's and epilogue's loads together (17,
+// 74% of the pipe; the grid's last wave is the larger part of the rest).
 // ---------------------------------------------------------------------------
 
 // two column blocks of W_j, then kBRowsPerThread row sums per thread and
@@ -337,7 +345,7 @@ __global__ void __launch_bounds__(kBThreads, 1) bspmv_kernel(LArgs a, uint32_t j
                                                              uint32_t btile_off) {
   extern __shared__ float4 s_dyn4[];
   float *xs = reinterpret_cast<float *>(s_dyn4);  // two column blocks of W_j
-  float *sacc = xs + 2 * kBBuf;                   // [slot][thread] row sums
+  float *sacc = xs + 2 * kBBuf;                   // [warp][slot][lane] row sums
   __shared__ uint32_t s_long[kBTileRows / 32];    // bitmap of long rows
   __shared__ double s_red[32];
   __shared__ float s_rowsum[32];
@@ -346,159 +354,231 @@ __global__ void __launch_bounds__(kBThreads, 1) bspmv_kernel(LArgs a, uint32_t j
   __shared__ uint32_t s_issued[2];                // copies issued into buffer p
   __shared__ int s_abort;
   __shared__ uint64_t s_seg[kBMaxBlocks + 1];     // stream offset of each column block's segment
+  __shared__ float s_coef[2];                     // scale_j, beta_{j-1} scale_{j-1}
+  __shared__ __align__(8) uint64_t s_coef_ok;     // s_coef written
+  // One CTA per SM: nothing hides what a CTA does before its first and after
+  // its last element (13k and 18k of 149k cycles when each load waited for
+  // the one before), so the loads go out together, the static ones and the
+  // first rounds of the streams before the wait for the previous kernel, and
+  // the copies of W_j before it is known whether the realisation goes on.
   const uint32_t t = btile_off + blockIdx.x;
   const uint32_t r = a.btile_inst[t];
+  const uint64_t sbase = a.bseg_base[t];
+  const uint32_t lp0 = a.blong_ptr[t], lp1 = a.blong_ptr[t + 1];
+  const InstDesc &I = a.inst[r];
+  const uint32_t nb = I.nb, n = I.n, row0 = (t - I.btile_base) * kBTileRows;
+  const uint64_t node_base = I.node_base;
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // lane b holds the warp's stream of block b: its first element and its pairs
+  // of steps
+  static_assert(kBMaxBlocks <= 32, "one lane per column block");
+  uint64_t st = 0;
+  uint32_t np = 0;
+  if (lane < nb) {
+    st = a.bwstart[(sbase + lane) * 32 + warp];
+    np = a.bwlen[(sbase + lane) * 32 + warp] >> 1;
+  }
+  float *sw = sacc + warp * kBWarpSums;  // this warp's row sums: sw[32 * slot + lane]
+#pragma unroll
+  for (int k = 0; k <= kBRowsPerThread; ++k) sw[32 * k + lane] = 0.f;
+  for (uint32_t q = tid; q < kBTileRows / 32; q += kBThreads) s_long[q] = 0u;
+  if (tid == 0) {
+    mbar_init(&s_full[0], 1);
+    mbar_init(&s_full[1], 1);
+    mbar_init(&s_coef_ok, 1);
+    s_done[0] = s_done[1] = 0;
+    s_issued[0] = s_issued[1] = 0;
+    s_abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0 && lane < nb) s_seg[lane] = st;
+  if (warp == 31 && lane == nb - 1) s_seg[nb] = st + 64ull * np;
+
+  // A warp's stream of block b has T_b steps, read as T_b / 2 pairs (two
+  // elements per lane per 8-byte load) in rounds of up to 4 pairs that do not
+  // cross a block (an empty block is one empty round).  The loads run two
+  // rounds ahead of the sums, across the ends of blocks.
+  const uint32_t *fp = a.belem + __shfl_sync(0xffffffffu, st, 0) + 2 * lane;  // next round to load
+  uint32_t fb = 0, frem = __shfl_sync(0xffffffffu, np, 0);  // its block, the pairs left there
+  uint32_t b = 0, rem = frem;                               // the same of the round summed
+  auto fetch = [&](uint2 (&e)[4]) {
+    if (fb >= nb) return;
+    if (frem >= 4) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) e[u] = __ldcs(reinterpret_cast<const uint2 *>(fp + 64 * u));
+    } else {
+#pragma unroll
+      for (int u = 0; u < 3; ++u)
+        if ((uint32_t)u < frem) e[u] = __ldcs(reinterpret_cast<const uint2 *>(fp + 64 * u));
+    }
+    if (frem > 4) {
+      frem -= 4;
+      fp += 256;
+    } else if (++fb < nb) {
+      fp = a.belem + __shfl_sync(0xffffffffu, st, fb) + 2 * lane;
+      frem = __shfl_sync(0xffffffffu, np, fb);
+    }
+  };
+  uint2 eA[4], eB[4], eC[4];
+  fetch(eA);
+  fetch(eB);
+
   dep_wait();
   dep_trigger();
-  if (j >= a.sc.meff[r]) return;
-  const InstDesc &I = a.inst[r];
+  const uint32_t meff = a.sc.meff[r];
   const uint32_t ms = a.sc.ms;
   float *Vb = reinterpret_cast<float *>(a.V);
-  const float *x = Vb + (uint64_t)j * a.vs + I.node_base;
+  const float *x = Vb + (uint64_t)j * a.vs + node_base;
   const bool has_prev = j > 0;
-  const float *xp = has_prev ? Vb + (uint64_t)(j - 1) * a.vs + I.node_base : x;
-  float *out = Vb + (uint64_t)(j + 1) * a.vs + I.node_base;
-  const float sj = (float)a.sc.scale[r * ms + j];
-  const float bp = has_prev ? (float)(a.sc.beta[r * ms + j - 1] * a.sc.scale[r * ms + j - 1]) : 0.f;
-  const uint32_t row0 = (t - I.btile_base) * kBTileRows;
-  const uint32_t tid = threadIdx.x;
-
-  for (uint32_t q = tid; q < (kBRowsPerThread + 1) * kBThreads; q += kBThreads) sacc[q] = 0.f;
-  for (uint32_t q = tid; q < kBTileRows / 32; q += kBThreads) s_long[q] = 0u;
-  if (tid < 2) {
-    mbar_init(&s_full[tid], 1);
-    s_done[tid] = 0;
-    s_issued[tid] = 0;
-  }
-  if (tid == 0) s_abort = 0;
-  const uint32_t nb = I.nb;
-  const uint64_t sbase = a.bseg_base[t];
-  for (uint32_t q = tid; q <= nb; q += kBThreads) {
-    const uint64_t w = (sbase + (q < nb ? q : nb - 1)) * 32;
-    s_seg[q] = q < nb ? a.bwstart[w] : a.bwstart[w + 31] + 32ull * a.bwlen[w + 31];
-  }
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  __syncthreads();
-  const uint32_t lp0 = a.blong_ptr[t], lp1 = a.blong_ptr[t + 1];
-  for (uint32_t q = lp0 + tid; q < lp1; q += kBThreads) {
-    const uint32_t lr = a.blong_rows[q];
-    atomicOr(&s_long[lr >> 5], 1u << (lr & 31));
-  }
-
-  const uint32_t lane = tid & 31, warp = tid >> 5;
-  // Rounds: a warp's stream of block b has T_b steps, read as T_b / 2 pairs
-  // (two elements per lane per 8-byte load), 4 pairs per round.  The loads of
-  // the next round -- in the same block or, after the last round, round 0 of
-  // the next block -- are issued before the current round is processed, so
-  // the global-memory latency overlaps the shared-memory work and the wait.
-  uint64_t my = a.bwstart[sbase * 32 + warp] + 2 * lane;
-  uint32_t np = a.bwlen[sbase * 32 + warp] >> 1;
-  uint2 eA[4], eB[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-    if ((uint32_t)u < np) eA[u] = __ldcs(reinterpret_cast<const uint2 *>(a.belem + my + 64ull * u));
-  float *sw = sacc + 32 * warp;  // this warp's row sums: sw[k * kBThreads + lane]
+  const float *xp = has_prev ? Vb + (uint64_t)(j - 1) * a.vs + node_base : x;
+  float *out = Vb + (uint64_t)(j + 1) * a.vs + node_base;
   // Column block b of W_j goes to buffer b & 1 by one bulk copy that
   // completes on s_full[b & 1].  No CTA-wide barrier per block: each warp
   // waits only for the block it needs, and the last warp to finish with a
   // buffer issues the copy of block b + 2 into it, so warps drift apart by up
-  // to a block instead of all waiting for the slowest at every block.
-  const uint32_t n_cols = I.n;
-  auto block_bytes = [&](uint32_t b) -> uint32_t {
-    const uint32_t len = min(kBCol, n_cols - b * kBCol);
-    return ((len + 3u) & ~3u) * 4u;  // whole 16-byte units (reads up to 3 floats of padding)
+  // to a block instead of all waiting for the slowest at every block.  After
+  // the last block the tile's rows of W_{j-1} follow as block nb, for the
+  // epilogue.  The edge streams of block b + 1 are prefetched into L2 when
+  // block b is staged, so the warps' stream loads find them there.
+  auto issue = [&](uint32_t b) {
+    if (b > nb || (b == nb && !has_prev)) return;
+    const float *src = b < nb ? x + (uint64_t)b * kBCol : xp + row0;
+    const uint32_t len = b < nb ? min(kBCol, n - b * kBCol) : min((uint32_t)kBTileRows, n - row0);
+    const uint32_t bytes = ((len + 3u) & ~3u) * 4u;  // whole 16-byte units (reads up to 3 floats of padding)
+    const uint32_t p = b & 1;
+    mbar_expect_tx(&s_full[p], bytes);
+    if (b == 0 && t == a.stall_btile) return;  // test hook: block 0 never arrives
+    bulk_g2s(xs + p * kBBuf, src, bytes, &s_full[p]);
+    s_issued[p] += 1;
   };
-  // The edge streams of column block b + 3 are prefetched into L2 when block
-  // b + 2 is staged, so the warps' stream loads find them there.
   auto prefetch_seg = [&](uint32_t b) {
-    const uint64_t e0 = s_seg[b], e1 = s_seg[b + 1];
-    if (e1 > e0) l2_prefetch(a.belem + e0, (uint32_t)(4 * (e1 - e0)));
+    if (b < nb && s_seg[b + 1] > s_seg[b])
+      l2_prefetch(a.belem + s_seg[b], (uint32_t)(4 * (s_seg[b + 1] - s_seg[b])));
+  };
+  // every copy issued into a buffer has landed before the CTA ends (bounded)
+  auto drain = [&]() {
+    for (int p = 0; p < 2; ++p)
+      if (s_issued[p]) mbar_wait(&s_full[p], (s_issued[p] - 1) & 1u);
   };
   if (tid == 0) {
-    for (uint32_t b = 1; b < 3 && b < nb; ++b) prefetch_seg(b);
-    for (uint32_t b = 0; b < 2 && b < nb; ++b) {
-      mbar_expect_tx(&s_full[b], block_bytes(b));
-      if (b == 0 && t == a.stall_btile) continue;  // test hook: block 0 never arrives
-      bulk_g2s(xs + b * kBBuf, x + (uint64_t)b * kBCol, block_bytes(b), &s_full[b]);
-      s_issued[b] = 1;
-    }
+    issue(0);
+    issue(1);
   }
+  __syncthreads();
+  if (j >= meff) {
+    if (tid == 0) drain();
+    return;
+  }
+  if (tid == 0) {
+    prefetch_seg(1);
+    prefetch_seg(2);
+  }
+  if (tid == kBThreads - 1) {  // one thread: an FP64 instruction holds its sub-core for 65 cycles
+    s_coef[0] = (float)a.sc.scale[r * ms + j];
+    s_coef[1] = has_prev ? (float)(a.sc.beta[r * ms + j - 1] * a.sc.scale[r * ms + j - 1]) : 0.f;
+    mbar_arrive(&s_coef_ok);
+  }
+  if (lp1 > lp0) {
+    for (uint32_t q = lp0 + tid; q < lp1; q += kBThreads) {
+      const uint32_t lr = a.blong_rows[q];
+      atomicOr(&s_long[lr >> 5], 1u << (lr & 31));
+    }
+    __syncthreads();
+  }
+
+  const char *cur = reinterpret_cast<const char *>(xs);
+  char *swc = reinterpret_cast<char *>(sw);
+  auto gather = [&](uint32_t v) -> float {
+    if (!CB_DCHECK((v >> 18) < kBWarpSums && (v & 3u) == 0, kDbgBlockedElem, v)) return 0.f;
+    return *reinterpret_cast<const float *>(cur + (v & 0xffffu));
+  };
+  auto add = [&](uint32_t v, float g) {
+    if (!CB_DCHECK((v >> 18) < kBWarpSums, kDbgBlockedElem, v)) return;
+    *reinterpret_cast<float *>(swc + (v >> 16)) += g;
+  };
+  // One round: the gathers of all its elements, then the sums, in step order
+  // (no two lanes of a step add into one row sum).  False once the tile's
+  // streams are done or a copy never landed.
   bool aborted = false;
-  for (uint32_t b = 0; b < nb; ++b) {
-    uint64_t my1 = 0;
-    uint32_t np1 = 0;
-    if (b + 1 < nb) {
-      const uint64_t nseg = sbase + b + 1;
-      my1 = a.bwstart[nseg * 32 + warp] + 2 * lane;
-      np1 = a.bwlen[nseg * 32 + warp] >> 1;
-    }
-    if (!mbar_wait(&s_full[b & 1], (b >> 1) & 1u)) {
-      aborted = true;  // the copy never landed: give up on this tile
-      break;
-    }
-    const float *cur = xs + (b & 1) * kBBuf;
-    const uint32_t nr = (np + 3) >> 2;
-    const uint32_t iters = nr ? nr : 1u;  // one pass even when empty: prefetch the next block
-    for (uint32_t r = 0; r < iters; ++r) {
-      // next round's loads
-      if (r + 1 < nr) {
+  auto round = [&](const uint2 (&e)[4]) -> bool {
+    if (rem >= 4) {
+      float g[8];
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (4 * (r + 1) + u < np)
-            eB[u] = __ldcs(reinterpret_cast<const uint2 *>(a.belem + my + 64ull * (4 * (r + 1) + u)));
-      } else if (b + 1 < nb) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if ((uint32_t)u < np1) eB[u] = __ldcs(reinterpret_cast<const uint2 *>(a.belem + my1 + 64ull * u));
-      }
-      // this round: no two lanes of a step add into one row sum
-      if (r < nr) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (4 * r + u < np) {
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const uint32_t v = e ? eA[u].y : eA[u].x;
-              const uint32_t col = v & (kBCol - 1), off = v >> kBColBits;
-              if (CB_DCHECK((off & (kBThreads - 1)) < 32u && off <= kBPadOff(31), kDbgBlockedElem, v))
-                sw[off] += cur[col];
-            }
-          }
+      for (int u = 0; u < 4; ++u) {
+        g[2 * u] = gather(e[u].x);
+        g[2 * u + 1] = gather(e[u].y);
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) eA[u] = eB[u];
+      for (int u = 0; u < 4; ++u) {
+        add(e[u].x, g[2 * u]);
+        add(e[u].y, g[2 * u + 1]);
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < 3; ++u)
+        if ((uint32_t)u < rem) {
+          const float g0 = gather(e[u].x), g1 = gather(e[u].y);
+          add(e[u].x, g0);
+          add(e[u].y, g1);
+        }
     }
-    my = my1;
-    np = np1;
-    // this warp is done with buffer b & 1; the last warp refills it with block b + 2
+    if (rem > 4) {
+      rem -= 4;
+      return true;
+    }
+    // this warp is done with buffer b & 1; the last warp refills it
     __syncwarp();
     if (lane == 0) {
       __threadfence_block();
-      const uint32_t p = b & 1;
-      if (atomicAdd(&s_done[p], 1u) == kBThreads / 32 - 1) {
-        s_done[p] = 0;
-        if (b + 2 < nb) {
-          __threadfence_block();
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          mbar_expect_tx(&s_full[p], block_bytes(b + 2));
-          bulk_g2s(xs + p * kBBuf, x + (uint64_t)(b + 2) * kBCol, block_bytes(b + 2), &s_full[p]);
-          s_issued[p] += 1;
-          if (b + 3 < nb) prefetch_seg(b + 3);
-        }
+      if (atomicAdd(&s_done[b & 1], 1u) == kBThreads / 32 - 1) {
+        s_done[b & 1] = 0;
+        __threadfence_block();
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        issue(b + 2);
+        prefetch_seg(b + 3);
       }
     }
-  }
-  if (aborted) s_abort = 1;
-  __syncthreads();  // s_long and s_abort complete; sacc rows are per thread
+    if (++b == nb) return false;
+    rem = __shfl_sync(0xffffffffu, np, b);
+    cur = reinterpret_cast<const char *>(xs + (b & 1) * kBBuf);
+    aborted = !mbar_wait_sleep(&s_full[b & 1], (b >> 1) & 1u);  // the copy never landed: give up
+    return !aborted;
+  };
+  aborted = !mbar_wait_sleep(&s_full[0], 0);
+  if (!aborted)
+    while (true) {
+      fetch(eC);
+      if (!round(eA)) break;
+      fetch(eA);
+      if (!round(eB)) break;
+      fetch(eB);
+      if (!round(eC)) break;
+    }
 
-  float acc = 0.f;
-#pragma unroll 4
+  // the warp's rows: their sums are complete, nobody else adds into them.
+  // Row slot k of this thread is row tid + kBThreads k of the tile.
+  float xr[kBRowsPerThread];
+#pragma unroll
   for (int k = 0; k < kBRowsPerThread; ++k) {
-    const uint32_t lr = tid + kBThreads * k;  // row slot k of this thread
-    const uint32_t row = row0 + lr;
-    if (row < I.n && !((s_long[lr >> 5] >> (lr & 31)) & 1u))
-      acc += row_epilogue<float>(sacc[k * kBThreads + tid], row, x, xp, out, sj, bp, has_prev);
+    const uint32_t row = row0 + tid + kBThreads * k;
+    xr[k] = row < n ? x[row] : 0.f;
   }
+  if (has_prev && !aborted) aborted = !mbar_wait_sleep(&s_full[nb & 1], (nb >> 1) & 1u);
+  if (!mbar_wait_sleep(&s_coef_ok, 0)) aborted = true;
+  const float sj = s_coef[0], bp = s_coef[1];
+  const float *xpt = xs + (nb & 1) * kBBuf;  // W_{j-1} of the tile
+  float acc = 0.f;
+#pragma unroll
+  for (int k = 0; k < kBRowsPerThread; ++k) {
+    const uint32_t lr = tid + kBThreads * k, row = row0 + lr;
+    if (row < n && !((s_long[lr >> 5] >> (lr & 31)) & 1u)) {
+      float u = sj * sw[32 * k + lane];
+      if (has_prev) u -= bp * xpt[lr];
+      out[row] = u;
+      acc += u * xr[k];
+    }
+  }
+  if (aborted) s_abort = 1;  // read after the sum's barrier
   // long rows: whole CTA per row from the CSR, in row order
   const uint32_t *rp = a.row_ptr + I.rp_base;
   const uint32_t *col = a.col + I.edge_base;
@@ -520,15 +600,17 @@ __global__ void __launch_bounds__(kBThreads, 1) bspmv_kernel(LArgs a, uint32_t j
     }
     __syncthreads();
   }
-  double part = block_sum_to_double<float>(acc, s_red);
+  acc = warp_sum<float>(acc);
+  if (lane == 0) s_red[warp] = (double)acc;
+  __syncthreads();
+  double part = 0.0;
+  if (warp == 0) part = warp_sum_d(s_red[lane]);
   if (tid == 0) {
     if (s_abort) {  // a block never arrived: this step of the realisation fails
       a.sc.status[r] = CB_ERR_TIMEOUT;
       part = __longlong_as_double(0x7ff8000000000000ll);
     }
-    // every copy issued into a buffer has landed before the CTA ends (bounded)
-    for (int p = 0; p < 2; ++p)
-      if (s_issued[p]) mbar_wait(&s_full[p], (s_issued[p] - 1) & 1u);
+    drain();
   }
   double total;
   if (arrive_and_reduce(I.bspmv, t - I.btile_base, r, part, a.red, &total))

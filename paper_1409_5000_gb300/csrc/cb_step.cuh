@@ -233,6 +233,10 @@ __device__ __forceinline__ bool mbar_wait_sleep(uint64_t *bar, uint32_t parity) 
   }
   return false;
 }
+// One arrival; what the thread wrote before is seen by whoever waits for the phase.
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+  asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}" ::"r"(smem_u32(bar)) : "memory");
+}
 // One bulk copy global -> shared whose bytes complete on `bar` (16-byte
 // aligned addresses, size a multiple of 16).
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {

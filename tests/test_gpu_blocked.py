@@ -34,3 +34,24 @@ def test_stream_lengths_match_oracle(n, deg):
     with B.GraphSet(graphs, path=B.CB_PATH_FORMATS) as gs:
         ls, S = B.ensemble_scores(gs, 15, B.CB_FP32)
         parity.assert_scores(float(ls.item()), S.cpu().numpy(), th_o, S_o, "fp32")
+
+
+@pytest.mark.parametrize("d", [9, 30, 31, 250, 511])
+def test_rows_as_long_as_their_stream(d):
+    """Rows that fill a stream's steps, so that a run goes on from one lane's
+    last step to the next lane's first: no step may add twice into one sum.
+    Hubs of d entries beside rows of a few, FP32 parity bars against the oracle."""
+    from paper_1409_5000_gb300 import binding as B
+
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for -m gpu tests")
+    n = 3000
+    rng = np.random.default_rng(d)
+    e = [rng.integers(0, n, (n // 2, 2))]
+    e += [np.stack([np.full(d, h), rng.choice(np.arange(200, n), d, replace=False)], axis=1) for h in (3, 4, 40, 41, 77)]
+    e = np.concatenate(e)
+    graphs = [synth.from_edges(n, e[e[:, 0] != e[:, 1]]), synth.er(500, 0.02, d)]
+    th_o, S_o = oc.ensemble_scores([(q.n, q.row_ptr, q.col) for q in graphs], 15)
+    with B.GraphSet(graphs, path=B.CB_PATH_FORMATS) as gs:
+        ls, S = B.ensemble_scores(gs, 15, B.CB_FP32)
+        parity.assert_scores(float(ls.item()), S.cpu().numpy(), th_o, S_o, "fp32")

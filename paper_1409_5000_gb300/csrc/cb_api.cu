@@ -15,7 +15,11 @@
 #include <cstdlib>
 #include <cstring>
 #include <atomic>
+#include <chrono>
+#include <condition_variable>
+#include <exception>
 #include <mutex>
+#include <system_error>
 #include <thread>
 #include <unordered_map>
 
@@ -90,19 +94,87 @@ static void prof_clear() {
   g_prof.clear();
 }
 
-void parallel_for(uint32_t n, const std::function<void(uint32_t)> &fn) {
-  unsigned hw = std::thread::hardware_concurrency();
-  const uint32_t nt = std::min<uint32_t>(n, hw ? std::min(hw, 32u) : 1u);
-  if (nt <= 1) {
-    for (uint32_t i = 0; i < n; ++i) fn(i);
-    return;
+// Helper threads of parallel_for.  Starting 16 threads for each of the three
+// scans of an upload took 0.9 ms a time on a 40-graph ensemble whose scans
+// take 0.1, most of the 3.2 ms of generating it; they are kept for a while
+// instead, and leave after kIdle without work.  One call at a time uses them: a
+// second one, from another thread, runs on its own thread alone.  The caller
+// takes items as the helpers do and waits only for helpers that hold one, so
+// it ends without any (after a fork, or when none could be started).  The
+// object is never destroyed: helpers may outlive static destructors.
+class HelperPool {
+ public:
+  void run(uint32_t n, uint32_t helpers, const std::function<void(uint32_t)> &fn) {
+    std::unique_lock<std::mutex> lk(mu_);
+    if (fn_ || helpers == 0) {
+      lk.unlock();
+      for (uint32_t i = 0; i < n; ++i) fn(i);
+      return;
+    }
+    fn_ = &fn;
+    n_ = n;
+    next_ = 0;
+    error_ = nullptr;
+    join_ = helpers;
+    for (uint32_t have = idle_; have < helpers; ++have) {
+      try {
+        std::thread([this] { help(); }).detach();
+      } catch (const std::system_error &) {
+        break;
+      }
+    }
+    lk.unlock();
+    work_.notify_all();
+    take();
+    lk.lock();
+    join_ = 0;  // nobody joins any more; whoever did finishes the item it holds
+    done_.wait(lk, [this] { return busy_ == 0; });
+    fn_ = nullptr;
+    const std::exception_ptr error = error_;
+    lk.unlock();
+    if (error) std::rethrow_exception(error);
   }
-  std::vector<std::thread> th;
-  for (uint32_t t = 0; t < nt; ++t)
-    th.emplace_back([&, t] {
-      for (uint32_t i = t; i < n; i += nt) fn(i);
-    });
-  for (auto &x : th) x.join();
+
+ private:
+  static constexpr std::chrono::seconds kIdle{2};
+  void take() {
+    for (uint32_t i; (i = next_.fetch_add(1)) < n_;) {
+      try {
+        (*fn_)(i);
+      } catch (...) {
+        std::lock_guard<std::mutex> lk(emu_);
+        if (!error_) error_ = std::current_exception();
+      }
+    }
+  }
+  void help() {
+    std::unique_lock<std::mutex> lk(mu_);
+    while (true) {
+      ++idle_;
+      const bool work = work_.wait_for(lk, kIdle, [this] { return join_ > 0; });
+      --idle_;
+      if (!work) return;
+      --join_;
+      ++busy_;
+      lk.unlock();
+      take();
+      lk.lock();
+      if (--busy_ == 0) done_.notify_one();
+    }
+  }
+  std::mutex mu_, emu_;
+  std::condition_variable work_, done_;
+  const std::function<void(uint32_t)> *fn_ = nullptr;
+  uint32_t n_ = 0, join_ = 0, busy_ = 0, idle_ = 0;
+  std::atomic<uint32_t> next_{0};
+  std::exception_ptr error_;
+};
+
+void parallel_for(uint32_t n, uint64_t work, const std::function<void(uint32_t)> &fn) {
+  static HelperPool *pool = new HelperPool;
+  const uint32_t hw = std::min(std::max(std::thread::hardware_concurrency(), 1u), 32u);
+  const uint64_t threads = std::min<uint64_t>(std::min(n, hw), 1 + work / kWorkPerHelper);
+  pool->run(n, threads ? (uint32_t)threads - 1 : 0u, fn);
 }
 
 void prefer_shared_impl(const void *kernel) {
@@ -704,12 +776,12 @@ static int upload_impl(uint32_t n_inst, const uint32_t *n, const uint64_t *nnz,
     delete h;
     return cuda_error(e, "cb_graph_upload: allocate / copy");
   }
-  // The column-blocked format needs only the sizes and the device arrays:
-  // its count and fill passes are queued first, and the host's scans of
-  // row_ptr below run while the device builds it.
+  // The column-blocked format needs only the sizes and the device arrays: its
+  // count passes are queued behind the copies, and the host's scans of row_ptr
+  // below run meanwhile; the fill pass, whose size the host waits for, follows
+  // them (40 graphs, 175 M entries: 3.5 ms of copies, 1 of scans).
   BlockedBuild bb;
   int rc = blocked_count(h, s, cp.groups, bb);
-  if (rc == CB_OK) rc = blocked_fill(h, s, bb);
   if (rc != CB_OK) {
     cp.finish();
     free_blocked(h);
@@ -724,7 +796,7 @@ static int upload_impl(uint32_t n_inst, const uint32_t *n, const uint64_t *nnz,
   // their chunks run in CTAs of their own), so hub-heavy regions of a graph
   // get short tiles and no CTA becomes a straggler.
   std::vector<std::vector<uint32_t>> heavy_rows(n_inst), tile_starts(n_inst);
-  parallel_for(n_inst, [&](uint32_t r) {
+  parallel_for(n_inst, node_off, [&](uint32_t r) {
     const uint32_t *rp = rp_of(r);
     uint32_t rows = 0, acc = 0;
     for (uint32_t i = 0; i < h->inst[r].n; ++i) {
@@ -838,6 +910,7 @@ static int upload_impl(uint32_t n_inst, const uint32_t *n, const uint64_t *nnz,
   std::vector<const uint32_t *> rpv(n_inst);
   for (uint32_t r = 0; r < n_inst; ++r) rpv[r] = rp_of(r);
   rc = blocked_long_rows(h, rpv, s);
+  if (rc == CB_OK) rc = blocked_fill(h, s, bb);
   if (rc == CB_OK) rc = build_twophase(h, rpv, s, cp.groups, h->force_pb);
   if (rc == CB_OK) {  // every copy has landed before the handle is returned
     for (const CopyGroup &g : cp.groups) chk(cudaStreamWaitEvent(s, g.ev, 0));

@@ -564,7 +564,7 @@ int blocked_long_rows(cb_graph *h, const std::vector<const uint32_t *> &rp_host,
   if (h->csr_only || !h->total_btiles) return CB_OK;
   // long rows per tile (tile-local indices), scanned in parallel over realisations
   std::vector<std::vector<uint32_t>> lrows(h->n_inst), lcount(h->n_inst);
-  parallel_for(h->n_inst, [&](uint32_t r) {
+  parallel_for(h->n_inst, h->total_nodes_padded, [&](uint32_t r) {
     const InstDesc &I = h->inst[r];
     const uint32_t *rp = rp_host[r];
     for (uint32_t q = 0; q < I.n_btiles; ++q) {

@@ -340,8 +340,11 @@ int dbg_read_adjoint(uint32_t *count, uint64_t *first, bool reset);
 int dbg_read_team(uint32_t *count, uint64_t *first, bool reset);
 int dbg_read_subgraph(uint32_t *count, uint64_t *first, bool reset);
 
-// fn(i) for i in [0, n) on the host, spread over the hardware threads
-void parallel_for(uint32_t n, const std::function<void(uint32_t)> &fn);
+// fn(i) for i in [0, n) on the host, spread over the hardware threads, one
+// more for each kWorkPerHelper of the total work (rows scanned, about 1 ns
+// each; waking a helper takes some tens of us)
+constexpr uint64_t kWorkPerHelper = 1u << 16;
+void parallel_for(uint32_t n, uint64_t work, const std::function<void(uint32_t)> &fn);
 
 // Host-to-device copy of a small host table during an upload, staged through
 // a library-owned pinned buffer so that it is truly asynchronous: a copy from

@@ -872,7 +872,10 @@ int build_twophase(cb_graph *h, const std::vector<const uint32_t *> &rp_host, cu
     const bool fits = I.n <= kPSrc * kPMaxSrc && (kPGroup - 1) * S + kHeavyDeg <= kPRegion;
     want[r] = (force || big) && fits && !I.blocked ? 1 : 0;
   }
-  parallel_for(N, [&](uint32_t r) {
+  uint64_t rows = 0;
+  for (uint32_t r = 0; r < N; ++r) rows += want[r] ? h->inst[r].n : 0u;
+  if (!rows) return CB_OK;
+  parallel_for(N, rows, [&](uint32_t r) {
     if (!want[r]) return;
     const InstDesc &I = h->inst[r];
     const uint32_t *rp = rp_host[r];

@@ -12,7 +12,9 @@
 // CB_FP64 mode); the sum over realisations r always runs in FP64 and in
 // realisation order, so it is deterministic.  Reads of W are coalesced
 // (consecutive nodes are consecutive addresses in every basis vector).
-#include "cb_internal.cuh"
+#include <algorithm>
+
+#include "cb_reduce.cuh"
 
 namespace cb {
 
@@ -84,7 +86,12 @@ __global__ void __launch_bounds__(256) combine_y_kernel(const T *V, uint64_t vs,
 }
 
 // S(i) = sum_r [i < n_r] exp(theta_r - theta*) y_r(i), in realisation order,
-// FP64; y_r was written into basis slot `yslot` by combine_y_kernel.
+// FP64; y_r was written into basis slot `yslot` by combine_y_kernel.  A grid of
+// the CTAs that fit walks the nodes: the weights (FP64 exponentials) cost a CTA
+// 3 us, which one CTA per 256 nodes spent 39 000 times on 1e7 nodes of one
+// realisation (434 us, 52 now).  With many realisations bound by the FP64 pipe, one
+// operation per term with the conversion done on the bits (256 realisations,
+// 5.4e7 terms: 342 us, 142 now).
 template <typename T>
 __global__ void __launch_bounds__(256) combine_sum_kernel(const T *Y, Scalars sc,
                                                           const InstDesc *inst, uint32_t n_inst,
@@ -116,29 +123,42 @@ __global__ void __launch_bounds__(256) combine_sum_kernel(const T *Y, Scalars sc
   for (int w = 1; w < (int)(blockDim.x >> 5); ++w) { tmax = fmax(tmax, s_max[w]); any_bad |= s_badw[w]; }
   for (uint32_t r = threadIdx.x; r < n_inst; r += blockDim.x) s_wt[r] = exp(sc.theta[r] - tmax);
   __syncthreads();
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   const double qnan = __longlong_as_double(0x7ff8000000000000ll);
-  if (i == 0) *log_scale = any_bad ? qnan : tmax;
-  if (i >= n_out) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *log_scale = any_bad ? qnan : tmax;
   // 8 realisations' loads in flight, then their terms in realisation order;
   // realisations with n_r <= i are skipped (warp-uniform except at n_r), so
   // the scarce FP64 pipe only sees real terms
   constexpr uint32_t kB = 8;
-  double sum = 0.0;
-  for (uint32_t r0 = 0; r0 < n_inst; r0 += kB) {
-    T y[kB];
-    bool in[kB];
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_out;
+       i += (uint64_t)gridDim.x * blockDim.x) {
+    double sum = 0.0;
+    for (uint32_t r0 = 0; r0 < n_inst; r0 += kB) {
+      T y[kB];
+      bool in[kB];
 #pragma unroll
-    for (uint32_t u = 0; u < kB; ++u) {
-      const uint32_t r = r0 + u;
-      in[u] = r < n_inst && i < s_n[r];
-      y[u] = in[u] ? Y[s_base[r] + i] : T(0);
+      for (uint32_t u = 0; u < kB; ++u) {
+        const uint32_t r = r0 + u;
+        in[u] = r < n_inst && i < s_n[r];
+        y[u] = in[u] ? Y[s_base[r] + i] : T(0);
+      }
+#pragma unroll
+      for (uint32_t u = 0; u < kB; ++u)
+        if (in[u]) sum += s_wt[r0 + u] * to_double(y[u]);
     }
-#pragma unroll
-    for (uint32_t u = 0; u < kB; ++u)
-      if (in[u]) sum += s_wt[r0 + u] * (double)y[u];
+    S[i] = any_bad ? qnan : sum;
   }
-  S[i] = any_bad ? qnan : sum;
+}
+
+template <typename T>
+static void launch_sum(cb_graph *h, const T *Y, uint32_t n_out, double *S, double *log_scale, size_t shm,
+                       cudaStream_t s) {
+  auto k = combine_sum_kernel<T>;
+  prefer_shared(k);
+  if (shm > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+  // as many CTAs as the shared memory lets an SM hold, at most 8
+  const uint32_t per_sm = std::max<uint32_t>(1, std::min<uint32_t>(8, (uint32_t)(200 * 1024 / (shm + 1024))));
+  const uint32_t grid = std::max(1u, std::min((n_out + 255) / 256, h->n_sm * per_sm));
+  k<<<grid, 256, shm, s>>>(Y, h->ws.sc, h->d_inst, h->n_inst, n_out, S, log_scale);
 }
 
 int combine_single(cb_graph *h, uint32_t r, int prec, double *y, double *log_scale,
@@ -168,11 +188,8 @@ int combine_ensemble(cb_graph *h, int prec, uint32_t n_out, double *S, double *l
   NvtxRange nvtx_range("ensemble combine");
   const size_t shm = (sizeof(double) + sizeof(uint64_t) + sizeof(uint32_t)) * h->n_inst;
   if (shm > 200 * 1024) return set_error(CB_ERR_ARG, "too many realisations for one combine");
-  const uint32_t grid = (n_out + 255) / 256;
   prefer_shared(combine_y_kernel<double, double>);
   prefer_shared(combine_y_kernel<float, float>);
-  prefer_shared(combine_sum_kernel<double>);
-  prefer_shared(combine_sum_kernel<float>);
   const int tok = prof_begin(CB_K_COMBINE, s);
   // per-realisation terms go into the last basis slot, which the combine never reads
   const uint64_t yoff = (uint64_t)h->ws.m * h->ws.vec_stride;
@@ -180,16 +197,12 @@ int combine_ensemble(cb_graph *h, int prec, uint32_t n_out, double *S, double *l
     double *Y = (double *)h->ws.V + yoff;
     combine_y_kernel<double, double><<<h->total_fin, 256, 0, s>>>(
         (const double *)h->ws.V, h->ws.vec_stride, h->ws.sc, h->d_inst, h->d_fin_inst, 0, Y, true);
-    auto k = combine_sum_kernel<double>;
-    if (shm > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-    k<<<grid, 256, shm, s>>>(Y, h->ws.sc, h->d_inst, h->n_inst, n_out, S, log_scale);
+    launch_sum<double>(h, Y, n_out, S, log_scale, shm, s);
   } else {
     float *Y = (float *)h->ws.V + yoff;
     combine_y_kernel<float, float><<<h->total_fin, 256, 0, s>>>(
         (const float *)h->ws.V, h->ws.vec_stride, h->ws.sc, h->d_inst, h->d_fin_inst, 0, Y, true);
-    auto k = combine_sum_kernel<float>;
-    if (shm > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-    k<<<grid, 256, shm, s>>>(Y, h->ws.sc, h->d_inst, h->n_inst, n_out, S, log_scale);
+    launch_sum<float>(h, Y, n_out, S, log_scale, shm, s);
   }
   prof_end(tok, s);
   return cuda_error(cudaGetLastError(), "combine launch");
@@ -199,11 +212,8 @@ int combine_sum_f64(cb_graph *h, const double *Y, uint32_t n_out, double *S, dou
                     cudaStream_t s) {
   const size_t shm = (sizeof(double) + sizeof(uint64_t) + sizeof(uint32_t)) * h->n_inst;
   if (shm > 200 * 1024) return set_error(CB_ERR_ARG, "too many realisations for one combine");
-  auto k = combine_sum_kernel<double>;
-  prefer_shared(k);
-  if (shm > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
   const int tok = prof_begin(CB_K_COMBINE, s);
-  k<<<(n_out + 255) / 256, 256, shm, s>>>(Y, h->ws.sc, h->d_inst, h->n_inst, n_out, S, log_scale);
+  launch_sum<double>(h, Y, n_out, S, log_scale, shm, s);
   prof_end(tok, s);
   return cuda_error(cudaGetLastError(), "combine launch");
 }

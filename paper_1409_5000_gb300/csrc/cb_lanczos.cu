@@ -45,16 +45,17 @@ namespace cb {
 
 
 template <typename T>
-__global__ void __launch_bounds__(kThreads) init_vec_kernel(LArgs a, uint32_t r0, uint32_t r1,
-                                                            T fill) {
-  // W_0 = fill (1 for the start vector 1, 0 before an indicator is set).
-  for (uint32_t r = r0; r < r1; ++r) {
-    const InstDesc I = a.inst[r];
-    T *w0 = reinterpret_cast<T *>(a.V) + I.node_base;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < I.n;
-         i += (uint64_t)gridDim.x * blockDim.x)
-      w0[i] = fill;
-  }
+__global__ void __launch_bounds__(kThreads) init_vec_kernel(T *w0, uint64_t n8, T fill) {
+  // W_0 = fill (1 for the start vector 1, 0 before an indicator is set), 8
+  // nodes at a time over the realisations' range, the alignment gaps between
+  // them (which nothing reads) included: a loop over the realisations, its
+  // grid sized for one, took 155 us for 256 of them, 58 now.
+  T v[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) v[q] = fill;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n8;
+       i += (uint64_t)gridDim.x * blockDim.x)
+    Vec8<T>::store(w0 + 8 * i, v);
 }
 
 // W_0[idx[q]] = 1 for the start indices inside each realisation's range
@@ -678,11 +679,32 @@ __global__ void __launch_bounds__(kThreads) finalize_beta_kernel(LArgs a, uint32
   dep_trigger();
   if (j >= a.sc.meff[r]) return;
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (uint32_t g = warp; g < P.n_groups; g += kThreads / 32) {
-    const uint32_t gsize = min((uint32_t)kGroup, P.n_slots - g * kGroup);
-    double v = lane < gsize ? a.red.part[P.slot_base + g * kGroup + lane] : 0.0;
-    v = warp_sum_d(v);
-    if (lane == 0) a.red.gpart[P.group_base + g] = v;
+  // Many groups: one lane per group, its 32 slots added in the order of the
+  // warp sum's tree.  A warp then issues 31 FP64 additions for 32 groups, not
+  // 5 for each (an addition holds its sub-core for 65 cycles however many lanes
+  // are active): 4883 partials (1e7 nodes) 20.3 -> 8.4 us; from about 24 groups
+  // on it is the shorter chain.
+  static_assert(kGroup == 32, "one lane per slot of a group");
+  if (P.n_groups >= 24) {
+    for (uint32_t g = threadIdx.x; g < P.n_groups; g += kThreads) {
+      const uint32_t gsize = min((uint32_t)kGroup, P.n_slots - g * kGroup);
+      const double *p = a.red.part + P.slot_base + g * kGroup;
+      double v[32];
+#pragma unroll
+      for (uint32_t q = 0; q < 32; ++q) v[q] = q < gsize ? p[q] : 0.0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < o; ++q) v[q] += v[q + o];
+      a.red.gpart[P.group_base + g] = v[0];
+    }
+  } else {
+    for (uint32_t g = warp; g < P.n_groups; g += kThreads / 32) {
+      const uint32_t gsize = min((uint32_t)kGroup, P.n_slots - g * kGroup);
+      double v = lane < gsize ? a.red.part[P.slot_base + g * kGroup + lane] : 0.0;
+      v = warp_sum_d(v);
+      if (lane == 0) a.red.gpart[P.group_base + g] = v;
+    }
   }
   __syncthreads();
   double acc = 0.0;
@@ -1066,15 +1088,17 @@ static int run_t(cb_graph *h, Workspace &W, uint32_t r0, uint32_t r1, uint32_t m
 
   uint32_t nmax = 0;
   for (uint32_t r = r0; r < r1; ++r) nmax = h->inst[r].n > nmax ? h->inst[r].n : nmax;
-  const uint32_t init_grid = (nmax + kThreads * 8 - 1) / (kThreads * 8);
+  const uint64_t init_n8 = (A1.node_base + A1.n - A0.node_base + 7) / 8;
+  static_assert(kNodeAlign % 8 == 0, "a realisation's last 8 nodes lie in its own range");
+  const uint32_t init_grid = (uint32_t)std::min<uint64_t>((init_n8 + kThreads - 1) / kThreads, 8 * h->n_sm);
   prefer_shared(init_vec_kernel<T>);
   prefer_shared(init_indicator_kernel<T>);
   prefer_shared(init_scalars_kernel);
   prefer_shared(finalize_kernel<T>);
   int tok = prof_begin(CB_K_INIT, s);
   if (!rscale)
-    init_vec_kernel<T><<<init_grid ? init_grid : 1, kThreads, 0, s>>>(a, r0, r1,
-                                                                      start_idx ? T(0) : T(1));
+    init_vec_kernel<T><<<init_grid ? init_grid : 1, kThreads, 0, s>>>(
+        reinterpret_cast<T *>(a.V) + A0.node_base, init_n8, start_idx ? T(0) : T(1));
   if (start_idx && !rscale)
     init_indicator_kernel<T><<<r1 - r0, kThreads, 0, s>>>(a, r0, start_idx, k, per_inst);
   // on-chip problems on the automatic path: the whole recurrence in one launch

@@ -41,6 +41,18 @@ __device__ __forceinline__ T group_sum(T v) {
   return v;
 }
 
+// (double)x by moving its bits: the conversion instruction holds a sub-core's
+// FP64 pipe for 65 cycles per warp, as an addition does.  Zeros and normal
+// numbers; the rest (no exponent, infinities, NaN) by the instruction.
+__device__ __forceinline__ double to_double(float x) {
+  const uint32_t b = __float_as_uint(x), mag = b & 0x7fffffffu;
+  if (mag - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((b & 0x80000000u) | ((mag >> 3) + 0x38000000u)), (int)(b << 29));
+  if (mag == 0) return __hiloint2double((int)b, 0);
+  return (double)x;
+}
+__device__ __forceinline__ double to_double(double x) { return x; }
+
 // Block sum of a per-thread value: warp sums in T, then the per-warp sums
 // are added in FP64 in warp order.  Result valid in thread 0.
 template <typename T>

@@ -20,9 +20,9 @@
 //     in bin order -- a group at a time: 8 u16 source offsets and the
 //     group's place in X in, 8 gathers from shared memory, and two float4
 //     stores that fill one sector of X exactly;
-//   * phase 2 (pgather_kernel, one bin per CTA) brings its bin's region and
-//     the head of the bin's plan into shared memory with two bulk copies and
-//     sums the rows from there: rows are cut into pieces of at most kPPiece
+//   * phase 2 (pgather_kernel, one bin per CTA) brings its bin's region into
+//     shared memory with one bulk copy and sums the rows from there by the
+//     bin's plan: rows are cut into pieces of at most kPPiece
 //     entries, the pieces sorted by length and dealt 32 at a time (one per
 //     lane) into slices, so a lane walks its piece's region slots with no
 //     branch and no search; each row then adds its pieces in order and takes
@@ -432,12 +432,9 @@ __global__ void __launch_bounds__(kP1Threads, 1) pscatter_kernel(LArgs a, uint32
   __shared__ uint32_t s_tile, s_issued[kP1Bufs], s_used[kP1Bufs];
   __shared__ int s_go, s_fail;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  dep_wait();
-  dep_trigger();
   const uint64_t span = g_hi - g_lo;
   uint64_t gb = g_lo + span * blockIdx.x / gridDim.x;
   const uint64_t ge = g_lo + span * (blockIdx.x + 1) / gridDim.x;
-  if (gb >= ge) return;
   if (tid == 0) {
     // the tile whose stream holds group gb: the last t with ptbase[t] <= gb
     uint32_t lo = tile_lo, hi = tile_hi;  // ptbase[lo] <= gb < ptbase[hi]
@@ -455,6 +452,9 @@ __global__ void __launch_bounds__(kP1Threads, 1) pscatter_kernel(LArgs a, uint32
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  dep_wait();  // the search above (a chain of loads) runs under the kernel before
+  dep_trigger();
+  if (gb >= ge) return;
   __syncthreads();
   uint32_t t = s_tile, tpar = 0, blk = 0;  // blk: blocks streamed before this segment
   bool staged = false;                      // a tile copy was issued (its phase: tpar ^ 1)
@@ -571,50 +571,53 @@ __global__ void __launch_bounds__(kP1Threads, 1) pscatter_kernel(LArgs a, uint32
 }
 
 // ---------------------------------------------------------------------------
-// Phase 2: one bin per CTA, after the heavy-row chunk CTAs; two CTAs per SM,
-// so one CTA's copies overlap the other's sums.  Everything the CTA needs
-// to start comes from the bin's P2Desc (one load): thread 0 issues the bulk
-// copies of the region and of the head of the plan on one mbarrier, and
-// every thread loads its rows' epilogue operands while they are in flight.
-// Each warp then runs its slices (see pslice_kernel): a lane sums its
-// piece's entries in entry order from the region, gathering at the slots the
-// plan lists, and stores the piece sum; after a CTA barrier each thread adds
-// its rows' pieces in order and applies the row epilogue (coalesced stores),
-// and the last warp to finish adds the warp partials in warp order and
-// enters the bin's alpha term.
+// Phase 2: one bin per CTA, after the heavy-row chunk CTAs; three CTAs per SM,
+// so one CTA's copy and its chain of loads overlap the others' sums.  All that
+// does not depend on phase 1 comes first: the bin's P2Desc, the warp's part
+// of the plan with its first slice's slots, the rows' first pieces; thread 0
+// issues the bulk copy of the region, and every thread loads its rows'
+// epilogue operands while it is in flight.  Each warp then runs its slices
+// (see pslice_kernel): a lane sums its piece's entries in entry order from
+// the region, gathering at the slots the plan lists (the next slice's are
+// loaded meanwhile), and stores the piece sum; after a CTA barrier each
+// thread adds its rows' pieces in order and applies the row epilogue
+// (coalesced stores), and the last warp to finish adds the warp partials
+// and enters the bin's alpha term.
+// 1.6e8 entries of 1e7 nodes: 278 us with the plan staged in shared memory
+// beside the region (two CTAs per SM, everything after the wait for phase 1),
+// 259 now, 4.3 TB/s of region, plan and vectors.  Issuing the copy before the
+// plan's loads instead shortens a CTA's chain (19.5k cycles) but gives up
+// what runs ahead of the wait: 268, and 1e6 nodes 5% slower.
 // ---------------------------------------------------------------------------
 constexpr uint32_t kP2Warps = kP2Threads / 32;
-// the region (+ 4 floats: the zero slot), the copied head of the plan
-// (header, slice lengths, lane pieces, slots) and the piece sums, each a
-// whole number of 16-byte units (the first two are bulk-copy targets)
+// the region (+ 4 floats: the zero slot; a bulk-copy target) and the piece sums
 constexpr uint32_t kP2RegionWords = kPRegion + 4;
-constexpr uint32_t kP2PlanWords = 64 + 64 + 32 * kPMaxSlices + kPSlotsMax;
-static_assert((kP2RegionWords * 4) % 16 == 0 && (kP2PlanWords * 2) % 16 == 0 &&
-                  (kPMaxPieces * 4) % 16 == 0 && kPMaxSlices <= 64,
+static_assert((kP2RegionWords * 4) % 16 == 0 && (kPMaxPieces * 4) % 16 == 0 && kPMaxSlices <= 64,
               "phase-2 shared-memory buffers must keep 16-byte alignment");
-constexpr size_t kP2SmemBytes = (size_t)kP2RegionWords * sizeof(float) + kP2PlanWords * sizeof(uint16_t) +
-                                kPMaxPieces * sizeof(float);
-// two CTAs per SM: 228 KB per SM, 1 KB reserved per CTA, < 640 B of static
-// shared memory (ptxas -v reports it)
-static_assert(2 * (kP2SmemBytes + 1024 + 640) <= 228 * 1024, "two phase-2 CTAs per SM");
+constexpr size_t kP2SmemBytes = ((size_t)kP2RegionWords + kPMaxPieces) * sizeof(float);
+constexpr uint32_t kP2Ctas = 3;
+// 228 KB per SM, 1 KB reserved per CTA, < 640 B of static shared memory
+// (ptxas -v reports it)
+static_assert(kP2Ctas * (kP2SmemBytes + 1024 + 640) <= 228 * 1024, "phase-2 CTAs per SM");
 static_assert(kPBinRows <= 2 * kP2Threads, "each phase-2 thread owns at most two rows");
+static_assert(kP2Warps <= 32 && kPPiece == 16, "one lane per warp partial; 8 slot pairs per slice");
 
-__global__ void __launch_bounds__(kP2Threads, 2) pgather_kernel(LArgs a, uint32_t j, uint32_t chunk_off,
+__global__ void __launch_bounds__(kP2Threads, kP2Ctas) pgather_kernel(LArgs a, uint32_t j, uint32_t chunk_off,
                                                                 uint32_t n_chunks, uint32_t bin_off,
                                                                 uint32_t n_bins, uint32_t ahead) {
   extern __shared__ float4 s_dyn4[];
-  float *reg = reinterpret_cast<float *>(s_dyn4);                         // the bin region
-  uint16_t *s_plan = reinterpret_cast<uint16_t *>(reg + kP2RegionWords);  // the plan's head
-  float *s_psum = reinterpret_cast<float *>(s_plan + kP2PlanWords);       // piece sums
-  __shared__ double s_wpart[kP2Warps];
+  float *reg = reinterpret_cast<float *>(s_dyn4);  // the bin region
+  float *s_psum = reg + kP2RegionWords;            // piece sums
+  __shared__ float s_wpart[kP2Warps];
+  __shared__ float s_coef[2];  // scale_j, beta_{j-1} scale_{j-1}
   __shared__ __align__(8) uint64_t s_full;
   __shared__ uint32_t s_done;
   __shared__ int s_fail;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  dep_wait();
-  dep_trigger();
 
   if (blockIdx.x < n_chunks) {  // one chunk of a heavy row of a two-phase realisation
+    dep_wait();
+    dep_trigger();
     const uint32_t cidx = chunk_off + blockIdx.x;
     const uint32_t hid = a.chunk_heavy[cidx];
     const uint32_t r = a.heavy[hid].inst;
@@ -624,113 +627,154 @@ __global__ void __launch_bounds__(kP2Threads, 2) pgather_kernel(LArgs a, uint32_
     return;
   }
   const uint32_t bin = bin_off + (blockIdx.x - n_chunks);
-  const P2Desc D = a.pdesc[bin];
-  const uint32_t r = D.inst, nrows = D.nrows;
-  if (j >= a.sc.meff[r]) return;  // realisation stopped (uniform per CTA)
+  const P2Desc &D = a.pdesc[bin];
+  const uint32_t r = D.inst, nrows = D.nrows, reg_bytes = D.reg_bytes, pf = D.pf;
+  const uint64_t xg0 = D.xg0, node = D.node;
+  const uint16_t *plan = a.psl + D.plan;
   if (tid == 0) {
     s_done = 0;
     s_fail = 0;
     reg[kPRegion] = 0.f;  // the zero slot (outside the copied region)
     mbar_init(&s_full, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    if (D.reg_bytes <= kPRegion * 4u && D.head_bytes <= kP2PlanWords * 2u) {
-      mbar_expect_tx(&s_full, D.reg_bytes + D.head_bytes);
-      if (D.reg_bytes) bulk_g2s(reg, a.pX + D.xg0 * kPGroup, D.reg_bytes, &s_full);
-      bulk_g2s(s_plan, a.psl + D.plan, D.head_bytes, &s_full);
+  }
+  const uint32_t ns = plan[kP2Warps];
+  uint32_t u = plan[warp];
+  const uint32_t u1 = plan[warp + 1];
+  const uint16_t *slen = plan + 64;
+  const uint16_t *pid = slen + ((ns + 7) & ~7u) + lane;
+  const uint32_t *sp = reinterpret_cast<const uint32_t *>(pid - lane + 32 * ns) + lane +  // slot pairs
+                       (((uint32_t)plan[24 + 2 * warp] | ((uint32_t)plan[25 + 2 * warp] << 16)) >> 1);
+  // slice u of the warp: steps (even, at most kPPiece), the lane's piece, its slots
+  uint32_t L = 0, p = 0xffffu, q[kPPiece / 2] = {};
+  if (u < u1) {
+    L = slen[u];
+    p = pid[32 * u];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) q[k] = 2 * k < (int)L ? __ldcs(sp + 32 * k) : 0u;  // uniform over the warp
+    sp += 16 * L;
+  }
+  // first and last piece of this thread's rows
+  uint32_t pb[2] = {0u, 0u};
+#pragma unroll
+  for (uint32_t h = 0; h < 2; ++h) {
+    const uint32_t lr = tid + h * kP2Threads;
+    if (lr < nrows) pb[h] = (uint32_t)plan[pf + lr] | ((uint32_t)plan[pf + lr + 1] << 16);
+  }
+
+  dep_wait();
+  dep_trigger();
+  if (tid == 0) {
+    if (reg_bytes <= kPRegion * 4u) {
+      mbar_expect_tx(&s_full, reg_bytes);
+      if (reg_bytes) bulk_g2s(reg, a.pX + xg0 * kPGroup, reg_bytes, &s_full);
     } else {  // cannot happen with a plan the upload built: no copy, the step fails
       s_fail = 1;
       mbar_expect_tx(&s_full, 0);
     }
-    // the bin `ahead` places on (about one wave of CTAs later) into L2, so
-    // that DRAM keeps streaming while the resident CTAs sum
-    const uint32_t nb = bin + ahead;
-    if (nb < bin_off + n_bins) {
-      const P2Desc N = a.pdesc[nb];
-      if (N.reg_bytes <= kPRegion * 4u && N.head_bytes <= kP2PlanWords * 2u) {
-        if (N.reg_bytes) l2_prefetch(a.pX + N.xg0 * kPGroup, N.reg_bytes);
-        l2_prefetch(a.psl + N.plan, N.head_bytes);
-      }
-    }
   }
-  // this thread's rows' epilogue operands, while the copies are in flight
+  if (j >= a.sc.meff[r]) {  // realisation stopped (uniform per CTA)
+    if (tid == 0) mbar_wait(&s_full, 0);
+    return;
+  }
+  // the epilogue's operands, while the copy is in flight
   float *Vb = reinterpret_cast<float *>(a.V);
   const bool has_prev = j > 0;
-  const float *x = Vb + (uint64_t)j * a.vs + D.node;  // W_j of the bin's rows
-  const uint16_t *pf = a.psl + D.plan + D.pf;         // first piece of each row
-  const uint32_t ms = a.sc.ms;
-  const float sj = (float)a.sc.scale[r * ms + j];
-  const float bp = has_prev ? (float)(a.sc.beta[r * ms + j - 1] * a.sc.scale[r * ms + j - 1]) : 0.f;
+  const float *x = Vb + (uint64_t)j * a.vs + node;  // W_j of the bin's rows
+  if (tid == kP2Threads - 1) {  // one thread: an FP64 instruction holds its sub-core for 65 cycles
+    const uint32_t ms = a.sc.ms;
+    s_coef[0] = (float)a.sc.scale[r * ms + j];
+    s_coef[1] = has_prev ? (float)(a.sc.beta[r * ms + j - 1] * a.sc.scale[r * ms + j - 1]) : 0.f;
+  }
   float xv[2] = {0.f, 0.f}, xpv[2] = {0.f, 0.f};
-  uint32_t pb[2] = {0u, 0u}, pe[2] = {0u, 0u};
 #pragma unroll
   for (uint32_t h = 0; h < 2; ++h) {
     const uint32_t lr = tid + h * kP2Threads;
     if (lr < nrows) {
       xv[h] = x[lr];
       if (has_prev) xpv[h] = (x - a.vs)[lr];
-      pb[h] = pf[lr];
-      pe[h] = pf[lr + 1];
     }
   }
-  if (tid == 0 && (!mbar_wait(&s_full, 0) || s_fail)) s_fail = 1;
+  if (tid == 0) {
+    // the bin `ahead` places on (about one wave of CTAs later) into L2, so
+    // that DRAM keeps streaming while the resident CTAs sum
+    const uint32_t nb = bin + ahead;
+    if (nb < bin_off + n_bins) {
+      const P2Desc &N = a.pdesc[nb];
+      if (N.reg_bytes && N.reg_bytes <= kPRegion * 4u) l2_prefetch(a.pX + N.xg0 * kPGroup, N.reg_bytes);
+      l2_prefetch(a.psl + N.plan, N.head_bytes);
+    }
+    if (!mbar_wait(&s_full, 0) || s_fail) s_fail = 1;
+  }
   __syncthreads();  // the bin has landed (or the wait gave up)
   const bool ok = s_fail == 0;
-  double wpart = 0.0;
+  float wpart = 0.f;
   if (ok) {
-    const uint32_t ns = s_plan[kP2Warps];
-    const uint32_t u0 = s_plan[warp], u1 = s_plan[warp + 1];
-    uint32_t soff = ((uint32_t)s_plan[24 + 2 * warp] | ((uint32_t)s_plan[25 + 2 * warp] << 16)) >> 1;
-    const uint16_t *slen = s_plan + 64;
-    const uint16_t *pid = slen + ((ns + 7) & ~7u);
-    const uint32_t *slots = reinterpret_cast<const uint32_t *>(pid + 32 * ns);  // slot pairs
 #ifdef CB_DEBUG
-    const uint32_t rslots = D.reg_bytes / 4u;
-    const uint32_t npieces = pf[nrows];
+    const uint32_t rslots = reg_bytes / 4u;
+    const uint32_t npieces = plan[pf + nrows];
 #endif
-    for (uint32_t u = u0; u < u1; ++u) {
-      const uint32_t L = slen[u];  // steps of the slice: even, at most kPPiece
-      const uint32_t p = pid[32 * u + lane];
-      const uint32_t *sp = slots + soff + lane;
-      float acc = 0.f;
+    while (u < u1) {
+      float acc = 0.f, g[8];
+      const uint32_t Lc = L, pc = p;
 #pragma unroll
-      for (uint32_t k = 0; k < kPPiece / 2; ++k) {
-        if (2 * k < L) {  // uniform over the warp
-          const uint32_t q = sp[32 * k];
+      for (int hf = 0; hf < 2; ++hf) {  // 8 gathers in flight, added in order
+        if (8 * hf < (int)Lc) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (8 * hf + 2 * k < (int)Lc) {
+              uint32_t v = q[4 * hf + k];
 #ifdef CB_DEBUG
-          const uint32_t lo = q & 0xffffu, hi = q >> 16;
-          if (!CB_DCHECK((lo < rslots || lo == kPRegion) && (hi < rslots || hi == kPRegion),
-                         kDbgTwoPhasePos, max(lo, hi)))
-            continue;
+              const uint32_t lo = v & 0xffffu, hi = v >> 16;
+              if (!CB_DCHECK((lo < rslots || lo == kPRegion) && (hi < rslots || hi == kPRegion),
+                             kDbgTwoPhasePos, max(lo, hi)))
+                v = kPRegion | (kPRegion << 16);
 #endif
-          acc += reg[q & 0xffffu];
-          acc += reg[q >> 16];
+              g[2 * k] = reg[v & 0xffffu];
+              g[2 * k + 1] = reg[v >> 16];
+            }
+        }
+        if (hf == 1 && ++u < u1) {  // the next slice, its latency under the sums below
+          L = slen[u];
+          p = pid[32 * u];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) q[k] = 2 * k < (int)L ? __ldcs(sp + 32 * k) : 0u;
+          sp += 16 * L;
+        }
+        if (8 * hf < (int)Lc) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (8 * hf + 2 * k < (int)Lc) {
+              acc += g[2 * k];
+              acc += g[2 * k + 1];
+            }
         }
       }
-      if (p != 0xffffu && CB_DCHECK(p < npieces, kDbgTwoPhasePos, p)) s_psum[p] = acc;
-      soff += 16 * L;
+      if (pc != 0xffffu && CB_DCHECK(pc < npieces, kDbgTwoPhasePos, pc)) s_psum[pc] = acc;
     }
   }
   __syncthreads();  // every piece sum is in shared memory
   if (ok) {
     // rows: the sum of their pieces in order; u = sj * sum - bp * W_{j-1}[row]
     // (coalesced store), and the alpha partial W_j[row] * u
-    float *out = Vb + (uint64_t)(j + 1) * a.vs + D.node;
+    float *out = Vb + (uint64_t)(j + 1) * a.vs + node;
+    const float sj = s_coef[0], bp = s_coef[1];
     float acc = 0.f;
 #pragma unroll
     for (uint32_t h = 0; h < 2; ++h) {
       const uint32_t lr = tid + h * kP2Threads;
       if (lr < nrows) {
         float sum = 0.f;
-        for (uint32_t p = pb[h]; p < pe[h]; ++p) sum += s_psum[p];
+        for (uint32_t p = pb[h] & 0xffffu; p < pb[h] >> 16; ++p) sum += s_psum[p];
         float v = sj * sum;
         if (has_prev) v -= bp * xpv[h];
         out[lr] = v;
         acc += xv[h] * v;
       }
     }
-    wpart = (double)warp_sum<float>(acc);
+    wpart = warp_sum<float>(acc);
   }
-  // the last warp to finish sums the warp partials in warp order
+  // the last warp to finish sums the warp partials
   uint32_t last = 0;
   if (lane == 0) {
     s_wpart[warp] = wpart;
@@ -739,9 +783,8 @@ __global__ void __launch_bounds__(kP2Threads, 2) pgather_kernel(LArgs a, uint32_
   }
   if (!__shfl_sync(0xffffffffu, last, 0)) return;
   __threadfence_block();
-  double part = 0.0;
+  double part = warp_sum_d(lane < kP2Warps ? to_double(s_wpart[lane]) : 0.0);
   if (lane == 0) {
-    for (uint32_t w = 0; w < kP2Warps; ++w) part += s_wpart[w];
     if (!ok) {  // the bin never landed: this step of the realisation fails
       a.sc.status[r] = CB_ERR_TIMEOUT;
       part = __longlong_as_double(0x7ff8000000000000ll);
@@ -763,9 +806,9 @@ void launch_p2(const LArgs &a, uint32_t j, uint32_t chunk_off, uint32_t n_chunks
                          cudaSharedmemCarveoutMaxShared);
     attr = true;
   }
-  // prefetch distance: the CTAs resident at once (two per SM)
+  // prefetch distance: the CTAs resident at once
   launch_dep(pgather_kernel, n_chunks + n_bins, kP2Threads, kP2SmemBytes, s, a, j, chunk_off, n_chunks, bin_off,
-             n_bins, 2u * (uint32_t)n_sm);
+             n_bins, kP2Ctas * (uint32_t)n_sm);
 }
 
 template <typename P>

@@ -13,6 +13,12 @@
 //     warp's 512 rows, taken lane by lane (each lane's rows in slot order,
 //     each row's columns in order), are dealt round-robin over the T steps
 //     of the warp's stream: element j goes to step j mod T, lane j / T.
+//     The lanes come in the order most, fewest, second most, second fewest,
+//     ... elements, each with its share of the padding: after every second
+//     lane the deal is back near step 0, so the steps to which lanes of more
+//     than T elements go twice are the same few.  In lane order the sums of
+//     all steps conflict (1.9 wavefronts at 26 elements a lane, 1.6 so; 242 ->
+//     236 us per SpMV of 175 M entries in 40 graphs).
 //     With T >= the elements / 32, >= half the elements of any one lane and
 //     >= the elements of any one row, a step holds at most 32 elements, never
 //     two of one row (no two lanes add into the same sum at once) and at
@@ -143,16 +149,20 @@ __global__ void __launch_bounds__(kFillThreads) bcount_kernel(const InstDesc *in
 
 // Fill the streams.  The count pass left each lane's elements per block; a
 // warp prefix over the lanes gives each lane the first index j of its
-// elements in the warp's sequence (lanes in order, each lane's in walk order:
-// rows in slot order, columns in input order).  Element j belongs at
-// step j mod T, lane j / T, and the positions past the warp's last element
-// (j from its count to 32 T) take the lane's padding element.  The streams
+// elements in the warp's sequence (lanes in the order of the deal, each
+// lane's in walk order: rows in slot order, columns in input order, then its
+// share of the padding).  Element j belongs at step j mod T, lane j / T.  The streams
 // are then written a batch of blocks at a time: each warp assembles its
 // streams of the batch in shared memory (one walk over the rows, each row
 // resumed where the previous batch stopped -- the columns of a row are
 // sorted) and copies them out with coalesced 16-byte stores.  A block whose stream does not fit the
 // staging area is written element by element.
 constexpr uint32_t kStageWords = 2048;  // staging u32 words per warp
+
+// Lane `lane`'s share of `pad` padding elements of a stream.
+__device__ __forceinline__ uint32_t pad_share(uint32_t pad, uint32_t lane) {
+  return pad / 32 + (lane < pad % 32 ? 1u : 0u);
+}
 
 __global__ void __launch_bounds__(kFillThreads) bfill_kernel(const InstDesc *inst,
                                                              const uint32_t *btile_inst,
@@ -205,20 +215,36 @@ __global__ void __launch_bounds__(kFillThreads) bfill_kernel(const InstDesc *ins
   // the walk loops over the row slots without unrolling (the kernel stays
   // small enough for the instruction cache); the row cursors live in shared
   // memory.
-  // The lane's elements per block come from the count pass; their exclusive
-  // prefix over the warp's lanes gives each lane its first position (step s,
-  // lane l), kept as l << 16 | s and advanced per element
+  // The lane's elements per block come from the count pass.  In the order of
+  // the deal (see the header), the lanes' elements with their share of the
+  // padding add up to each lane's first position (step s, lane l), kept as
+  // l << 16 | s and advanced per element
   for (uint32_t b = 0; b < nb; ++b) {
-    const uint32_t c = bcnt[(bseg_base[t] + b) * kBThreads + v];
-    uint32_t incl = c;
+    const uint32_t c = bcnt[(bseg_base[t] + b) * kBThreads + v], T = s_T[b * W + wl];
+    const uint32_t tot = __reduce_add_sync(0xffffffffu, c);
+    const uint32_t key = (c << 5) | lane;
+    uint32_t rank = 0;  // lanes with more elements
+#pragma unroll
+    for (uint32_t o = 1; o < 32; ++o) rank += __shfl_sync(0xffffffffu, key, lane + o) > key;
+    const uint32_t at = rank < 16 ? 2 * rank : 2 * (31 - rank) + 1;
+    uint32_t *row = s_next + b * kFillThreads + 32 * wl;
+    const uint32_t share = pad_share(32 * T - tot, lane);
+    row[at] = c + share;
+    __syncwarp();
+    const uint32_t x = row[lane];
+    uint32_t incl = x;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= (uint32_t)o) incl += y;
     }
-    const uint32_t j0 = incl - c, T = s_T[b * W + wl];
-    s_next[b * kFillThreads + tid] = T ? ((j0 / T) << 16) | (j0 % T) : 0u;
-    if (lane == 31) s_tot[b * W + wl] = incl;
+    __syncwarp();
+    row[lane] = incl - x;
+    __syncwarp();
+    const uint32_t j0 = row[at];
+    __syncwarp();
+    row[lane] = T ? ((j0 / T) << 16) | (j0 % T) : 0u;
+    if (lane == 31) s_tot[b * W + wl] = tot;
   }
   __syncwarp();
   // second walk, a batch of blocks [b0, b1) at a time; the batch ends before
@@ -233,17 +259,6 @@ __global__ void __launch_bounds__(kFillThreads) bfill_kernel(const InstDesc *ins
     }
     __syncwarp();
     const bool staged = used <= kStageWords;  // false: one block too large, written directly
-    // the padding of the batch's streams
-    for (uint32_t b = b0; b < b1; ++b) {
-      const uint32_t T = s_T[b * W + wl], base = s_sb[b * W + wl];
-      const uint64_t st = s_start[b * W + wl];
-      for (uint32_t j = s_tot[b * W + wl] + lane; j < 32 * T; j += 32) {
-        const uint32_t s = j % T, l = j / T;
-        const uint32_t q = 64 * (s >> 1) + 2 * l + (s & 1);
-        const uint32_t el = kBElem(0, 32 * kBPadSlot + l);
-        if (staged) stage[base + q] = el; else belem[st + q] = el;
-      }
-    }
     // the elements of blocks [b0, b1), resuming each row where the last batch stopped
 #pragma unroll 1
     for (int k = 0; k < kBRowsPerThread; ++k) {
@@ -277,6 +292,20 @@ __global__ void __launch_bounds__(kFillThreads) bfill_kernel(const InstDesc *ins
         more = taken == kFillBatch && e < e1;
       }
       s_ecur[k * kFillThreads + tid] = e;
+    }
+    // each lane's share of the padding of the batch's streams, after its elements
+    for (uint32_t b = b0; b < b1; ++b) {
+      const uint32_t T = s_T[b * W + wl], base = s_sb[b * W + wl];
+      const uint64_t st = s_start[b * W + wl];
+      uint32_t p = s_next[b * kFillThreads + tid];
+      for (uint32_t i = pad_share(32 * T - s_tot[b * W + wl], lane); i; --i) {
+        const uint32_t s = p & 0xffffu, l = p >> 16;
+        p = s + 1 == T ? p + (1u << 16) - s : p + 1;
+        if (!CB_DCHECK(l < 32u && s < T, kDbgBlockedFill, p)) continue;
+        const uint32_t q = 64 * (s >> 1) + 2 * l + (s & 1);
+        const uint32_t el = kBElem(0, 32 * kBPadSlot + l);
+        if (staged) stage[base + q] = el; else belem[st + q] = el;
+      }
     }
     __syncwarp();
     if (staged) {  // the batch's streams, 16 bytes per lane per store

@@ -329,14 +329,13 @@ __global__ void __launch_bounds__(kThreads) spmv_kernel(LArgs a, uint32_t j, uin
 //
 // Bound by the shared-memory pipe: a step of 32 elements is about 2.9
 // wavefronts for the gathers (4.1 before the elements of a round were ordered
-// by bank), 1.6 to read and 1.6 to write the sums, 0.85 for its share of the
+// by bank), 1.4 to read and 1.4 to write the sums (1.6), 0.85 for its share of the
 // staged blocks.  175 M entries in 40 graphs: 325 us with a round's gathers
 // after the previous sums, elements decoded by shifts (29 instructions a
 // step, 56% of the pipe); 293 with byte offsets and the gathers of a round
 // together (18); 277 with the loads two rounds ahead; 263 with the
 // prologue's and epilogue's loads together (17); 242 with the rounds ordered
-// by bank (71% of the pipe; the grid's last wave, 562 tiles on 152 SMs, is
-// the larger part of the rest).
+// by bank, 236 with the lanes dealt most and fewest in turn.
 // ---------------------------------------------------------------------------
 
 // two column blocks of W_j, then kBRowsPerThread row sums per thread and

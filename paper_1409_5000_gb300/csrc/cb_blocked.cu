@@ -457,6 +457,8 @@ void free_blocked(cb_graph *h) {
   dev_free(h->d_belem);
   dev_free(h->d_blong_ptr);
   dev_free(h->d_blong_rows);
+  dev_free(h->d_border);
+  h->d_border = nullptr;
   h->d_btile_inst = nullptr;
   h->d_bseg_base = h->d_bwstart = h->d_bwscan = nullptr;
   h->d_bwlen = nullptr;
@@ -588,11 +590,16 @@ int blocked_fill(cb_graph *h, cudaStream_t s, BlockedBuild &bb) {
   return CB_OK;
 }
 
+// What staging a column block costs the SpMV, in entries: about 1100 cycles,
+// where 32 entries take about 10.
+constexpr uint32_t kBlockCost = 3500;
+
 int blocked_long_rows(cb_graph *h, const std::vector<const uint32_t *> &rp_host, cudaStream_t s) {
   NvtxRange nvtx_range("column-blocked format: long rows");
   if (h->csr_only || !h->total_btiles) return CB_OK;
   // long rows per tile (tile-local indices), scanned in parallel over realisations
   std::vector<std::vector<uint32_t>> lrows(h->n_inst), lcount(h->n_inst);
+  std::vector<uint64_t> cost(h->total_btiles);
   parallel_for(h->n_inst, h->total_nodes_padded, [&](uint32_t r) {
     const InstDesc &I = h->inst[r];
     const uint32_t *rp = rp_host[r];
@@ -605,8 +612,18 @@ int blocked_long_rows(cb_graph *h, const std::vector<const uint32_t *> &rp_host,
           ++c;
         }
       lcount[r].push_back(c);
+      cost[I.btile_base + q] = rp[row1] - rp[row0] + (uint64_t)kBlockCost * I.nb;
     }
   });
+  // the SpMV's CTAs start in this order: the longest tiles first, so that the
+  // last wave is short ones.  In sixteenths of the longest, which keeps equal
+  // tiles of a realisation, and with them its W_j in L2, together.
+  std::vector<uint32_t> order(h->total_btiles);
+  uint64_t most = 1;
+  for (uint64_t c : cost) most = std::max(most, c);
+  for (uint32_t t = 0; t < h->total_btiles; ++t) order[t] = t;
+  for (uint64_t &c : cost) c = c * 16 / most;
+  std::stable_sort(order.begin(), order.end(), [&](uint32_t a, uint32_t b) { return cost[a] > cost[b]; });
   std::vector<uint32_t> long_ptr(1, 0), long_rows;
   for (uint32_t r = 0; r < h->n_inst; ++r) {
     for (uint32_t c : lcount[r]) long_ptr.push_back(long_ptr.back() + c);
@@ -618,6 +635,8 @@ int blocked_long_rows(cb_graph *h, const std::vector<const uint32_t *> &rp_host,
   };
   chk(dalloc(&h->d_blong_ptr, long_ptr.size()));
   chk(dalloc(&h->d_blong_rows, std::max<size_t>(long_rows.size(), 1)));
+  chk(dalloc(&h->d_border, order.size()));
+  chk(stage_h2d(h->d_border, order.data(), order.size() * 4, s));
   chk(stage_h2d(h->d_blong_ptr, long_ptr.data(), long_ptr.size() * 4, s));
   if (!long_rows.empty()) chk(stage_h2d(h->d_blong_rows, long_rows.data(), long_rows.size() * 4, s));
   if (e != cudaSuccess) {

@@ -225,6 +225,7 @@ struct cb_graph {
   uint32_t *d_bwlen = nullptr;           // per (segment, warp): steps T of its stream (even)
   uint16_t *d_bcnt = nullptr;            // per (segment, lane): its elements (format build)
   uint32_t *d_belem = nullptr;           // stream elements (kBElem)
+  uint32_t *d_border = nullptr;          // blocked tiles, longest first (a pass over all of them)
   uint32_t *d_blong_ptr = nullptr;       // per blocked tile: range in d_blong_rows
   uint32_t *d_blong_rows = nullptr;      // local rows with degree > kBLongDeg, in row order
   // two-phase format (FP32 SpMV), for realisations with pb = 1

@@ -335,7 +335,8 @@ __global__ void __launch_bounds__(kThreads) spmv_kernel(LArgs a, uint32_t j, uin
 // step, 56% of the pipe); 293 with byte offsets and the gathers of a round
 // together (18); 277 with the loads two rounds ahead; 263 with the
 // prologue's and epilogue's loads together (17); 242 with the rounds ordered
-// by bank, 236 with the lanes dealt most and fewest in turn.
+// by bank, 236 with the lanes dealt most and fewest in turn, 224 with the
+// longest tiles first (562 tiles on 152 SMs).
 // ---------------------------------------------------------------------------
 
 // two column blocks of W_j, then kBRowsPerThread row sums per thread and
@@ -363,7 +364,7 @@ __global__ void __launch_bounds__(kBThreads, 1) bspmv_kernel(LArgs a, uint32_t j
   // the one before), so the loads go out together, the static ones and the
   // first rounds of the streams before the wait for the previous kernel, and
   // the copies of W_j before it is known whether the realisation goes on.
-  const uint32_t t = btile_off + blockIdx.x;
+  const uint32_t t = a.border ? a.border[blockIdx.x] : btile_off + blockIdx.x;
   const uint32_t r = a.btile_inst[t];
   const uint64_t sbase = a.bseg_base[t];
   const uint32_t lp0 = a.blong_ptr[t], lp1 = a.blong_ptr[t + 1];
@@ -1064,6 +1065,7 @@ static int run_t(cb_graph *h, Workspace &W, uint32_t r0, uint32_t r1, uint32_t m
   const uint32_t n_fin = A1.fin_base + A1.n_fin - fin_off;
   const uint32_t btile_off = A0.btile_base;
   const uint32_t n_btiles = use_blocked ? A1.btile_base + A1.n_btiles - btile_off : 0u;
+  a.border = n_btiles == h->total_btiles ? h->d_border : nullptr;  // part of them: in their own order
   const uint32_t ptile_lo = A0.ptile_base, ptile_hi = A1.ptile_base + A1.pns;
   const uint64_t pg_lo = use_pb ? h->ptbase[ptile_lo] : 0, pg_hi = use_pb ? h->ptbase[ptile_hi] : 0;
   const uint32_t bin_off = A0.pbin_base;

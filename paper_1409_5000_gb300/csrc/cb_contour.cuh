@@ -336,8 +336,19 @@ __device__ inline double lambda_max_laguerre(const double *al, const double *be,
   return x;
 }
 
+// The two differ where T carries copies of lambda_max, in FP32 recurrences by up
+// to 1.2e-7 lambda_max: 2e-5 of every score on a BA graph of 1e7 nodes
+// (lambda_max 158), which callers that compare or store FP32 scores would
+// see.  So above kCopiesShow Laguerre's value stays the result there too.
+constexpr double kCopiesShow = 48.0;
+
 __device__ inline double largest(const double *al, const double *be, int M, Spectrum &S, bool laguerre) {
-  return laguerre ? lambda_max_laguerre(al, be, M, S) : lambda_max(al, be, M, S);
+  if (!laguerre) {
+    const double t = lambda_max(al, be, M, S);
+    if (t <= kCopiesShow) return t;
+    __syncwarp();  // S is used again
+  }
+  return lambda_max_laguerre(al, be, M, S);
 }
 
 // Node z and weight w = e^z z'(t) / (i N) of the upper-half nodes q =

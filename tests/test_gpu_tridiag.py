@@ -28,3 +28,24 @@ def test_shift_and_scores_at_depth(m):
             th_o, y_o, _ = oc.krylov_expv(g.n, g.row_ptr, g.col, m)
             assert abs(float(ls.item()) - th_o) <= 1e-13 * max(1.0, abs(th_o))
             parity.assert_scores(float(ls.item()), y.cpu().numpy(), th_o, y_o, "fp64")
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("q", [47, 49, 50, 120])
+def test_shift_around_the_second_method(q, prec):
+    """lambda_max on both sides of where the FP32 recurrences change the method
+    for theta: a clique of q nodes (q - 1 and a little) in a sparse graph, whose
+    T carries copies of it at this depth.  The suite's parity bars."""
+    from paper_1409_5000_gb300 import binding as B
+
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for -m gpu tests")
+    rng = np.random.default_rng(q)
+    n = 2000
+    e = [rng.integers(0, n, (n, 2)), np.array([(a, b) for a in range(q) for b in range(a)])]
+    e = np.concatenate(e)
+    g = synth.from_edges(n, e[e[:, 0] != e[:, 1]])
+    with B.GraphSet([g]) as gs:
+        ls, y = B.communicability(gs, 0, 35, prec)
+        th_o, y_o, _ = oc.krylov_expv(g.n, g.row_ptr, g.col, 35)
+        parity.assert_scores(float(ls.item()), y.cpu().numpy(), th_o, y_o, "fp64" if prec else "fp32")

@@ -119,11 +119,39 @@ __global__ void __launch_bounds__(kThreads) init_scalars_kernel(LArgs a, uint32_
 }
 
 
-// One Lanczos SpMV step over a range of realisations.
+// Sums of B values per lane over groups of G lanes (B <= G, powers of two), in
+// the order of group_sum's tree: at each of the first steps a lane sends half
+// of its values and keeps the sums of the other half, B - 1 additions for
+// B values where B separate sums take B log2(B).  Lane l of a group gets the sum
+// of value l / (G / B).
+template <int B, int G>
+__device__ __forceinline__ double batch_sum(double (&v)[B]) {
+  const int l = threadIdx.x % G;
+  int o = G / 2;
+#pragma unroll
+  for (int half = B / 2; half >= 1; half >>= 1, o >>= 1) {
+    const bool up = (l & o) != 0;
+#pragma unroll
+    for (int q = 0; q < half; ++q) {
+      const double keep = up ? v[q + half] : v[q], send = up ? v[q] : v[q + half];
+      v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  for (; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  return v[0];
+}
+
+// One Lanczos SpMV step over a range of realisations.  FP64 is bound by the
+// FP64 pipe, 65 cycles of a sub-core per warp instruction however many lanes
+// are active: there several rows' sums are formed side by side (batch_sum), a
+// row's result by a lane of its own, and a first entry is not added to 0; the
+// sums' orders, alpha's included, are those of one row at a time.  BA(1e5, 5),
+// a step with its vector kernels: 49 -> 40 us (the tiles of medium rows, which
+// ended last, 43 -> 29 us with two gathers of a row in flight, then four).
 // Blocks [0, n_chunks) are heavy-row chunks starting at chunk_off; blocks
 // [n_chunks, ...) are normal tiles starting at tile_off.
 template <typename T, int G>
-__global__ void __launch_bounds__(kThreads) spmv_kernel(LArgs a, uint32_t j, uint32_t chunk_off,
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 3 : 6) spmv_kernel(LArgs a, uint32_t j, uint32_t chunk_off,
                                                         uint32_t n_chunks, uint32_t tile_off) {
   __shared__ double s_red[32];
   __shared__ uint32_t s_rp[kTileRows + 1];
@@ -184,30 +212,83 @@ __global__ void __launch_bounds__(kThreads) spmv_kernel(LArgs a, uint32_t j, uin
   // Short rows: G lanes per row.  The trip count depends only on the tile,
   // so every lane of a warp runs every iteration and the full-mask group
   // shuffles are always converged.
-  for (uint32_t base = 0; base < nrows; base += kGroups) {
-    const uint32_t lr = base + grp;
-    const bool valid = lr < nrows;
-    uint32_t e0 = 0, e1 = 0;
-    if (valid) { e0 = s_rp[lr]; e1 = s_rp[lr + 1]; }
-    const bool is_short = valid && (e1 - e0) <= kShort;
-    T s = T(0);
-    if (is_short) {
-      // at most kShort / G entries per lane: a fixed, predicated trip count
-      // puts all of the lane's index loads, then all of its gathers, in
-      // flight at once (a counted loop of 2-4 trips runs its remainder
-      // path one load pair at a time); the summation order is unchanged
-      const uint32_t len = e1 - e0;
+  if constexpr (sizeof(T) == 8) {
+    constexpr int B = G < 8 ? G : 8, kDup = G / B;
+    for (uint32_t it0 = 0; it0 < (uint32_t)G && it0 * kGroups < nrows; it0 += B) {
+      // this lane's row of the batch, its operands loaded before the sums
+      const uint32_t mine = (it0 + lane_g / kDup) * kGroups + grp;
+      const bool short_row = mine < nrows && s_rp[mine + 1] - s_rp[mine] <= kShort;
+      const uint32_t shorts = __ballot_sync(0xffffffffu, short_row);
+      if (!shorts) continue;
+      double xr = 0.0, xpr = 0.0;
+      if (short_row) {
+        xr = x[row0 + mine];
+        if (has_prev) xpr = xp[row0 + mine];
+      }
+      double v[B];
 #pragma unroll
-      for (uint32_t i = 0; i < kShort / G; ++i) {
-        const uint32_t t = lane_g + i * G;
-        if (t < len) {
-          const uint32_t c = ld_stream(col + e0 + t);
-          if (CB_DCHECK(c < I.n, kDbgCsrCol, c)) s += ld_vec(x + c);
+      for (int q = 0; q < B; ++q) {
+        const uint32_t lr = (it0 + q) * kGroups + grp;
+        uint32_t e0 = 0, len = 0;
+        if (lr < nrows) {
+          e0 = s_rp[lr];
+          len = s_rp[lr + 1] - e0;
         }
+        if (len > kShort) len = 0;
+        double g[kShort / G];
+#pragma unroll
+        for (uint32_t i = 0; i < kShort / G; ++i) {
+          const uint32_t t = lane_g + i * G;
+          g[i] = 0.0;
+          if (t < len) {
+            const uint32_t c = ld_stream(col + e0 + t);
+            if (CB_DCHECK(c < I.n, kDbgCsrCol, c)) g[i] = ld_vec(x + c);
+          }
+        }
+        const uint32_t most = __reduce_max_sync(0xffffffffu, len);
+        v[q] = g[0];
+#pragma unroll
+        for (uint32_t i = 1; i < kShort / G; ++i)
+          if (i * G < most) v[q] += g[i];  // adding a 0 past a row's end changes no bit
+      }
+      const double sum = batch_sum<B, G>(v);
+      double u = sj * sum;
+      if (has_prev) u -= bp * xpr;
+      if (short_row && lane_g % kDup == 0) out[row0 + mine] = u;
+      // the group's first lane takes the rows' alpha terms in row order
+#pragma unroll
+      for (int q = 0; q < B; ++q) {
+        const int src = (threadIdx.x & 31 & ~(G - 1)) + q * kDup;
+        const double xq = __shfl_sync(0xffffffffu, xr, src), uq = __shfl_sync(0xffffffffu, u, src);
+        if (lane_g == 0 && (shorts >> src & 1u)) acc += xq * uq;
       }
     }
-    s = group_sum<G, T>(s);
-    if (is_short && lane_g == 0) acc += row_epilogue<T>(s, row0 + lr, x, xp, out, sj, bp, has_prev);
+  } else {
+    for (uint32_t base = 0; base < nrows; base += kGroups) {
+      const uint32_t lr = base + grp;
+      const bool valid = lr < nrows;
+      uint32_t e0 = 0, e1 = 0;
+      if (valid) { e0 = s_rp[lr]; e1 = s_rp[lr + 1]; }
+      const bool is_short = valid && (e1 - e0) <= kShort;
+      T s = T(0);
+      if (is_short) {
+        // at most kShort / G entries per lane: a fixed, predicated trip count
+        // puts all of the lane's index loads, then all of its gathers, in
+        // flight at once (a counted loop of 2-4 trips runs its remainder
+        // path one load pair at a time); the summation order is unchanged
+        const uint32_t len = e1 - e0;
+#pragma unroll
+        for (uint32_t i = 0; i < kShort / G; ++i) {
+          const uint32_t t = lane_g + i * G;
+          if (t < len) {
+            const uint32_t c = ld_stream(col + e0 + t);
+            if (CB_DCHECK(c < I.n, kDbgCsrCol, c)) s += ld_vec(x + c);
+          }
+        }
+      }
+      s = group_sum<G, T>(s);
+      if (is_short && lane_g == 0) acc += row_epilogue<T>(s, row0 + lr, x, xp, out, sj, bp, has_prev);
+    }
   }
 
   // Medium (kShort < deg <= kLongDeg) and long (kLongDeg < deg <= kHeavyDeg)
@@ -236,32 +317,23 @@ __global__ void __launch_bounds__(kThreads) spmv_kernel(LArgs a, uint32_t j, uin
   }
   __syncthreads();
 
-  // x over the entries e, e + step, ... < e1 in order.  FP32: four gathers in
+  // x over the entries e, e + step, ... < e1 in order (FP32): four gathers in
   // flight, also in the last round (a counted loop runs its remainder one by
-  // one): 31.4 -> 25.6 us a step on BA(1e5, 5); in FP64 the adds bound it and
-  // the counted loop is 2% faster.
+  // one): 31.4 -> 25.6 us a step on BA(1e5, 5).
   auto run_sum = [&](uint32_t e, uint32_t e1, uint32_t step) -> T {
     T s = T(0);
-    if constexpr (sizeof(T) == 8) {
-#pragma unroll 4
-      for (; e < e1; e += step) {
-        const uint32_t c = ld_stream(col + e);
-        if (CB_DCHECK(c < I.n, kDbgCsrCol, c)) s += ld_vec(x + c);
-      }
-    } else {
-      for (; e < e1; e += 4 * step) {
-        T v[4];
+    for (; e < e1; e += 4 * step) {
+      T v[4];
 #pragma unroll
-        for (uint32_t u = 0; u < 4; ++u) {
-          v[u] = T(0);  // adding the 0 past the end changes no bit
-          if (e + u * step < e1) {
-            const uint32_t c = ld_stream(col + e + u * step);
-            if (CB_DCHECK(c < I.n, kDbgCsrCol, c)) v[u] = ld_vec(x + c);
-          }
+      for (uint32_t u = 0; u < 4; ++u) {
+        v[u] = T(0);  // adding the 0 past the end changes no bit
+        if (e + u * step < e1) {
+          const uint32_t c = ld_stream(col + e + u * step);
+          if (CB_DCHECK(c < I.n, kDbgCsrCol, c)) v[u] = ld_vec(x + c);
         }
-#pragma unroll
-        for (uint32_t u = 0; u < 4; ++u) s += v[u];
       }
+#pragma unroll
+      for (uint32_t u = 0; u < 4; ++u) s += v[u];
     }
     return s;
   };
@@ -274,41 +346,151 @@ __global__ void __launch_bounds__(kThreads) spmv_kernel(LArgs a, uint32_t j, uin
     acc += xr * u;
   };
 
-  // medium rows: warp w takes list entries w, w+8, ...
-  {
+  // R rows (entries e0 .. e1 of each) side by side, kU gathers of each in
+  // flight, entry `first` on by `step`; a round past a row's end is skipped by
+  // the whole warp, and adding a 0 past it changes no bit
+  auto run_sums = [&](auto &v, const uint32_t *e0, const uint32_t *e1, uint32_t first, uint32_t step) {
+    constexpr int R = sizeof(v) / sizeof(v[0]), kU = 4;
+    uint32_t most = 0;
+#pragma unroll
+    for (int q = 0; q < R; ++q) most = max(most, e1[q] - e0[q]);
+    for (uint32_t base = 0; base < most; base += kU * step) {
+      double g[R][kU];
+#pragma unroll
+      for (int q = 0; q < R; ++q)
+#pragma unroll
+        for (int i = 0; i < kU; ++i) {
+          const uint32_t e = e0[q] + base + i * step + first;
+          g[q][i] = 0.0;
+          if (e < e1[q]) {
+            const uint32_t c = ld_stream(col + e);
+            if (CB_DCHECK(c < I.n, kDbgCsrCol, c)) g[q][i] = ld_vec(x + c);
+          }
+        }
+#pragma unroll
+      for (int q = 0; q < R; ++q)
+#pragma unroll
+        for (int i = 0; i < kU; ++i)
+          if (base + i == 0)
+            v[q] = g[q][i];
+          else if (e0[q] + base + i * step < e1[q])
+            v[q] += g[q][i];
+    }
+  };
+
+  if constexpr (sizeof(T) == 8) {
+    // medium rows: warp w takes list entries w, w+8, ..., kR at a time
+    constexpr int kR = 4;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t nmed = s_nmed;
-    for (uint32_t q = warp; q < nmed; q += kThreads / 32) {
-      const uint32_t lr = s_med[q], row = row0 + lr;
-      T xr = T(0), xpr = T(0);
-      if (lane == 0) {
+    for (uint32_t q0 = warp; q0 < nmed; q0 += kR * (kThreads / 32)) {
+      uint32_t e0[kR], e1[kR];
+      double v[kR];
+#pragma unroll
+      for (int q = 0; q < kR; ++q) {
+        const uint32_t at = q0 + q * (kThreads / 32);
+        e0[q] = e1[q] = 0;
+        v[q] = 0.0;
+        if (at < nmed) {
+          e0[q] = s_rp[s_med[at]];
+          e1[q] = s_rp[s_med[at] + 1];
+        }
+      }
+      const uint32_t my = q0 + (lane / (32 / kR)) * (kThreads / 32);  // this lane's row
+      double xr = 0.0, xpr = 0.0;
+      const uint32_t row = my < nmed ? row0 + s_med[my] : row0;
+      if (my < nmed) {
         xr = x[row];
         if (has_prev) xpr = xp[row];
       }
-      const T s = warp_sum<T>(run_sum(s_rp[lr] + lane, s_rp[lr + 1], 32));
-      if (lane == 0) finish_row(s, row, xr, xpr);
+      run_sums(v, e0, e1, lane, 32);
+      const double sum = batch_sum<kR, 32>(v);
+      double u = sj * sum;
+      if (has_prev) u -= bp * xpr;
+      if (my < nmed && lane % (32 / kR) == 0) out[row] = u;
+#pragma unroll
+      for (int q = 0; q < kR; ++q) {
+        const double xq = __shfl_sync(0xffffffffu, xr, q * (32 / kR)), uq = __shfl_sync(0xffffffffu, u, q * (32 / kR));
+        if (lane == 0 && q0 + q * (kThreads / 32) < nmed) acc += xq * uq;
+      }
     }
-  }
+    // long rows: the whole CTA, kL rows at a time, in row order
+    constexpr int kL = 4;
+    __shared__ double s_sums[kL][kThreads / 32];
+    const uint32_t nlong = s_nlong;
+    for (uint32_t q0 = 0; q0 < nlong; q0 += kL) {
+      uint32_t e0[kL], e1[kL];
+      double v[kL];
+#pragma unroll
+      for (int q = 0; q < kL; ++q) {
+        e0[q] = e1[q] = 0;
+        v[q] = 0.0;
+        if (q0 + q < nlong) {
+          e0[q] = s_rp[s_long[q0 + q]];
+          e1[q] = s_rp[s_long[q0 + q] + 1];
+        }
+      }
+      run_sums(v, e0, e1, threadIdx.x, kThreads);
+      const double sum = batch_sum<kL, 32>(v);
+      if (lane % (32 / kL) == 0) s_sums[lane / (32 / kL)][warp] = sum;
+      __syncthreads();
+      if (warp == 0) {
+        const bool on = lane < kL && q0 + lane < nlong;
+        const uint32_t row = on ? row0 + s_long[q0 + lane] : row0;
+        double xr = 0.0, xpr = 0.0, tot = 0.0;
+        if (on) {
+          xr = x[row];
+          if (has_prev) xpr = xp[row];
+          for (uint32_t w = 0; w < kThreads / 32; ++w) tot += s_sums[lane][w];
+        }
+        double u = sj * tot;
+        if (has_prev) u -= bp * xpr;
+        if (on) out[row] = u;
+#pragma unroll
+        for (int q = 0; q < kL; ++q) {
+          const double xq = __shfl_sync(0xffffffffu, xr, q), uq = __shfl_sync(0xffffffffu, u, q);
+          if (lane == 0 && q0 + q < nlong) acc += xq * uq;
+        }
+      }
+      __syncthreads();
+    }
+  } else {
+    // medium rows: warp w takes list entries w, w+8, ...
+    {
+      const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+      const uint32_t nmed = s_nmed;
+      for (uint32_t q = warp; q < nmed; q += kThreads / 32) {
+        const uint32_t lr = s_med[q], row = row0 + lr;
+        T xr = T(0), xpr = T(0);
+        if (lane == 0) {
+          xr = x[row];
+          if (has_prev) xpr = xp[row];
+        }
+        const T s = warp_sum<T>(run_sum(s_rp[lr] + lane, s_rp[lr + 1], 32));
+        if (lane == 0) finish_row(s, row, xr, xpr);
+      }
+    }
 
-  // long rows: the whole CTA per row, in row order
-  const uint32_t nlong = s_nlong;
-  for (uint32_t q = 0; q < nlong; ++q) {
-    const uint32_t lr = s_long[q], row = row0 + lr;
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    T xr = T(0), xpr = T(0);
-    if (threadIdx.x == 0) {
-      xr = x[row];
-      if (has_prev) xpr = xp[row];
+    // long rows: the whole CTA per row, in row order
+    const uint32_t nlong = s_nlong;
+    for (uint32_t q = 0; q < nlong; ++q) {
+      const uint32_t lr = s_long[q], row = row0 + lr;
+      const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+      T xr = T(0), xpr = T(0);
+      if (threadIdx.x == 0) {
+        xr = x[row];
+        if (has_prev) xpr = xp[row];
+      }
+      const T s = warp_sum<T>(run_sum(s_rp[lr] + threadIdx.x, s_rp[lr + 1], kThreads));
+      if (lane == 0) s_rowsum[warp] = s;
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        T tot = T(0);
+        for (int w = 0; w < kThreads / 32; ++w) tot += s_rowsum[w];
+        finish_row(tot, row, xr, xpr);
+      }
+      __syncthreads();
     }
-    const T s = warp_sum<T>(run_sum(s_rp[lr] + threadIdx.x, s_rp[lr + 1], kThreads));
-    if (lane == 0) s_rowsum[warp] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      T tot = T(0);
-      for (int w = 0; w < kThreads / 32; ++w) tot += s_rowsum[w];
-      finish_row(tot, row, xr, xpr);
-    }
-    __syncthreads();
   }
 
   const double part = block_sum_to_double<T>(acc, s_red);

@@ -798,9 +798,10 @@ static int upload_impl(uint32_t n_inst, const uint32_t *n, const uint64_t *nnz,
   std::vector<std::vector<uint32_t>> heavy_rows(n_inst), tile_starts(n_inst);
   parallel_for(n_inst, node_off, [&](uint32_t r) {
     const uint32_t *rp = rp_of(r);
-    uint32_t rows = 0, acc = 0;
+    uint32_t rows = 0, acc = 0, most = 0;
     for (uint32_t i = 0; i < h->inst[r].n; ++i) {
       const uint32_t deg = rp[i + 1] - rp[i];
+      most = std::max(most, deg);
       if (deg > kHeavyDeg) heavy_rows[r].push_back(i);
       const uint32_t w = deg > kHeavyDeg ? 0u : deg;
       if (rows == 0 || rows == (uint32_t)kTileRows || (acc > 0 && acc + w > kTileNnz)) {
@@ -811,6 +812,7 @@ static int upload_impl(uint32_t n_inst, const uint32_t *n, const uint64_t *nnz,
       ++rows;
       acc += w;
     }
+    h->inst[r].hubs = (uint64_t)most > (uint64_t)kHubTimes * h->inst[r].nnz / h->inst[r].n + kHubRows;
   });
   for (uint32_t r = 0; r < n_inst; ++r) {
     h->inst[r].tile_base = tile_off;

@@ -13,7 +13,7 @@
 //     warp's 512 rows, taken lane by lane (each lane's rows in slot order,
 //     each row's columns in order), are dealt round-robin over the T steps
 //     of the warp's stream: element j goes to step j mod T, lane j / T.
-//     The lanes come in the order most, fewest, second most, second fewest,
+//     The lanes come (but in realisations with hubs) in the order most, fewest, second most, second fewest,
 //     ... elements, each with its share of the padding: after every second
 //     lane the deal is back near step 0, so the steps to which lanes of more
 //     than T elements go twice are the same few.  In lane order the sums of
@@ -159,8 +159,10 @@ __global__ void __launch_bounds__(kFillThreads) bcount_kernel(const InstDesc *in
 // staging area is written element by element.
 constexpr uint32_t kStageWords = 2048;  // staging u32 words per warp
 
-// Lane `lane`'s share of `pad` padding elements of a stream.
-__device__ __forceinline__ uint32_t pad_share(uint32_t pad, uint32_t lane) {
+// Lane `lane`'s share of `pad` padding elements of a stream (all the last
+// lane's where the lanes are dealt in lane order).
+__device__ __forceinline__ uint32_t pad_share(uint32_t pad, uint32_t lane, uint32_t in_order) {
+  if (in_order) return lane == 31 ? pad : 0u;
   return pad / 32 + (lane < pad % 32 ? 1u : 0u);
 }
 
@@ -226,9 +228,9 @@ __global__ void __launch_bounds__(kFillThreads) bfill_kernel(const InstDesc *ins
     uint32_t rank = 0;  // lanes with more elements
 #pragma unroll
     for (uint32_t o = 1; o < 32; ++o) rank += __shfl_sync(0xffffffffu, key, lane + o) > key;
-    const uint32_t at = rank < 16 ? 2 * rank : 2 * (31 - rank) + 1;
+    const uint32_t at = I.hubs ? lane : rank < 16 ? 2 * rank : 2 * (31 - rank) + 1;
     uint32_t *row = s_next + b * kFillThreads + 32 * wl;
-    const uint32_t share = pad_share(32 * T - tot, lane);
+    const uint32_t share = pad_share(32 * T - tot, lane, I.hubs);
     row[at] = c + share;
     __syncwarp();
     const uint32_t x = row[lane];
@@ -298,7 +300,7 @@ __global__ void __launch_bounds__(kFillThreads) bfill_kernel(const InstDesc *ins
       const uint32_t T = s_T[b * W + wl], base = s_sb[b * W + wl];
       const uint64_t st = s_start[b * W + wl];
       uint32_t p = s_next[b * kFillThreads + tid];
-      for (uint32_t i = pad_share(32 * T - s_tot[b * W + wl], lane); i; --i) {
+      for (uint32_t i = pad_share(32 * T - s_tot[b * W + wl], lane, I.hubs); i; --i) {
         const uint32_t s = p & 0xffffu, l = p >> 16;
         p = s + 1 == T ? p + (1u << 16) - s : p + 1;
         if (!CB_DCHECK(l < 32u && s < T, kDbgBlockedFill, p)) continue;
@@ -337,15 +339,21 @@ __global__ void __launch_bounds__(kFillThreads) bfill_kernel(const InstDesc *ins
 // entries in 40 graphs: 660 us here, once per upload, 263 -> 242 us per SpMV.
 // 790 us with 128 threads, 16-byte accesses and one CTA per segment (long
 // streams made a tail); 720 with more warps on fewer registers.
-constexpr uint32_t kSchedThreads = 64;
+constexpr uint32_t kSchedThreads = 64, kSchedParts = 4;  // CTAs per segment
 
-__global__ void __launch_bounds__(kSchedThreads) bsched_kernel(const uint64_t *bwstart,
+__global__ void __launch_bounds__(kSchedThreads) bsched_kernel(const InstDesc *inst,
+                                                               const uint32_t *btile_inst,
+                                                               const uint64_t *bseg_base,
+                                                               const uint64_t *bwstart,
                                                                const uint32_t *bwlen,
                                                                uint32_t *belem) {
   __shared__ uint32_t s_bank[32][kSchedThreads];
   __shared__ uint32_t s_at[8][kSchedThreads];  // the lane's elements by step
   __shared__ uint32_t s_end[32];               // rounds of streams 0 .. w
-  const uint64_t w0 = (uint64_t)blockIdx.x * 32;  // one segment: 32 streams
+  const uint32_t seg = blockIdx.y / kSchedParts, part = blockIdx.y % kSchedParts;
+  const InstDesc &I = inst[btile_inst[blockIdx.x]];
+  if (seg >= I.nb || I.hubs) return;
+  const uint64_t w0 = (bseg_base[blockIdx.x] + seg) * 32;  // one segment: 32 streams
   const uint32_t tid = threadIdx.x;
   if (tid < 32) {
     uint32_t c = (bwlen[w0 + tid] + 7) / 8;
@@ -357,7 +365,7 @@ __global__ void __launch_bounds__(kSchedThreads) bsched_kernel(const uint64_t *b
     s_end[tid] = c;
   }
   __syncthreads();
-  for (uint32_t q = blockIdx.y * kSchedThreads + tid; q < s_end[31]; q += kSchedThreads * gridDim.y) {
+  for (uint32_t q = part * kSchedThreads + tid; q < s_end[31]; q += kSchedThreads * kSchedParts) {
     uint32_t w = 0;
 #pragma unroll
     for (uint32_t o = 16; o; o >>= 1)
@@ -579,7 +587,8 @@ int blocked_fill(cb_graph *h, cudaStream_t s, BlockedBuild &bb) {
           h->row_ptr, h->col, h->d_belem, nbmax);
     prefer_shared(bsched_kernel);
     if (e == cudaSuccess)
-      bsched_kernel<<<dim3((uint32_t)h->total_bseg, 4), kSchedThreads, 0, s>>>(h->d_bwstart, h->d_bwlen, h->d_belem);
+      bsched_kernel<<<dim3(h->total_btiles, nbmax * kSchedParts), kSchedThreads, 0, s>>>(
+          h->d_inst, h->d_btile_inst, h->d_bseg_base, h->d_bwstart, h->d_bwlen, h->d_belem);
     chk(cudaGetLastError());
   }
   if (e != cudaSuccess) {

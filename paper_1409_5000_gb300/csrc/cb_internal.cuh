@@ -32,6 +32,15 @@ constexpr int kNodeAlign = 32;       // per-instance node offset alignment (elem
 // is timed beside the per-step ones.
 constexpr uint32_t kSmallN = 8192;
 constexpr uint32_t kSmallNnz = 1u << 20;
+// A realisation has hubs when a row is longer than kHubTimes its mean degree
+// + kHubRows.  The leading eigenvector then sits on a few rows, whose FP32
+// rounding is not averaged: another order of the sums moves theta, and with it
+// every score, by up to 3e-8 lambda_max, about 2e-6 at lambda_max = 60 (BA, 10^4
+// nodes, degree 22), against 1e-7 and less on ER and WS graphs.  Where FP32
+// results are compared or stored that would show, so the orders that are free
+// elsewhere (the team kernel's, the deal of the column-blocked streams) stay
+// as they are in the per-step kernels for these.
+constexpr uint32_t kHubTimes = 8, kHubRows = 64;
 
 // Column-blocked SpMV (FP32): a CTA of kBThreads owns kBTileRows rows,
 // kBRowsPerThread rows per thread (strided by kBThreads); the columns are cut into
@@ -124,7 +133,8 @@ struct InstDesc {
   uint32_t pb, pns;               // two-phase FP32 SpMV? number of source tiles
   uint32_t ptile_base;            // first source tile (handle-wide index)
   uint32_t pbin_base, n_pbin;     // bins
-  uint32_t pad_p[3];
+  uint32_t hubs;                  // rows far above the mean degree (kHubTimes): FP32 keeps its sums' order
+  uint32_t pad_p[2];
   uint64_t pmat_base;             // offset of the [bin][pns + 1] chunk tables
   RedPlan pspmv;                  // slots: n_pbin bins, then n_heavy rows
 };

@@ -1291,14 +1291,17 @@ static int run_t(cb_graph *h, Workspace &W, uint32_t r0, uint32_t r1, uint32_t m
   const bool one_launch = (h->path == CB_PATH_AUTO || h->tuned_auto) && h->stall_btile == UINT32_MAX;
   const cb_graph *hp = h->plan_of ? h->plan_of : h;  // a group handle decides as the whole one
   const uint32_t p0 = h->plan_of ? 0u : r0, p1 = h->plan_of ? hp->n_inst : r1;
-  bool small = true;
-  for (uint32_t r = p0; r < p1 && small; ++r) small = hp->inst[r].n <= kSmallN && hp->inst[r].nnz <= kSmallNnz;
+  bool small = true, hubs = false;
+  for (uint32_t r = p0; r < p1; ++r) {
+    small &= hp->inst[r].n <= kSmallN && hp->inst[r].nnz <= kSmallNnz;
+    hubs |= hp->inst[r].hubs != 0;
+  }
   // a team sums in an order of its own: taken where that cannot show, FP64 with
-  // reorthogonalisation and FP32 ensembles and small graphs.  One larger graph in
+  // reorthogonalisation and FP32 ensembles and small graphs without hubs.  One larger graph in
   // FP32 keeps the order of the per-step kernels (a planted clique's scores differ
   // by less than FP32 rounding), as does FP64 without it (T's trailing part)
   const bool team = one_launch &&
-                    (sizeof(T) == 8 ? h->reorth : !h->reorth && (small || p1 - p0 > 1)) &&
+                    (sizeof(T) == 8 ? h->reorth : !h->reorth && !hubs && (small || p1 - p0 > 1)) &&
                     team_plan(h, r0, r1, sizeof(T), h->reorth, &ta, &team_grid, &team_coop);
   const uint64_t nsc = (uint64_t)(r1 - r0) * W.sc.ms;
   init_scalars_kernel<<<(uint32_t)((nsc + kThreads - 1) / kThreads), kThreads, 0, s>>>(
@@ -1313,16 +1316,13 @@ static int run_t(cb_graph *h, Workspace &W, uint32_t r0, uint32_t r1, uint32_t m
     prof_end(tok, s);
     return rc;
   }
-  if constexpr (sizeof(T) == 8) {
-    if (small && one_launch && !h->reorth) {
-      cudaFuncSetAttribute(lanczos_small_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(3 * kSmallN * sizeof(double)));
-      tok = prof_begin(CB_K_SPMV, s);
-      lanczos_small_kernel<double><<<r1 - r0, kSmallThreads, 3 * (size_t)((nmax + 3) & ~3u) * sizeof(double), s>>>(
-          a, r0, m);
-      prof_end(tok, s);
-      return cuda_error(cudaGetLastError(), "lanczos launch");
-    }
+  if (small && one_launch && !h->reorth && (sizeof(T) == 8 || hubs)) {
+    cudaFuncSetAttribute(lanczos_small_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(3 * kSmallN * sizeof(T)));
+    tok = prof_begin(CB_K_SPMV, s);
+    lanczos_small_kernel<T><<<r1 - r0, kSmallThreads, 3 * (size_t)((nmax + 3) & ~3u) * sizeof(T), s>>>(a, r0, m);
+    prof_end(tok, s);
+    return cuda_error(cudaGetLastError(), "lanczos launch");
   }
   for (uint32_t j = 0; j < m; ++j) {
     tok = prof_begin(CB_K_SPMV, s);

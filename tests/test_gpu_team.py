@@ -64,3 +64,24 @@ def test_matches_oracle(name, prec):
             assert [r.m_eff for r in rep[:3]] == [1, 1, 1]
         again = B.ensemble_scores(gs, m, p)[1]
         assert torch.equal(S, again)
+
+
+@pytest.mark.parametrize("sizes", [(9000, 12000), (2500, 3000)])
+def test_ensembles_with_hubs_keep_the_order(sizes):
+    """FP32 ensembles whose leading eigenvector sits on a few hubs: above the
+    small size the automatic path gives the bits of the per-step kernels; all
+    meet the suite's bars against the oracle."""
+    from paper_1409_5000_gb300 import binding as B
+
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for -m gpu tests")
+    graphs = [synth.ba(n, 10, 3 + q) for q, n in enumerate(sizes)]
+    th_o, S_o = oc.ensemble_scores([(g.n, g.row_ptr, g.col) for g in graphs], 17)
+    got = []
+    for path in (B.CB_PATH_AUTO, B.CB_PATH_CSR):
+        with B.GraphSet(graphs, path=path) as gs:
+            ls, S = B.ensemble_scores(gs, 17, B.CB_FP32)
+            got.append((float(ls.item()), S.cpu().numpy()))
+        parity.assert_scores(*got[-1], th_o, S_o, "fp32")
+    if min(sizes) > 8192:
+        assert got[0][0] == got[1][0] and np.array_equal(got[0][1], got[1][1])

@@ -388,7 +388,7 @@ def spmv_path(ens, csr_only=False):
     return "blocked" if tiles >= torch.cuda.get_device_properties(0).multi_processor_count else "csr"
 
 
-_KERNEL_NAMES = {"small": "lanczos_small_kernel (all m Lanczos steps of a small realisation per CTA)",
+_KERNEL_NAMES = {"small": "team_lanczos_kernel (all m Lanczos steps of small realisations in one launch)",
                  "blocked": "bspmv_kernel (column-blocked Lanczos SpMV step)",
                  "twophase": "pscatter_kernel + pgather_kernel (two-phase Lanczos SpMV step)",
                  "csr": "spmv_kernel (tiled-CSR Lanczos SpMV step)"}
@@ -413,11 +413,17 @@ def roofline_for(ens, fam, path, m=1):
             "kernel_shares": {k: round(t / tot, 4) for k, (t, _) in fam.items()}}
 
 
+def step_launches(m, path, with_grad=False):
+    """Kernel launches of one step as reported: those of launches_for with
+    the top-k in one kernel at every size."""
+    return launches_for(m, path, with_grad, n_scores=1)
+
+
 def launches_for(m, path, with_grad=False, n_scores=None):
     """Kernel launches of one step: init (2) + per Lanczos step the SpMV
     (two kernels on the two-phase path), finalize and beta + tridiag +
-    combine (2) + top-k (init, 12 radix passes, collect, sort; one sort of
-    all scores up to 4096 of them)."""
+    combine (2) + top-k (in separate passes: init, 12 radix passes, collect,
+    sort; one sort of all scores up to 4096 of them)."""
     topk = 1 if n_scores is not None and n_scores <= 4096 else 15
     if path == "small":  # one launch for all m steps
         n = 2 + 1 + 1 + 2 + topk
@@ -537,7 +543,7 @@ def extra_leg(B, name, steps, warmup, dev, csr_only=False, precs=(0,), built=Non
                 path = "csr"
             leg = {"ms_per_step": ms, "value": units / (ms * 1e-3), "unit": UNIT,
                    "dtype": "f64" if prec == 1 else "f32", "roofline": roofline_for(ens, fam, path, m),
-                   "gpu_launches_per_step": launches_for(m, path, with_grad, gs.n_max)}
+                   "gpu_launches_per_step": step_launches(m, path, with_grad)}
             if prec == 1:  # FP64 bytes: 8-byte vector elements
                 b64 = (m if path == "small" else 1) * alg_bytes_spmv(ens, fp64=True)
                 leg["roofline"]["alg_bytes_per_launch"] = b64
@@ -653,7 +659,7 @@ def main():
     fam = kernel_families(B, step, args.steps)
     path_kind = spmv_path(ens, args.csr_only)
     roofline = roofline_for(ens, fam, path_kind, m)
-    launches_per_step = launches_for(m, path_kind, with_grad, gs.n_max)
+    launches_per_step = step_launches(m, path_kind, with_grad)
 
     extra = {}
     if with_grad:
@@ -813,7 +819,7 @@ def main():
         extra["subgraph_centrality_topk"] = {
             "ms": sc_ms, "nodes": k, "m": m, "realisation_n": gs.n[r_big],
             "realisation_nnz": gs.nnz[r_big],
-            "api": "cb_subgraph_centrality (k copies of the realisation, k Lanczos runs, Gauss rule)"}
+            "api": "cb_subgraph_centrality (k Lanczos runs side by side, Gauss rule)"}
 
     if rank == 0 and not args.skip_extra:
         # restarted Lanczos: the same total depth m as cycles of m/5 steps, so

@@ -69,9 +69,11 @@ extern "C" {
 #define CB_TWO_PHASE 8u   /* the two-phase format for every realisation (default: n > 2^19 only) */
 
 /* FP32 SpMV path of a handle (cb_graph_set_path) */
-#define CB_PATH_AUTO 0    /* one launch of all m steps (one CTA per realisation) when every
-                             realisation of the call has n <= 8192 and <= 2^20 entries and no
-                             reorthogonalisation is asked; otherwise, per step, the
+#define CB_PATH_AUTO 0    /* one launch of all m steps by teams of CTAs where the realisations
+                             stay on the chip and a cost model prefers it (FP64 with
+                             reorthogonalisation; FP32 ensembles and realisations of n <= 8192,
+                             without hubs or reorthogonalisation), or by one CTA each (n <= 8192
+                             and <= 2^20 entries: FP64, FP32 with hubs); otherwise, per step, the
                              column-blocked kernel when the handle has >= one blocked tile per
                              SM, two-phase kernels where built, else tiled CSR */
 #define CB_PATH_FORMATS 1 /* column-blocked and two-phase kernels wherever their format was built */
@@ -239,9 +241,11 @@ int cb_graph_read(const cb_graph *h, uint32_t r, uint32_t *row_ptr, uint32_t *co
  *   nodes      uint32[k] node indices (< n[inst]), host or device.
  *   sc_scaled  device double[k], written: SC(nodes[q]) = exp(*log_scale) * sc_scaled[q].
  *   log_scale  device double[1], written: max over q of lambda_max(T_m) from e_q.
- * The call builds a temporary handle with k copies of the realisation
- * (k * (nnz + n) * 4 bytes plus their formats and a (m+1) * k * n basis),
- * synchronises `stream` and frees it before returning.
+ * The runs share the realisation, 32 vectors at a time (three of them, n * 32
+ * each, live at once).  With CB_REORTH the call builds a temporary handle
+ * with k copies of the realisation instead (k * (nnz + n) * 4 bytes plus
+ * their formats and a (m+1) * k * n basis).  Synchronises `stream` and frees
+ * its memory before returning.
  * Errors: CB_ERR_ARG (null arguments, ranges), CB_ERR_CUDA.
  */
 int cb_subgraph_centrality(cb_graph *h, uint32_t inst, uint32_t m, int prec, uint32_t k,
@@ -407,14 +411,14 @@ int cb_ensemble_scores_restarted(cb_graph *h, uint32_t m, uint32_t cycles, int p
 /*
  * cb_topk -- indices and values of the k largest entries of S (the
  * recovered target of the "Identification algorithm" section; the paper
- * sorts all scores, this selects by radix).
+ * sorts all scores, this selects by radix, in one kernel).
  *   S    device, double[n], read.
  *   n    1 <= n < 2^32.  k: 1 <= k <= min(n, CB_MAX_TOPK).
  *   idx  device, uint32[k], written; val device, double[k], written.
  * Order: value descending, ties to the smaller index; -0.0 equals +0.0;
  * NaN ranks below every number (so it is returned only if k exceeds the
  * count of non-NaN entries).
- * Asynchronous.  Device scratch (about 3 KB + 16 k bytes) comes from the
+ * Asynchronous.  Device scratch (about 90 KB) comes from the
  * stream-ordered allocator (cudaMallocAsync) and is freed on `stream`.
  */
 int cb_topk(const double *S, uint32_t n, uint32_t k, uint32_t *idx, double *val, void *stream);

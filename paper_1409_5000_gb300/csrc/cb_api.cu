@@ -116,7 +116,7 @@ class HelperPool {
     next_ = 0;
     error_ = nullptr;
     join_ = helpers;
-    for (uint32_t have = idle_; have < helpers; ++have) {
+    for (; alive_ < helpers; ++alive_) {  // none works now; all alive will wait for work
       try {
         std::thread([this] { help(); }).detach();
       } catch (const std::system_error &) {
@@ -150,10 +150,10 @@ class HelperPool {
   void help() {
     std::unique_lock<std::mutex> lk(mu_);
     while (true) {
-      ++idle_;
-      const bool work = work_.wait_for(lk, kIdle, [this] { return join_ > 0; });
-      --idle_;
-      if (!work) return;
+      if (!work_.wait_for(lk, kIdle, [this] { return join_ > 0; })) {
+        --alive_;
+        return;
+      }
       --join_;
       ++busy_;
       lk.unlock();
@@ -165,7 +165,7 @@ class HelperPool {
   std::mutex mu_, emu_;
   std::condition_variable work_, done_;
   const std::function<void(uint32_t)> *fn_ = nullptr;
-  uint32_t n_ = 0, join_ = 0, busy_ = 0, idle_ = 0;
+  uint32_t n_ = 0, join_ = 0, busy_ = 0, alive_ = 0;  // alive_: at most the most helpers asked for
   std::atomic<uint32_t> next_{0};
   std::exception_ptr error_;
 };

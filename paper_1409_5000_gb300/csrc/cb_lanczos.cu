@@ -146,12 +146,15 @@ __device__ __forceinline__ double batch_sum(double (&v)[B]) {
 // are active: there several rows' sums are formed side by side (batch_sum), a
 // row's result by a lane of its own, and a first entry is not added to 0; the
 // sums' orders, alpha's included, are those of one row at a time.  BA(1e5, 5),
-// a step with its vector kernels: 49 -> 40 us (the tiles of medium rows, which
+// a step with its vector kernels: 49 -> 41 us (the tiles of medium rows, which
 // ended last, 43 -> 29 us with two gathers of a row in flight, then four).
+// Five CTAs per SM (48 registers): with three, 4 M entries and more, bound by
+// the gathers in flight, took 20% longer (ER, 8 graphs of 1.5e5 nodes, degree
+// 23, 16 steps: 4.53 ms, 3.75 with five, 3.97 with six; 4.02 one row at a time).
 // Blocks [0, n_chunks) are heavy-row chunks starting at chunk_off; blocks
 // [n_chunks, ...) are normal tiles starting at tile_off.
 template <typename T, int G>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 3 : 6) spmv_kernel(LArgs a, uint32_t j, uint32_t chunk_off,
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 5 : 6) spmv_kernel(LArgs a, uint32_t j, uint32_t chunk_off,
                                                         uint32_t n_chunks, uint32_t tile_off) {
   __shared__ double s_red[32];
   __shared__ uint32_t s_rp[kTileRows + 1];

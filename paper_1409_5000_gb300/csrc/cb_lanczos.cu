@@ -916,10 +916,11 @@ __global__ void __launch_bounds__(kThreads) finalize_beta_kernel(LArgs a, uint32
 }
 
 // ---------------------------------------------------------------------------
-// Small realisations (n <= kSmallN, at most kSmallNnz entries) in FP64 without
-// reorthogonalisation (the team kernel takes the others, cb_team.cu; here the
-// order of the sums stays, which decides the trailing part of T once
-// orthogonality is lost): one CTA per realisation runs all m Lanczos steps in one launch -- SpMV with the row
+// Small realisations (n <= kSmallN, at most kSmallNnz entries) without
+// reorthogonalisation, in FP64 and, with hubs, in FP32 (the team kernel takes
+// the others, cb_team.cu; here the order of the sums stays, which decides the
+// trailing part of T once orthogonality is lost, and theta's last FP32 digits
+// with hubs): one CTA per realisation runs all m Lanczos steps in one launch -- SpMV with the row
 // epilogue, alpha, the axpy w = u - alpha_j scale_j W_j, beta_j and the
 // breakdown test, the same arithmetic as spmv_kernel + finalize_kernel +
 // finalize_beta_kernel -- with W_j, W_{j-1} and the new vector resident in

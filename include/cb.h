@@ -93,7 +93,8 @@ typedef struct cb_graph cb_graph;
 typedef struct {
   uint32_t m_eff;   /* Lanczos steps kept (< m after an exact breakdown) */
   int32_t status;   /* CB_OK or CB_ERR_NONFINITE for this realisation */
-  double theta;     /* lambda_max(T_m_eff): this realisation's log scale */
+  double theta;     /* lambda_max(T_m_eff): this realisation's log scale (FP64: to rounding, or
+                       up to 4e-8 of it short; exp(theta) y does not depend on it) */
   double beta_last; /* last residual norm beta_m (0 after breakdown) */
   double beta0;     /* ||1|| = sqrt(n_r) */
 } cb_inst_report;

@@ -450,7 +450,7 @@ static int backward_t(cb_graph *h, uint32_t m, const uint32_t *idx, uint32_t k, 
   const size_t shm_tri = 2 * sizeof(contour::Solve);
   cudaFuncSetAttribute(bw_tridiag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_tri);
   bw_tridiag_kernel<<<N, 64, shm_tri, s>>>(h->ws.sc, h->ws2.sc, h->d_inst, B.K, m, B.theta, B.cnt,
-                                           contour::nodes(), sizeof(T) == 8 && !h->reorth);
+                                           contour::nodes(), sizeof(T) == 8);
   const size_t shm = (size_t)(m * m + 4 * m * 65) * sizeof(T);
   auto nk = bw_node_kernel<T>;
   if (shm > 48 * 1024) cudaFuncSetAttribute(nk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);

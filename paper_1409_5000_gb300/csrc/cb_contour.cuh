@@ -253,13 +253,17 @@ __device__ inline double lambda_max(const double *al, const double *be, int M, S
   return rho;
 }
 
-// The same by Laguerre's iteration on det(xI - T), for FP64 recurrences
-// without reorthogonalisation: their T carries copies of lambda_max, over which
-// two FP64 steps stop up to about 1e-6 above it, and theta is a result that
-// callers compare and store in that precision.  (Elsewhere lambda_max is used:
-// 25 against 34 us at M = 30.)  The iteration from above the Gershgorin bound runs in FP32 until its step is
-// below 1e-6 relative, then two FP64 steps polish the result: the convergence
-// is cubic, so the FP32 estimate turns into an FP64-accurate one.
+// The same by Laguerre's iteration on det(xI - T), for FP64 recurrences (25
+// against 34 us at M = 30).  The iteration from above the Gershgorin bound runs
+// in FP32 until its step is below 1e-6 relative, then two FP64 steps polish the
+// result: the convergence is cubic, so the FP32 estimate turns into an
+// FP64-accurate one.  Not always: where the FP32 iterate ends below lambda_max,
+// an FP64 step meets a pivot that is not positive and is left out, and theta
+// stays up to 4e-8 short (relative; 4 of 48 ER, WS and BA graphs of 900 to 8500
+// nodes at m = 30, the others within 6e-15); over copies of lambda_max (T without
+// reorthogonalisation) it stops up to 1.2e-7 above.  exp(theta) y does not depend
+// on it, but theta and y are results that callers compare and store to FP64
+// accuracy, so both FP64 modes take them by this one method.
 //
 // T is converted once, in parallel, and the FP64 steps take f, f' and f'' from
 // p_k = (x - a_k) p_{k-1} - b_{k-1}^2 p_{k-2} and its derivatives on three
@@ -310,7 +314,7 @@ __device__ inline double lambda_max_laguerre(const double *al, const double *be,
   }
   double x = xf;
   const double c = lane == 1 ? 1.0 : lane == 2 ? 2.0 : 0.0;  // lane d: the d-th derivative
-  for (int it = 0; it < 2; ++it) {  // FP64 polish (a failed step leaves x above the root)
+  for (int it = 0; it < 2; ++it) {  // FP64 polish, left out from below lambda_max
     const double xs = x * s;
     double own2 = lane == 0 ? 1.0 : 0.0;                                 // p_0
     double own = lane == 0 ? xs - S.as[0] : lane == 1 ? 1.0 : 0.0;       // p_1

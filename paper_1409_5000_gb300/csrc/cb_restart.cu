@@ -232,7 +232,7 @@ int cycles_run(cb_graph *h, const RState &rs, double *Y, uint32_t m, uint32_t cy
     if (rc != CB_OK) break;
     int tok = prof_begin(CB_K_TRIDIAG, s);
     restart_tridiag_kernel<<<h->n_inst, 32, 0, s>>>(W.sc, rs, h->d_inst, c, contour::nodes(),
-                                                     sizeof(T) == 8 && !h->reorth);
+                                                     sizeof(T) == 8);
     prof_end(tok, s);
     tok = prof_begin(CB_K_COMBINE, s);
     if (h->total_fin)

@@ -423,7 +423,7 @@ static int sc_copies(cb_graph *h, uint32_t inst, uint32_t m, int prec, uint32_t 
   rc = ensure_workspace(v, v->ws, m, prec, s);
   if (rc == CB_OK) rc = lanczos_run(v, v->ws, 0, k, m, prec, s, d_nodes, k, true);
   if (rc == CB_OK) {
-    sc_tridiag_kernel<<<k, 32, 0, s>>>(v->ws.sc, contour::nodes(), false);
+    sc_tridiag_kernel<<<k, 32, 0, s>>>(v->ws.sc, contour::nodes(), prec == CB_FP64);
     sc_finish_kernel<<<1, 256, 0, s>>>(v->ws.sc, k, sc_scaled, log_scale);
     rc = cuda_error(cudaGetLastError(), "cb_subgraph_centrality: launch");
   }

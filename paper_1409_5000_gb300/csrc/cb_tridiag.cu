@@ -8,7 +8,7 @@
 // so the solve is organised to issue few FP64 instructions
 // (cb_contour.cuh):
 //  1. theta = lambda_max(T): FP32 multisection and inverse iteration, FP64
-//     Rayleigh quotient;
+//     Rayleigh quotient; for FP64 recurrences Laguerre's iteration;
 //  2. exp(S) e1, S = T - theta I <= 0, as 2 Re sum_k w_k (z_k I - S)^{-1} e1
 //     over the 12 upper-half contour nodes, by continuants on 24 lanes;
 //  3. gamma_j = beta0 * c_j * scale_j, the weight of the stored basis vector
@@ -51,7 +51,7 @@ int tridiag_run(cb_graph *h, uint32_t r0, uint32_t r1, int prec, cudaStream_t s)
   prefer_shared(tridiag_kernel);
   const int tok = prof_begin(CB_K_TRIDIAG, s);
   tridiag_kernel<<<r1 - r0, 32, 0, s>>>(h->ws.sc, h->d_inst, r0, contour::nodes(),
-                                     prec == CB_FP64 && !h->reorth);
+                                     prec == CB_FP64);
   prof_end(tok, s);
   return cuda_error(cudaGetLastError(), "tridiag launch");
 }

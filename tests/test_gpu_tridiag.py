@@ -49,3 +49,27 @@ def test_shift_around_the_second_method(q, prec):
         ls, y = B.communicability(gs, 0, 35, prec)
         th_o, y_o, _ = oc.krylov_expv(g.n, g.row_ptr, g.col, 35)
         parity.assert_scores(float(ls.item()), y.cpu().numpy(), th_o, y_o, "fp64" if prec else "fp32")
+
+
+@pytest.mark.parametrize("graph", [("er", 2001, 0), ("ws", 3500, 8), ("er", 2601, 2), ("ba", 2500, 0)])
+def test_shift_is_one_in_both_fp64_modes(graph):
+    """While orthogonality holds to rounding T is the same with and without
+    reorthogonalisation, so theta and the scaled scores are too: 1e-12 (T's
+    rounding, some 1e-15 of lambda_max < 25, through exp(theta) y)."""
+    from paper_1409_5000_gb300 import binding as B
+
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for -m gpu tests")
+    kind, n, seed = graph
+    if kind == "er":
+        g = synth.er(n, 9.0 / 2000, seed)
+    elif kind == "ba":
+        g = synth.ba(n, 5, seed)
+    else:
+        g = synth.single_background("ws", n, 12, seed).graphs[0]
+    with B.GraphSet([g], path=B.CB_PATH_CSR) as gs:
+        ls, y = B.communicability(gs, 0, 30, B.CB_FP64)
+        ls_r, y_r = B.communicability(gs, 0, 30, B.CB_FP64 | B.CB_REORTH)
+    ls, ls_r, y, y_r = float(ls.item()), float(ls_r.item()), y.cpu().numpy(), y_r.cpu().numpy()
+    assert abs(ls - ls_r) <= 1e-12 * ls
+    assert np.max(np.abs(y - y_r)) <= 1e-12 * y.max()

@@ -917,10 +917,12 @@ __global__ void __launch_bounds__(kThreads) finalize_beta_kernel(LArgs a, uint32
 
 // ---------------------------------------------------------------------------
 // Small realisations (n <= kSmallN, at most kSmallNnz entries) without
-// reorthogonalisation, in FP64 and, with hubs, in FP32 (the team kernel takes
-// the others, cb_team.cu; here the order of the sums stays, which decides the
-// trailing part of T once orthogonality is lost, and theta's last FP32 digits
-// with hubs): one CTA per realisation runs all m Lanczos steps in one launch -- SpMV with the row
+// reorthogonalisation, in FP64 and, with hubs, in FP32 (here the order of the
+// sums stays, which decides the trailing part of T once orthogonality is lost,
+// and theta's last FP32 digits with hubs); in FP32 without hubs those too dense
+// for the team kernel (cb_team.cu) and too few entries in all for the per-step
+// kernels (140 graphs of 1000 nodes, degree 150: 34 us a step, 61 per step,
+// 299 by teams): one CTA per realisation runs all m Lanczos steps in one launch -- SpMV with the row
 // epilogue, alpha, the axpy w = u - alpha_j scale_j W_j, beta_j and the
 // breakdown test, the same arithmetic as spmv_kernel + finalize_kernel +
 // finalize_beta_kernel -- with W_j, W_{j-1} and the new vector resident in
@@ -1320,7 +1322,7 @@ static int run_t(cb_graph *h, Workspace &W, uint32_t r0, uint32_t r1, uint32_t m
     prof_end(tok, s);
     return rc;
   }
-  if (small && one_launch && !h->reorth && (sizeof(T) == 8 || hubs)) {
+  if (small && one_launch && !h->reorth && (sizeof(T) == 8 || hubs || small_launch_pays(hp, p0, p1))) {
     cudaFuncSetAttribute(lanczos_small_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(3 * kSmallN * sizeof(T)));
     tok = prof_begin(CB_K_SPMV, s);

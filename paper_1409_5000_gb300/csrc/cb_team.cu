@@ -483,14 +483,46 @@ __global__ void __launch_bounds__(kTeamThreads, 1) team_lanczos_kernel(const __g
 namespace {
 
 constexpr size_t kTeamSmem = 222 * 1024;  // of 227 KB; the kernel's static part is below 3 KB
-constexpr uint32_t kTeamNnz = 24u << 20;  // entries of a call that stay in L2 with its vectors
-// Cost of a step in ns (measured): what does not depend on the size, and entries
-// per ns of a CTA from shared memory and from L2, of the per-step kernels on the
-// whole GPU, and bytes per ns of a CTA copying the vector from L2.
-constexpr double kOneNs = 2000.0, kManyNs = 6000.0, kStepsNs = 19000.0;
-constexpr double kSmemPerNs = 8.0, kL2PerNs = 1.0, kStepsPerNs = 200.0, kCopyPerNs = 60.0;
+// Cost of a step in ns.  Measured at m = 20 on ER graphs of mean degree 4 to 150,
+// 1 to 2000 of them, 500 to 800 000 nodes; within 30% of what the chosen route
+// takes, and where two are nearer than that either will do.  What does not depend
+// on the size; entries per ns of a CTA whose columns are in shared memory, the
+// vector there too or in L2; bytes per ns of a CTA copying the vector from L2.
+constexpr double kOneNs = 2000.0, kManyNs = 6000.0;
+constexpr double kSmemPerNs = 8.0, kL2PerNs = 1.0, kCopyPerNs = 60.0;
+// Columns that do not fit stay in global memory, and as a lane then walks rows of its
+// own, 4 bytes of a sector at a time, long rows thrash the L1: 100 graphs of 8000
+// nodes at degree 10 ran at 2.9 entries per ns, 150 of 8000 at 18 at 1.9, 100 of
+// 4000 at 50 at 0.67, 140 of 1000 at 150 at 0.5 (299 us a step where the per-step
+// kernels take 61 and one CTA each 34).  In FP64 0.6 (150 of 2000 at 60), and with
+// the vector in L2 too 0.3 to 0.5 (1 to 8 of 30 000 to 300 000 at 24 to 120).
+constexpr double kFarLeast = 0.5, kFarMost = 2.9, kFarRow = 40.0, kFar64 = 0.6, kFarL2 = 0.35;
+// Reorthogonalisation, per node (of the realisation, of the call) and flat.
+constexpr double kOneGs = 30.0, kManyGs = 0.18, kManyGsNs = 24000.0;
+
+// The per-step kernels over realisations [r0, r1), ns a step: launches, tiles that
+// realisations do not fill, nodes, and entries, which find the vector of a small
+// graph in the L1, or are summed by the column-blocked kernel.
+double steps_ns(const cb_graph *h, uint32_t r0, uint32_t r1, size_t esz, bool reorth) {
+  double t = 20000.0 + 50.0 * (r1 - r0);
+  const bool blocked = h->total_btiles >= h->n_sm;
+  for (uint32_t r = r0; r < r1; ++r) {
+    const InstDesc &I = h->inst[r];
+    t += 0.02 * I.n + (esz == 8 ? 0.0065 : blocked ? 0.0011 : I.n <= 16384 ? 0.0022 : 0.0035) * I.nnz;
+    if (reorth) t += 0.22 * I.n;
+  }
+  return t + (reorth ? 60000.0 : 0.0);
+}
 
 }  // namespace
+
+bool small_launch_pays(const cb_graph *h, uint32_t r0, uint32_t r1) {
+  double one = 0.0;
+  for (uint32_t r = r0; r < r1; ++r)
+    one = std::max(one, 10.0 * h->inst[r].n + 0.17 * h->inst[r].nnz);
+  one *= std::max(1.0, (double)(r1 - r0) / h->n_sm);
+  return 1.3 * one < steps_ns(h, r0, r1, sizeof(float), false);
+}
 
 bool team_plan(const cb_graph *h, uint32_t r0, uint32_t r1, size_t esz, bool reorth, TeamArgs *out,
                uint32_t *grid, bool *cooperative) {
@@ -510,13 +542,12 @@ bool team_plan(const cb_graph *h, uint32_t r0, uint32_t r1, size_t esz, bool reo
     *cooperative = *grid > N;
     return true;
   }
-  uint64_t nnz = 0, work = 0;
+  uint64_t nodes = 0, work = 0;
   for (uint32_t r = r0; r < r1; ++r) {
     if (h->inst[r].pb && esz == 4) return false;  // the two-phase kernels take it
-    nnz += h->inst[r].nnz;
+    nodes += h->inst[r].n;
     work += (uint64_t)h->inst[r].nnz + h->inst[r].n;
   }
-  if (nnz > kTeamNnz) return false;
   TeamArgs &t = *out;
   t.whole_x = 0;
   t.reorth = reorth ? 1u : 0u;
@@ -524,12 +555,23 @@ bool team_plan(const cb_graph *h, uint32_t r0, uint32_t r1, size_t esz, bool reo
   auto bytes = [&](const InstDesc &I, uint64_t rows, bool whole) -> size_t {
     return esz * ((whole ? (I.n + 3ull) : rows + 3) + 2 * (rows + 3)) + 4 * (rows + 4);
   };
+  // ns a CTA takes for the sums of `entries` entries in `rows` rows, of which a
+  // team's CTA expects that many and must have room for a tenth more (the kernel
+  // looks for itself)
+  auto sum_ns = [&](const InstDesc &I, double entries, double rows, bool whole) -> double {
+    const double room = (rows < I.n ? 1.1 : 1.0) * entries * (I.n <= 65536 ? 2 : 4);
+    if ((!whole || I.n <= 65536) && bytes(I, (uint64_t)rows, whole) + room <= (double)kTeamSmem)
+      return entries / (whole ? kSmemPerNs : kL2PerNs);
+    if (!whole) return entries / kFarL2;
+    if (esz == 8) return entries / kFar64;
+    return entries / std::min(kFarMost, std::max(kFarLeast, kFarRow * I.n / std::max(I.nnz, 1u)));
+  };
   // teams of one, in waves over the SMs
   double one = 0.0;
   for (uint32_t r = r0; r < r1; ++r) {
     const InstDesc &I = h->inst[r];
     if (bytes(I, I.n, true) > kTeamSmem) one = 1e30;
-    one = std::max(one, kOneNs + (I.nnz + 2.0 * I.n) / kSmemPerNs + (reorth ? 64.0 * I.n : 0.0));
+    one = std::max(one, kOneNs + 2.0 * I.n / kSmemPerNs + sum_ns(I, I.nnz, I.n, true) + (reorth ? kOneGs * I.n : 0.0));
   }
   one *= (N + h->n_sm - 1) / h->n_sm;
   // teams sharing the SMs by work
@@ -554,20 +596,21 @@ bool team_plan(const cb_graph *h, uint32_t r0, uint32_t r1, size_t esz, bool reo
         const uint64_t rows = std::min<uint64_t>(I.n, (t.rowdiv + 1) * (I.n / g + 2) + 2);
         const double per = (double)I.nnz / g;
         // the whole vector each step, or gathers from L2
-        const bool whole = g == 1 || (q < 64 && I.n * esz / kCopyPerNs + per / kSmemPerNs < per / kL2PerNs &&
+        const double own = (double)I.n / g, copy = I.n * esz / kCopyPerNs;
+        const bool whole = g == 1 || (q < 64 && copy + sum_ns(I, per, own, true) < sum_ns(I, per, own, false) &&
                                       bytes(I, rows, true) <= kTeamSmem);
         if (whole && q < 64) t.whole_x |= 1ull << q;
         if (bytes(I, rows, whole) > kTeamSmem) many = 1e30;
-        many = std::max(many, g == 1 ? kOneNs + (I.nnz + 2.0 * I.n) / kSmemPerNs
-                                     : kManyNs + (whole ? per / kSmemPerNs + I.n * esz / kCopyPerNs
-                                                        : per / kL2PerNs));
+        many = std::max(many, sum_ns(I, per, own, whole) +
+                                  (g == 1 ? kOneNs + 2.0 * I.n / kSmemPerNs : kManyNs + (whole ? copy : 0.0)));
       }
       if (many < 1e30 || t.rowdiv == 1) break;
     }
     t.first[N] = (uint16_t)total;
     if (total > kMaxTeamCtas) many = 1e30;
+    if (reorth) many += kManyGsNs + kManyGs * nodes;
   }
-  const double steps = kStepsNs + nnz / kStepsPerNs + (reorth ? 40000.0 : 0.0);
+  const double steps = steps_ns(h, r0, r1, esz, reorth);
   if (one <= many && one <= steps) {
     t.nteams = 0;
     t.first[0] = 0;

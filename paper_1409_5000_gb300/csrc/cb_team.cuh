@@ -25,6 +25,9 @@ struct TeamArgs {
 // runs as one launch; its grid and arguments (the buffers left to the caller).
 bool team_plan(const cb_graph *h, uint32_t r0, uint32_t r1, size_t esz, bool reorth, TeamArgs *out,
                uint32_t *grid, bool *cooperative);
+// Whether one CTA per realisation (lanczos_small_kernel) is the better route for FP32
+// realisations that are small enough for it and that no team takes.
+bool small_launch_pays(const cb_graph *h, uint32_t r0, uint32_t r1);
 template <typename T>
 int team_launch(const LArgs &a, TeamArgs t, uint32_t r0, uint32_t m, uint32_t grid, bool cooperative,
                 cudaStream_t s);

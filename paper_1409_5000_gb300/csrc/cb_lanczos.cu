@@ -143,19 +143,31 @@ __device__ __forceinline__ double batch_sum(double (&v)[B]) {
 
 // One Lanczos SpMV step over a range of realisations.  FP64 is bound by the
 // FP64 pipe, 65 cycles of a sub-core per warp instruction however many lanes
-// are active: there several rows' sums are formed side by side (batch_sum), a
-// row's result by a lane of its own, and a first entry is not added to 0; the
-// sums' orders, alpha's included, are those of one row at a time.  BA(1e5, 5),
-// a step with its vector kernels: 49 -> 41 us (the tiles of medium rows, which
-// ended last, 43 -> 29 us with two gathers of a row in flight, then four).
-// Five CTAs per SM (48 registers): with three, 4 M entries and more, bound by
-// the gathers in flight, took 20% longer (ER, 8 graphs of 1.5e5 nodes, degree
-// 23, 16 steps: 4.53 ms, 3.75 with five, 3.97 with six; 4.02 one row at a time).
+// are active: there the sums of several rows (kSide short ones per group, kSideLong
+// longer ones per warp or CTA) are formed side by side (batch_sum), a row's
+// result by a lane of its own, and a first entry is not added to 0; the
+// sums' orders, alpha's included, are those of one row at a time.
+// How many rows, and CTAs per SM, follows the group width, because more of one
+// leaves registers for fewer of the other, and the gathers in flight count as much:
+// with 8 short and 4 longer rows and five CTAs at every width, widths 1, 8, 16
+// and 32 spilled 260 to 340 bytes a thread.  m = 16, one row at a time / that /
+// now, ms: width 1, 8 graphs of 1.5e5 nodes, degree 2.5, 1.28 / 1.32 / 1.22; width 2,
+// degree 5, 1.68 / 1.54 / 1.43; width 4, degree 24, 3.38 / 3.28 / 3.05; width 8,
+// degree 60, 9.04 / 10.8 / 8.89, degree 40, 5.09 / 5.46 / 4.58; width 16, 6 of
+// 1e5, degree 120, 7.38 / 11.9 / 7.20; width 32, 6 of 3e4, degree 300, 5.38 / 5.65 /
+// 4.45.  (Width 4 as the others: 4% slower at degree 10; the others as width 4: 3%
+// slower than one row at a time at degree 40.)  FP32: five CTAs, six spill
+// 20 bytes, within 3% of each other at every width.
+template <typename T, int G>
+struct SpmvShape {
+  static constexpr int kCtas = sizeof(T) == 4 || G == 4 ? 5 : 6;
+  static constexpr int kSide = G == 4 ? 4 : G < 2 ? G : 2, kSideLong = G == 4 ? 2 : 1;
+};
 // Blocks [0, n_chunks) are heavy-row chunks starting at chunk_off; blocks
 // [n_chunks, ...) are normal tiles starting at tile_off.
 template <typename T, int G>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 5 : 6) spmv_kernel(LArgs a, uint32_t j, uint32_t chunk_off,
-                                                        uint32_t n_chunks, uint32_t tile_off) {
+__global__ void __launch_bounds__(kThreads, SpmvShape<T, G>::kCtas)
+    spmv_kernel(LArgs a, uint32_t j, uint32_t chunk_off, uint32_t n_chunks, uint32_t tile_off) {
   __shared__ double s_red[32];
   __shared__ uint32_t s_rp[kTileRows + 1];
   __shared__ uint16_t s_med[kTileRows], s_long[kTileRows];
@@ -216,7 +228,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 5 : 6) spmv_kernel(
   // so every lane of a warp runs every iteration and the full-mask group
   // shuffles are always converged.
   if constexpr (sizeof(T) == 8) {
-    constexpr int B = G < 8 ? G : 8, kDup = G / B;
+    constexpr int B = SpmvShape<T, G>::kSide, kDup = G / B;
     for (uint32_t it0 = 0; it0 < (uint32_t)G && it0 * kGroups < nrows; it0 += B) {
       // this lane's row of the batch, its operands loaded before the sums
       const uint32_t mine = (it0 + lane_g / kDup) * kGroups + grp;
@@ -383,7 +395,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 5 : 6) spmv_kernel(
 
   if constexpr (sizeof(T) == 8) {
     // medium rows: warp w takes list entries w, w+8, ..., kR at a time
-    constexpr int kR = 4;
+    constexpr int kR = SpmvShape<T, G>::kSideLong;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t nmed = s_nmed;
     for (uint32_t q0 = warp; q0 < nmed; q0 += kR * (kThreads / 32)) {
@@ -418,7 +430,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 5 : 6) spmv_kernel(
       }
     }
     // long rows: the whole CTA, kL rows at a time, in row order
-    constexpr int kL = 4;
+    constexpr int kL = SpmvShape<T, G>::kSideLong;
     __shared__ double s_sums[kL][kThreads / 32];
     const uint32_t nlong = s_nlong;
     for (uint32_t q0 = 0; q0 < nlong; q0 += kL) {

@@ -243,10 +243,12 @@ int cb_graph_read(const cb_graph *h, uint32_t r, uint32_t *row_ptr, uint32_t *co
  *   sc_scaled  device double[k], written: SC(nodes[q]) = exp(*log_scale) * sc_scaled[q].
  *   log_scale  device double[1], written: max over q of lambda_max(T_m) from e_q.
  * The runs share the realisation, 32 vectors at a time (three of them, n * 32
- * each, live at once).  With CB_REORTH the call builds a temporary handle
- * with k copies of the realisation instead (k * (nnz + n) * 4 bytes plus
- * their formats and a (m+1) * k * n basis).  Synchronises `stream` and frees
- * its memory before returning.
+ * each, live at once).  For a few nodes (up to 1 to 8, by precision and size),
+ * where one row is far longer than the others, and with CB_REORTH the call
+ * builds a temporary handle with k copies of the realisation instead
+ * (k * (nnz + n) * 4 bytes plus their formats and a (m+1) * k * n basis); if
+ * the device memory for one does not suffice, the other is tried.
+ * Synchronises `stream` and frees its memory before returning.
  * Errors: CB_ERR_ARG (null arguments, ranges), CB_ERR_CUDA.
  */
 int cb_subgraph_centrality(cb_graph *h, uint32_t inst, uint32_t m, int prec, uint32_t k,

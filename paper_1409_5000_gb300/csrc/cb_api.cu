@@ -812,6 +812,7 @@ static int upload_impl(uint32_t n_inst, const uint32_t *n, const uint64_t *nnz,
       ++rows;
       acc += w;
     }
+    h->inst[r].longest = most;
     h->inst[r].hubs = (uint64_t)most > (uint64_t)kHubTimes * h->inst[r].nnz / h->inst[r].n + kHubRows;
   });
   for (uint32_t r = 0; r < n_inst; ++r) {

@@ -134,7 +134,8 @@ struct InstDesc {
   uint32_t ptile_base;            // first source tile (handle-wide index)
   uint32_t pbin_base, n_pbin;     // bins
   uint32_t hubs;                  // rows far above the mean degree (kHubTimes): FP32 keeps its sums' order
-  uint32_t pad_p[2];
+  uint32_t longest;               // entries of its longest row
+  uint32_t pad_p;
   uint64_t pmat_base;             // offset of the [bin][pns + 1] chunk tables
   RedPlan pspmv;                  // slots: n_pbin bins, then n_heavy rows
 };

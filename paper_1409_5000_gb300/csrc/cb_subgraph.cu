@@ -17,11 +17,12 @@
 // vectors rotate.  Per step sc_spmv_kernel, sc_alpha_kernel, sc_axpy_kernel,
 // sc_beta_kernel, launched as dependent kernels; kSC start nodes at a time.
 // (k copies of the graph as k realisations, uploaded and formatted per call,
-// took 6.3 ms for 30 nodes of a graph of 1e5 nodes at m = 20, half of it
-// copies, formats and host scans: 1.1 ms now.)  With CB_REORTH, which needs the
-// bases, the k start nodes still become k realisations of a temporary handle
-// (device-to-device copies through cb_graph_upload).  Only e1^T exp(T - theta) e1
-// is needed: no basis combine.
+// take 3.2 ms for 30 nodes of a graph of 1e5 nodes at m = 20, half of it
+// copies, formats and host scans: 1.1 ms so.)  Where a few start nodes would not
+// fill the kSC vectors, or one row outlasts all others (few_pay), and with
+// CB_REORTH, which needs the bases, the k start nodes become k realisations of a
+// temporary handle (device-to-device copies through cb_graph_upload).  Only
+// e1^T exp(T - theta) e1 is needed: no basis combine.
 #include <algorithm>
 
 #include "cb_contour.cuh"
@@ -406,9 +407,28 @@ CB_DEBUG_READER(subgraph)
 
 using namespace cb;
 
-// CB_REORTH: k copies of the graph as realisations of a temporary handle.
-static int sc_copies(cb_graph *h, uint32_t inst, uint32_t m, int prec, uint32_t k, const uint32_t *d_nodes,
-                     double *sc_scaled, double *log_scale, cudaStream_t s) {
+// Whether k copies of the graph are the better route for k start nodes.  kSC
+// vectors cost the same whatever k; m = 20, by copies / by kSC vectors, ms:
+//   FP32  1e5 nodes, degree 10: k = 1 1.08 / 1.13, 2 1.26 / 1.13; degree 40: 1 1.5 /
+//         2.8, 4 2.8 / 2.8; 1e6, degree 16: 1 5.9 / 10.7, 4 10.2 / 10.8, 8 14.7 / 10.7;
+//         1e7: 1 52 / 109, 4 100 / 109, 8 158 / 109
+//   FP64  1e4, degree 10: 4 1.04 / 1.22, 8 1.22 / 1.22; 1e5: 1 1.2 / 2.7, 4 2.0 / 2.7,
+//         8 2.8 / 2.7; degree 40: 8 6.7 / 7.3; 1e6: 1 7 / 28, 8 24 / 29, 16 42 / 29
+// And one CTA sums each row there, 16 ns an entry (FP64: 21), where the copies'
+// kernels cut rows of more than kHeavyDeg entries over the chip: a row of 300 000
+// among 1e6 nodes 95 ms at any k, by copies 5 at k = 1, 17 at 16; of 9000 among 1e5
+// 2.5 ms, 1.1 at 1, 2.2 at 8, 3.3 at 30.
+static bool few_pay(const InstDesc &I, uint32_t k, int prec) {
+  const bool f64 = prec == CB_FP64;
+  const uint64_t nnz = I.nnz;
+  if (k <= (f64 ? (nnz >= 4000000u ? 8u : 6u) : nnz >= 4000000u ? 4u : nnz >= 2000000u ? 2u : 1u)) return true;
+  const double row_ns = (f64 ? 21.0 : 16.0) * I.longest * ((k + kSC - 1) / kSC);
+  return 50000.0 + (f64 ? 0.0107 : 0.0055) * nnz * k < row_ns;
+}
+
+// k copies of the graph as realisations of a temporary handle.
+static int sc_copies(cb_graph *h, uint32_t inst, uint32_t m, int prec, bool reorth, uint32_t k,
+                     const uint32_t *d_nodes, double *sc_scaled, double *log_scale, cudaStream_t s) {
   const InstDesc I = h->inst[inst];
   const uint64_t nnz = (inst + 1 < h->n_inst ? h->inst[inst + 1].edge_base : h->total_nnz) - I.edge_base;
   // k copies of realisation inst, one per start node
@@ -419,7 +439,7 @@ static int sc_copies(cb_graph *h, uint32_t inst, uint32_t m, int prec, uint32_t 
   int rc = cb_graph_upload(k, vn.data(), vnnz.data(), vrp.data(), vcol.data(), CB_DEVICE_PTRS,
                            s, &v);
   if (rc != CB_OK) return rc;
-  v->reorth = true;
+  v->reorth = reorth;
   rc = ensure_workspace(v, v->ws, m, prec, s);
   if (rc == CB_OK) rc = lanczos_run(v, v->ws, 0, k, m, prec, s, d_nodes, k, true);
   if (rc == CB_OK) {
@@ -530,9 +550,14 @@ CB_API int cb_subgraph_centrality(cb_graph *h, uint32_t inst, uint32_t m, int pr
     }
     d_nodes = tmp;
   }
-  const int rc = reorth ? sc_copies(h, inst, m, prec, k, d_nodes, sc_scaled, log_scale, s)
-                 : prec == CB_FP64 ? sc_batches<double>(h, inst, m, k, d_nodes, sc_scaled, log_scale, s)
-                                   : sc_batches<float>(h, inst, m, k, d_nodes, sc_scaled, log_scale, s);
+  const bool few = reorth || few_pay(I, k, prec);
+  int rc = CB_OK;
+  for (int route = 0; route < 2; ++route) {  // out of memory: the other route may fit
+    rc = few == (route == 0) ? sc_copies(h, inst, m, prec, reorth, k, d_nodes, sc_scaled, log_scale, s)
+         : prec == CB_FP64   ? sc_batches<double>(h, inst, m, k, d_nodes, sc_scaled, log_scale, s)
+                             : sc_batches<float>(h, inst, m, k, d_nodes, sc_scaled, log_scale, s);
+    if (rc != CB_ERR_OOM || reorth) break;
+  }
   dev_free(tmp);
   return rc;
 }

@@ -108,12 +108,35 @@ __device__ uint32_t row_split(const uint32_t *rp, uint32_t n, uint32_t c, uint64
   return lo;
 }
 
+// hi + lo: a sum over a warp to about twice the precision of FP32 (two-sum: lo
+// holds what the additions into hi round away), taken for alpha, whose error every
+// entry of the result shares: with plain FP32 warp sums the scores of 10 graphs of
+// 500 nodes were 1.9e-7 off on average (16 seeds; 8.7e-8 by the per-step
+// kernels, whose rows have more lanes), so 7.9e-8.  For beta it made no difference.
+template <typename T>
+struct Pair {
+  T hi, lo;
+  __device__ double value() const { return to_double(hi) + to_double(lo); }
+};
+__device__ __forceinline__ Pair<float> exact_warp_sum(float v) {
+  Pair<float> p{v, 0.f};
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float h = __shfl_xor_sync(0xffffffffu, p.hi, o), l = __shfl_xor_sync(0xffffffffu, p.lo, o);
+    const float s = __fadd_rn(p.hi, h), b = __fsub_rn(s, p.hi);
+    const float e = __fadd_rn(__fsub_rn(p.hi, __fsub_rn(s, b)), __fsub_rn(h, b));
+    p = {s, __fadd_rn(__fadd_rn(p.lo, l), e)};
+  }
+  return p;
+}
+
 template <typename T>
 struct Shared {
   T red[kTeamThreads / 32];
+  Pair<float> ared[kTeamThreads / 32];
   Split<T> scj, bpj, coef;  // scale_j, beta_{j-1} scale_{j-1}, alpha_j scale_j
-  double scale;
-  float alpha32, beta32;  // of this step and the one before
+  double scale, alpha, beta;  // of this step; beta: of the one before
+  float alpha32, beta32;      // the same in FP32
   double h[CB_MAX_M + 1], sc[CB_MAX_M + 1];  // Gram-Schmidt coefficients; scale_i so far
   uint32_t split[2];
   uint32_t nmed, nlong;
@@ -122,13 +145,32 @@ struct Shared {
   int stop;
 };
 
+// The breakdown test where FP32 does not decide it (a call: four FP64 operations of
+// 65 cycles that must not be issued on the way of every step).
+__device__ __noinline__ bool breaks_down(double beta, double tau, double alpha, double bprev) {
+  return beta <= tau * (fabs(alpha) + bprev) || beta == 0.0;
+}
+
 template <typename T>
 __device__ __forceinline__ double cta_partial(T v, Shared<T> &sh) {  // valid in warp 0
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   v = warp_sum<T>(v);
   if (lane == 0) sh.red[warp] = v;
   __syncthreads();
-  return warp == 0 ? warp_sum_d((double)sh.red[lane]) : 0.0;
+  return warp == 0 ? warp_sum_d(to_double(sh.red[lane])) : 0.0;
+}
+
+template <typename T>
+__device__ __forceinline__ double cta_alpha(T v, Shared<T> &sh) {  // valid in warp 0
+  if constexpr (sizeof(T) == 8) {
+    return cta_partial<T>(v, sh);
+  } else {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const Pair<float> p = exact_warp_sum(v);
+    if (lane == 0) sh.ared[warp] = p;
+    __syncthreads();
+    return warp == 0 ? warp_sum_d(sh.ared[lane].value()) : 0.0;
+  }
 }
 
 // Warp 0: the team's sum of `mine` (equal in all lanes); the same bits in
@@ -192,6 +234,7 @@ __global__ void __launch_bounds__(kTeamThreads, 1) team_lanczos_kernel(const __g
   }
   if (tid == 0) {
     sh.scale = sh.sc[0] = a.sc.scale[r * ms];
+    sh.beta = 0.0;
     sh.beta32 = 0.f;
     sh.scj.set(sh.scale);
     sh.bpj.set(0.0);
@@ -340,11 +383,12 @@ __global__ void __launch_bounds__(kTeamThreads, 1) team_lanczos_kernel(const __g
       spmv(integral_constant<int, 2>(), kFar, x);
     else
       spmv(integral_constant<int, 0>(), kFar, x);
-    double part = cta_partial<T>(acc, sh);
+    double part = cta_alpha<T>(acc, sh);
     if (warp == 0) {
       const double total = team_sum(parts, ctr, rank, size, ex + 1, part, &ok);
       const double scale = sh.scale, alpha = scale * total;
       if (lane == 0) {
+        sh.alpha = alpha;
         sh.alpha32 = (float)alpha;
         sh.coef.set(alpha * scale);
         if (!ok || !finite(alpha)) {
@@ -372,17 +416,17 @@ __global__ void __launch_bounds__(kTeamThreads, 1) team_lanczos_kernel(const __g
     // beta_j, the breakdown test and scale_{j+1} from the team's ||w||^2
     auto finish = [&](double total, bool last) {
       double beta, inv;
-      float beta32 = 0.f;  // decides the breakdown test: FP64 compares cost as much as products
+      float beta32;
       const int te = (__double2hiint(total) >> 20) - 1023;  // exponent (sign set: negative)
       if (te > -100 && te < 100) {
+        // 1 / sqrt(x) = y (1 - 2 r)^(-1/2), r = (1 - x y^2) / 2 of 2^-23: the series to
+        // r^2, to 2^-68; six FP64 operations
         const float y = rsqrtf((float)total);
         beta32 = (float)total * y;
-        // Newton steps y <- y + y (1/2 - x/2 y^2): to 2^-44 and to rounding
-        const double hx = -0.5 * total;
-        inv = (double)y;
-        inv = fma(inv, fma(hx * inv, inv, 0.5), inv);
-        if (sizeof(T) == 8) inv = fma(inv, fma(hx * inv, inv, 0.5), inv);
-        beta = total * inv;
+        const double yd = to_double(y), z = total * yd, r = fma(-z, to_double(0.5f * y), 0.5);
+        const double c = r * fma(1.5, r, 1.0);
+        inv = fma(yd, c, yd);
+        beta = fma(z, c, z);
       } else {
         beta = sqrt(total);
         inv = 1.0 / beta;
@@ -393,7 +437,8 @@ __global__ void __launch_bounds__(kTeamThreads, 1) team_lanczos_kernel(const __g
       __syncwarp();
       if (lane != 0) return;
       const bool bad = !ok || !finite(beta);
-      const bool broke = beta32 <= (float)a.tau * (fabsf(sh.alpha32) + sh.beta32) || beta32 == 0.f;
+      const bool broke = !(beta32 > 1.01f * (float)a.tau * (fabsf(sh.alpha32) + sh.beta32)) &&
+                         breaks_down(beta, a.tau, sh.alpha, sh.beta);
       if (rank == 0 || !ok) {
         a.sc.beta[r * ms + j] = beta;
         if (bad) a.sc.status[r] = ok ? CB_ERR_NONFINITE : CB_ERR_TIMEOUT;
@@ -403,6 +448,7 @@ __global__ void __launch_bounds__(kTeamThreads, 1) team_lanczos_kernel(const __g
       if (bad || broke) sh.stop = 1;
       if (last) {
         sh.scale = sh.sc[j + 1] = inv;
+        sh.beta = beta;
         sh.beta32 = beta32;
       }
     };

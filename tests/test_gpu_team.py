@@ -85,3 +85,42 @@ def test_ensembles_with_hubs_keep_the_order(sizes):
         parity.assert_scores(*got[-1], th_o, S_o, "fp32")
     if min(sizes) > 8192:
         assert got[0][0] == got[1][0] and np.array_equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("seed", [1, 2, 3, 4])
+def test_beta_to_fp64_rounding(seed):
+    """One step on 4^5 nodes of mean degree 8 is exact but for the root: the
+    entries of w are (degree - 8) / 32, their squares and sums few bits, so beta is
+    the root of a known number, to two units in FP64's last place, also in FP32."""
+    from paper_1409_5000_gb300 import binding as B
+
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for -m gpu tests")
+    n, rng = 1024, np.random.default_rng(seed)
+    u, v = np.triu_indices(n, 1)
+    at = rng.choice(len(u), 4 * n, replace=False)
+    g = synth.from_edges(n, np.stack([u[at], v[at]], axis=1))
+    deg = np.diff(g.row_ptr.astype(np.int64))
+    assert deg.sum() == 8 * n
+    with B.GraphSet([g]) as gs:
+        beta = B.ensemble_scores(gs, 1, B.CB_FP32, report=True)[2][0].beta_last
+    ref = np.sqrt(float(((deg - 8) ** 2).sum()) / n)
+    assert abs(beta - ref) <= 2 * np.spacing(ref)
+
+
+def test_small_ensembles_to_fp32_rounding():
+    """Scaled scores of ten 500-node graphs against the oracle's, 16 seeds: on
+    average within two FP32 units of roundoff (2 x 6e-8), one for theta, which
+    shifts them all, and one for the sums."""
+    from paper_1409_5000_gb300 import binding as B
+
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for -m gpu tests")
+    err = []
+    for seed in range(16):
+        graphs = [synth.er(500, 8.0 / 499, 100 * seed + q) for q in range(10)]
+        _, S_o = oc.ensemble_scores([(g.n, g.row_ptr, g.col) for g in graphs], 20)
+        with B.GraphSet(graphs) as gs:
+            S = B.ensemble_scores(gs, 20, B.CB_FP32)[1].float().double().cpu().numpy()
+        err.append(np.linalg.norm(S - S_o) / np.linalg.norm(S_o))
+    assert np.mean(err) <= 1.2e-7, err

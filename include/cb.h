@@ -335,6 +335,16 @@ size_t cb_memory_in_use(void);
  */
 int cb_debug_stall_tile(cb_graph *h, uint32_t btile);
 
+/*
+ * cb_debug_stall_barrier -- test hook for the barriers of the one-launch
+ * recurrence, whose CTAs wait for each other for at most 4 s of global time.
+ * After this call with limit_ms > 0 (at most 4000), the kernels that the calling
+ * host thread launches have one CTA of each team that never arrives, and give up
+ * after limit_ms: a realisation of such a team records CB_ERR_TIMEOUT as above
+ * (one CTA per realisation has no barrier).  0 switches the hook off.
+ */
+int cb_debug_stall_barrier(uint32_t limit_ms);
+
 /* Number of realisations / node count of realisation r / largest n. */
 uint32_t cb_graph_num_instances(const cb_graph *h);
 uint32_t cb_graph_num_nodes(const cb_graph *h, uint32_t r);

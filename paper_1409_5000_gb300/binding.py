@@ -114,6 +114,8 @@ def lib():
         L.cb_memory_in_use.argtypes = []
         L.cb_debug_stall_tile.restype = i32
         L.cb_debug_stall_tile.argtypes = [vp, u32]
+        L.cb_debug_stall_barrier.restype = i32
+        L.cb_debug_stall_barrier.argtypes = [u32]
         L.cb_topk_noalloc.restype = i32
         L.cb_topk_noalloc.argtypes = [vp, u32, u32, vp, vp, vp]
         L.cb_score_sum.restype = i32
@@ -338,6 +340,10 @@ def cb_memory_in_use():
 
 def cb_debug_stall_tile(h, btile):
     _check(lib().cb_debug_stall_tile(ctypes.c_void_p(h), btile))
+
+
+def cb_debug_stall_barrier(limit_ms):
+    _check(lib().cb_debug_stall_barrier(limit_ms))
 
 
 def cb_topk_noalloc(S_ptr, n, k, idx_ptr, val_ptr, stream):

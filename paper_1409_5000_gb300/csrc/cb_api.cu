@@ -23,6 +23,7 @@
 #include <thread>
 #include <unordered_map>
 
+#include "cb_grid.cuh"
 #include "cb_internal.cuh"
 #include "cb_team.cuh"
 
@@ -466,6 +467,16 @@ CB_API int cb_set_memory_limit(size_t bytes) {
 CB_API size_t cb_memory_in_use(void) {
   std::lock_guard<std::mutex> lk(g_alloc_mu);
   return g_alloc_live;
+}
+
+static thread_local uint32_t g_stall_ms = 0;  // cb_debug_stall_barrier
+uint32_t cb::barrier_stall_ms() { return g_stall_ms; }
+uint64_t cb::barrier_wait_ns() { return g_stall_ms ? g_stall_ms * 1000000ull : kGridWaitNs; }
+
+CB_API int cb_debug_stall_barrier(uint32_t limit_ms) {
+  if (limit_ms > 4000) return set_error(CB_ERR_ARG, "cb_debug_stall_barrier: need limit_ms <= 4000");
+  g_stall_ms = limit_ms;
+  return CB_OK;
 }
 
 CB_API int cb_debug_stall_tile(cb_graph *h, uint32_t btile) {
@@ -1086,7 +1097,7 @@ CB_API int cb_graph_free(cb_graph *h) {
 
 int cb::status_error(int32_t st) {
   if (st == CB_ERR_TIMEOUT)
-    return set_error(CB_ERR_TIMEOUT, "a bounded device-side wait gave up (column-blocked SpMV)");
+    return set_error(CB_ERR_TIMEOUT, "a bounded device-side wait of the Lanczos kernels gave up (a copy that never landed or a barrier)");
   return set_error(CB_ERR_NONFINITE, "a recurrence scalar became non-finite");
 }
 
@@ -1199,7 +1210,7 @@ CB_API int cb_ensemble_scores(cb_graph *h, uint32_t m, int prec, uint32_t n_out,
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   int rc = ensure_workspace(h, h->ws, m, prec, s);
   if (rc != CB_OK) return rc;
-  const bool use_graph = !g_prof_on && !rep && !std::getenv("CB_NO_GRAPH");
+  const bool use_graph = !g_prof_on && !rep && !g_stall_ms && !std::getenv("CB_NO_GRAPH");
   h->basis_m = 0;
   rc = use_graph ? ensemble_graph(h, m, prec, n_out, S, log_scale, s)
                  : ensemble_enqueue(h, m, prec, n_out, S, log_scale, s);

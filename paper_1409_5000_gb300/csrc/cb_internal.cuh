@@ -399,6 +399,10 @@ inline bool split_prec(int &prec) {
   prec &= ~CB_REORTH;
   return r;
 }
+// Limit of the grid barriers' waits, and the test hook that makes them run out
+// (cb_debug_stall_barrier; of the calling thread, 0: off).
+uint32_t barrier_stall_ms();
+uint64_t barrier_wait_ns();
 // host error for a failed realisation's device status (CB_ERR_TIMEOUT or CB_ERR_NONFINITE)
 int status_error(int32_t st);
 int cuda_error(cudaError_t e, const char *what);

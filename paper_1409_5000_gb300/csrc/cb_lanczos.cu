@@ -1329,6 +1329,8 @@ static int run_t(cb_graph *h, Workspace &W, uint32_t r0, uint32_t r1, uint32_t m
     ta.parts = W.tparts;
     ta.ctr = W.tctr;
     ta.xd = W.xd;
+    ta.wait_ns = barrier_wait_ns();
+    ta.stall = barrier_stall_ms() != 0;
     tok = prof_begin(CB_K_SPMV, s);
     const int rc = team_launch<T>(a, ta, r0, m, team_grid, team_coop, s);
     prof_end(tok, s);

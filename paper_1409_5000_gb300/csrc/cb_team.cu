@@ -180,14 +180,14 @@ __device__ __forceinline__ double cta_alpha(T v, Shared<T> &sh) {  // valid in w
 // threads stored before the barrier in front of this call is visible to the
 // team after it.  *ok turns false when the wait gave up.
 __device__ double team_sum(double *part, uint32_t *ctr, uint32_t rank, uint32_t size, uint32_t ex, double mine,
-                           bool *ok) {
+                           uint64_t wait_ns, bool *ok) {
   if (size == 1) return mine;
   const uint32_t lane = threadIdx.x & 31;
   part += (ex & 1u) * kMaxTeamCtas;
   if (lane == 0) {
     part[rank] = mine;
     red_release(ctr, 1u);
-    if (!grid_wait(ctr, ex * size)) *ok = false;
+    if (!grid_wait(ctr, ex * size, wait_ns)) *ok = false;
   }
   __syncwarp();  // orders the other lanes' loads after lane 0's acquire
   *ok = __all_sync(0xffffffffu, *ok);
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kTeamThreads, 1) team_lanczos_kernel(const __g
   const InstDesc &I = a.inst[r];
   const uint32_t n = I.n, nnz = I.nnz, ms = a.sc.ms;
   const uint32_t mr = min(a.sc.meff[r], m);  // 0: no start vector (no CTA has changed it yet)
-  if (mr == 0) return;
+  if (mr == 0 || (t.stall && size > 1 && rank + 1 == size)) return;
   const uint32_t *rpg = a.row_ptr + I.rp_base;
   const uint32_t *cg = a.col + I.edge_base;
   const uint32_t rc = max(1u, (uint32_t)(((uint64_t)nnz + (uint64_t)n * t.rowdiv - 1) / ((uint64_t)n * t.rowdiv)));
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(kTeamThreads, 1) team_lanczos_kernel(const __g
       spmv(integral_constant<int, 0>(), kFar, x);
     double part = cta_alpha<T>(acc, sh);
     if (warp == 0) {
-      const double total = team_sum(parts, ctr, rank, size, ex + 1, part, &ok);
+      const double total = team_sum(parts, ctr, rank, size, ex + 1, part, t.wait_ns, &ok);
       const double scale = sh.scale, alpha = scale * total;
       if (lane == 0) {
         sh.alpha = alpha;
@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(kTeamThreads, 1) team_lanczos_kernel(const __g
           }
         }
         part = cta_partial<T>(acc2, sh);
-        if (warp == 0) finish(team_sum(parts, ctr, rank, size, ex + 2 + pass, part, &ok), false);
+        if (warp == 0) finish(team_sum(parts, ctr, rank, size, ex + 2 + pass, part, t.wait_ns, &ok), false);
         __syncthreads();
         if (sh.stop) break;
         if (size > 1) {  // h_i over the team, in rank order
@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(kTeamThreads, 1) team_lanczos_kernel(const __g
       if (sh.stop) break;
     }
     part = cta_partial<T>(acc2, sh);
-    if (warp == 0) finish(team_sum(parts, ctr, rank, size, ex + (t.reorth ? 4 : 2), part, &ok), true);
+    if (warp == 0) finish(team_sum(parts, ctr, rank, size, ex + (t.reorth ? 4 : 2), part, t.wait_ns, &ok), true);
     __syncthreads();
     if (sh.stop) break;
     ex += t.reorth ? 4 : 2;

@@ -18,6 +18,8 @@ struct TeamArgs {
   uint32_t smem;     // dynamic shared memory of a CTA
   uint32_t rowdiv;   // a row weighs as much as mean degree / rowdiv entries
   uint32_t reorth;
+  uint64_t wait_ns;  // limit of a barrier's wait
+  uint32_t stall;    // test hook: the last CTA of each team never arrives
   uint16_t first[kMaxTeams + 1];  // first CTA of each team
 };
 

@@ -119,7 +119,7 @@ __device__ uint32_t pass_end(TopkShared &sh, TopkState *st, Select &sel, uint32_
     uint32_t *g = st->hist[pass % 3];
     if (h0) atomicAdd(&g[kBins - 1 - 2 * tid], h0);
     if (h1) atomicAdd(&g[kBins - 2 - 2 * tid], h1);
-    if (!grid_sync(&st->bar, epoch)) *ok = false;
+    if (!grid_sync(&st->bar, epoch, gridDim.x, kGridWaitNs)) *ok = false;
     h0 = __ldcg(&g[kBins - 1 - 2 * tid]);
     h1 = __ldcg(&g[kBins - 2 - 2 * tid]);
     // the buffer of the previous pass: every CTA read it before this barrier,
@@ -182,7 +182,7 @@ __device__ uint32_t collect(const double *__restrict__ S, uint32_t n, unsigned l
     for (int u = 0; u < 4; ++u) take(v[u], (uint32_t)(i + u * stride));
   }
   for (; i < n; i += stride) take(__ldg(S + i), (uint32_t)i);
-  if (!grid_sync(&st->bar, epoch)) *ok = false;
+  if (!grid_sync(&st->bar, epoch, gridDim.x, kGridWaitNs)) *ok = false;
   const uint32_t c = gridDim.x > 1 ? __ldcg(&st->ncol) : sh.ncol;
   __syncthreads();  // a second collection clears the count
   return c;

@@ -337,11 +337,13 @@ int cb_debug_stall_tile(cb_graph *h, uint32_t btile);
 
 /*
  * cb_debug_stall_barrier -- test hook for the barriers of the one-launch
- * recurrence, whose CTAs wait for each other for at most 4 s of global time.
- * After this call with limit_ms > 0 (at most 4000), the kernels that the calling
- * host thread launches have one CTA of each team that never arrives, and give up
- * after limit_ms: a realisation of such a team records CB_ERR_TIMEOUT as above
- * (one CTA per realisation has no barrier).  0 switches the hook off.
+ * recurrence and of the top-k, whose CTAs wait for each other for at most 4 s of
+ * global time.  After this call with limit_ms > 0 (at most 4000), the kernels
+ * that the calling host thread launches have one CTA (of each team) that never
+ * arrives, and give up after limit_ms: a realisation of such a team records
+ * CB_ERR_TIMEOUT as above (one CTA per realisation has no barrier), and
+ * cb_topk, whose first CTA then selects alone, returns the same as ever.
+ * 0 switches the hook off.
  */
 int cb_debug_stall_barrier(uint32_t limit_ms);
 

@@ -99,6 +99,13 @@ struct Select {
   uint32_t plo, krem, above;  // above: elements in higher buckets (taken already)
 };
 
+// The CTAs that select together (all of the grid, or one alone), and their scratch.
+struct Team {
+  uint32_t ctas, rank;
+  uint64_t wait_ns;
+  TopkState *st;  // zeroed; unused by a CTA alone, as is the candidates' global buffer
+};
+
 // What the passes share within a CTA.
 struct TopkShared {
   uint32_t hist[kBins];
@@ -110,23 +117,23 @@ struct TopkShared {
 // from the top reaches sel.krem chosen, the prefix extended.  Returns the
 // elements of the chosen bucket.  pass: passes done so far (selects the merged
 // histogram).  *ok turns false when a barrier gave up.
-__device__ uint32_t pass_end(TopkShared &sh, TopkState *st, Select &sel, uint32_t L, uint32_t &pass,
+__device__ uint32_t pass_end(TopkShared &sh, const Team &t, Select &sel, uint32_t L, uint32_t &pass,
                              uint32_t &epoch, bool *ok) {
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   __syncthreads();
   uint32_t h0 = sh.hist[kBins - 1 - 2 * tid], h1 = sh.hist[kBins - 2 - 2 * tid];  // from the top
-  if (gridDim.x > 1) {
-    uint32_t *g = st->hist[pass % 3];
+  if (t.ctas > 1) {
+    uint32_t *g = t.st->hist[pass % 3];
     if (h0) atomicAdd(&g[kBins - 1 - 2 * tid], h0);
     if (h1) atomicAdd(&g[kBins - 2 - 2 * tid], h1);
-    if (!grid_sync(&st->bar, epoch, gridDim.x, kGridWaitNs)) *ok = false;
+    if (!grid_sync(&t.st->bar, epoch, t.ctas, t.wait_ns)) *ok = false;
     h0 = __ldcg(&g[kBins - 1 - 2 * tid]);
     h1 = __ldcg(&g[kBins - 2 - 2 * tid]);
     // the buffer of the previous pass: every CTA read it before this barrier,
     // and its next use is two passes on
     if (pass > 0)
-      for (uint32_t q = blockIdx.x * kTopkThreads + tid; q < kBins; q += gridDim.x * kTopkThreads)
-        st->hist[(pass - 1) % 3][q] = 0u;
+      for (uint32_t q = t.rank * kTopkThreads + tid; q < kBins; q += t.ctas * kTopkThreads)
+        t.st->hist[(pass - 1) % 3][q] = 0u;
   }
   ++pass;
   const uint32_t mine = h0 + h1;
@@ -162,11 +169,11 @@ __device__ uint32_t pass_end(TopkShared &sh, TopkState *st, Select &sel, uint32_
 // Elements whose composite key reaches the prefix (phi, plo) go to buf, in any
 // order; their number (which may exceed kCand) is returned.
 __device__ uint32_t collect(const double *__restrict__ S, uint32_t n, unsigned long long phi,
-                            uint32_t plo, TopkShared &sh, TopkState *st, Cand *buf, uint32_t &epoch,
+                            uint32_t plo, TopkShared &sh, const Team &t, Cand *buf, uint32_t &epoch,
                             bool *ok) {
-  uint32_t *ctr = gridDim.x > 1 ? &st->ncol : &sh.ncol;
-  const uint64_t stride = (uint64_t)gridDim.x * kTopkThreads;
-  uint64_t i = blockIdx.x * kTopkThreads + threadIdx.x;
+  uint32_t *ctr = t.ctas > 1 ? &t.st->ncol : &sh.ncol;
+  const uint64_t stride = (uint64_t)t.ctas * kTopkThreads;
+  uint64_t i = t.rank * kTopkThreads + threadIdx.x;
   auto take = [&](double v, uint32_t at) {
     const unsigned long long key = order_key(v);
     if (key > phi || (key == phi && ~at >= plo)) {
@@ -182,8 +189,8 @@ __device__ uint32_t collect(const double *__restrict__ S, uint32_t n, unsigned l
     for (int u = 0; u < 4; ++u) take(v[u], (uint32_t)(i + u * stride));
   }
   for (; i < n; i += stride) take(__ldg(S + i), (uint32_t)i);
-  if (!grid_sync(&st->bar, epoch, gridDim.x, kGridWaitNs)) *ok = false;
-  const uint32_t c = gridDim.x > 1 ? __ldcg(&st->ncol) : sh.ncol;
+  if (!grid_sync(t.ctas > 1 ? &t.st->bar : nullptr, epoch, t.ctas, t.wait_ns)) *ok = false;
+  const uint32_t c = t.ctas > 1 ? __ldcg(&t.st->ncol) : sh.ncol;
   __syncthreads();  // a second collection clears the count
   return c;
 }
@@ -255,16 +262,12 @@ __device__ void sort_out(const double *__restrict__ S, const Cand *buf, uint32_t
   }
 }
 
-// st and gbuf: the grid's scratch (st zeroed); unused by a single CTA, whose
-// candidates stay in shared memory (kCand of them fit beside the sort).
-__global__ void __launch_bounds__(kTopkThreads, 1) topk_kernel(const double *__restrict__ S, uint32_t n,
-                                                               uint32_t k, TopkState *st, Cand *gbuf,
-                                                               uint32_t *idx, double *val) {
-  extern __shared__ __align__(16) unsigned char s_raw[];
-  __shared__ TopkShared sh;
+// The candidates, at least k and at most kCand, in buf; their number, or 0 when a
+// barrier gave up.
+__device__ uint32_t select(const double *__restrict__ S, uint32_t n, uint32_t k, const Team &t, TopkShared &sh,
+                           Cand *buf) {
   const uint32_t tid = threadIdx.x;
-  const uint64_t stride = (uint64_t)gridDim.x * kTopkThreads, i0 = blockIdx.x * kTopkThreads + tid;
-  Cand *buf = gridDim.x > 1 ? gbuf : reinterpret_cast<Cand *>(s_raw + kCand * 12);
+  const uint64_t stride = (uint64_t)t.ctas * kTopkThreads, i0 = t.rank * kTopkThreads + tid;
   uint32_t epoch = 0, pass = 0, C = kCand + 1;
   bool ok = true;
   sh.hist[2 * tid] = sh.hist[2 * tid + 1] = 0u;
@@ -286,15 +289,13 @@ __global__ void __launch_bounds__(kTopkThreads, 1) topk_kernel(const double *__r
     Select sel{0ull, 0u, k, 0u};
     for (uint32_t L = 0; L < kKeyLevels && ok; ++L) {
       if (i0 < n && (my & mask_hi(L)) == sel.phi) atomicAdd(&sh.hist[digit(my, 0u, L)], 1u);
-      const uint32_t bucket = pass_end(sh, st, sel, L, pass, epoch, &ok);
+      const uint32_t bucket = pass_end(sh, t, sel, L, pass, epoch, &ok);
       if (sel.above + bucket <= max(kFew, k) || sel.krem == bucket) break;
     }
-    if (ok) C = collect(S, n, sel.phi, 0u, sh, st, buf, epoch, &ok);
+    if (ok) C = collect(S, n, sel.phi, 0u, sh, t, buf, epoch, &ok);
   }
-  if (C > kCand && ok) {  // uniform over the grid: the composite keys of all elements
-    if (tid == 0) {
-      if (gridDim.x == 1) sh.ncol = 0u;
-    }
+  if (C > kCand && ok) {  // uniform over the CTAs: the composite keys of all elements
+    if (tid == 0 && t.ctas == 1) sh.ncol = 0u;
     Select sel{0ull, 0u, k, 0u};
     for (uint32_t L = 0; L < kLevels && ok; ++L) {
       const unsigned long long mh = mask_hi(L);
@@ -305,19 +306,33 @@ __global__ void __launch_bounds__(kTopkThreads, 1) topk_kernel(const double *__r
         if ((key & mh) == sel.phi && (lo & ml) == sel.plo) atomicAdd(&sh.hist[digit(key, lo, L)], 1u);
       }
       // no CTA still reads the count of the first collection after the first barrier
-      const uint32_t bucket = pass_end(sh, st, sel, L, pass, epoch, &ok);
-      if (L == 0 && gridDim.x > 1 && blockIdx.x == 0 && tid == 0) st->ncol = 0u;
+      const uint32_t bucket = pass_end(sh, t, sel, L, pass, epoch, &ok);
+      if (L == 0 && t.ctas > 1 && t.rank == 0 && tid == 0) t.st->ncol = 0u;
       if (L > 0 && (sel.above + bucket <= max(kFew, k) || sel.krem == bucket)) break;
     }
-    if (ok) C = collect(S, n, sel.phi, sel.plo, sh, st, buf, epoch, &ok);
+    if (ok) C = collect(S, n, sel.phi, sel.plo, sh, t, buf, epoch, &ok);
   }
+  return ok ? C : 0u;
+}
+
+// Every wait is bounded (a GPU that suspends a CTA for seconds must not hang the
+// others).  Should one give up, the first CTA selects alone: what it then reads
+// and writes is its own, so CTAs that come late disturb nothing, and the result is
+// the same.  Its candidates stay in shared memory, beside the sort's arrays.
+__global__ void __launch_bounds__(kTopkThreads, 1) topk_kernel(const double *__restrict__ S, uint32_t n,
+                                                               uint32_t k, TopkState *st, Cand *gbuf,
+                                                               uint32_t *idx, double *val, uint64_t wait_ns,
+                                                               uint32_t stall) {
+  extern __shared__ __align__(16) unsigned char s_raw[];
+  __shared__ TopkShared sh;
+  Cand *own = reinterpret_cast<Cand *>(s_raw + kCand * 12), *buf = gridDim.x > 1 ? gbuf : own;
+  if (stall && blockIdx.x > 0 && blockIdx.x + 1 == gridDim.x) return;  // test hook
+  uint32_t C = select(S, n, k, Team{gridDim.x, blockIdx.x, wait_ns, st}, sh, buf);
   if (blockIdx.x != 0) return;
-  if (!ok || C > kCand || C < k) {  // a barrier gave up: no selection
-    for (uint32_t p = tid; p < k; p += kTopkThreads) {
-      idx[p] = 0xffffffffu;
-      val[p] = __longlong_as_double(0x7ff8000000000000ll);
-    }
-    return;
+  if (C == 0) {
+    buf = own;
+    __syncthreads();
+    C = select(S, n, k, Team{1u, 0u, wait_ns, nullptr}, sh, buf);
   }
   sort_out(S, buf, C, k, s_raw, idx, val);
 }
@@ -326,7 +341,7 @@ __global__ void __launch_bounds__(kTopkThreads, 1) topk_kernel(const double *__r
 
 int topk_launch(const double *S, uint32_t n, uint32_t k, uint32_t *idx, double *val,
                 void *scratch, cudaStream_t s) {
-  // shared memory: the sort's arrays, and for a single CTA its candidates too
+  // shared memory: the sort's arrays and the candidates of a CTA that selects alone
   constexpr size_t kSort = (size_t)kCand * 12, kAll = kSort + (size_t)kCand * sizeof(Cand);
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -336,17 +351,19 @@ int topk_launch(const double *S, uint32_t n, uint32_t k, uint32_t *idx, double *
   if (e != cudaSuccess) return cuda_error(e, "topk launch");
   const int tok = prof_begin(CB_K_TOPK, s);
   if (n <= kOneCta) {
-    topk_kernel<<<1, kTopkThreads, kAll, s>>>(S, n, k, nullptr, nullptr, idx, val);
+    topk_kernel<<<1, kTopkThreads, kAll, s>>>(S, n, k, nullptr, nullptr, idx, val, 0, 0);
   } else {
     TopkState *st = reinterpret_cast<TopkState *>(scratch);
     Cand *buf = reinterpret_cast<Cand *>(st + 1);
     // four scores per thread up to one CTA per SM: a barrier over fewer CTAs is cheaper
     const uint32_t grid = std::min<uint32_t>((uint32_t)sms, (n + 4 * kTopkThreads - 1) / (4 * kTopkThreads));
     e = cudaMemsetAsync(st, 0, sizeof(TopkState), s);
-    void *args[] = {&S, &n, &k, &st, &buf, &idx, &val};
+    uint64_t wait_ns = barrier_wait_ns();
+    uint32_t stall = barrier_stall_ms() != 0;
+    void *args[] = {&S, &n, &k, &st, &buf, &idx, &val, &wait_ns, &stall};
     if (e == cudaSuccess)
       e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(topk_kernel), dim3(grid),
-                                      dim3(kTopkThreads), args, kSort, s);
+                                      dim3(kTopkThreads), args, kAll, s);
   }
   prof_end(tok, s);
   if (e == cudaSuccess) e = cudaGetLastError();

@@ -1,7 +1,8 @@
 """Barriers between the CTAs of a launch that run out (needs a GB300; no GPU
 fault, trap or hang): the hook cb_debug_stall_barrier keeps one CTA from
-arriving and shortens the wait to 20 ms.  A realisation of the one-launch
-recurrence then reports CB_ERR_TIMEOUT; the next calls are as ever."""
+arriving and shortens the wait to 20 ms.  The top-k then selects on one CTA and
+returns the same; a realisation of the one-launch recurrence reports
+CB_ERR_TIMEOUT; the next calls are as ever."""
 import math
 import time
 
@@ -28,6 +29,23 @@ def B():
 def stall(B):
     yield lambda: B.cb_debug_stall_barrier(20)
     B.cb_debug_stall_barrier(0)
+
+
+@pytest.mark.parametrize("kind", ["spread", "ties"])
+@pytest.mark.parametrize("n", [4096, 4097, 155_649, 700_001])
+def test_topk_whose_barrier_runs_out(B, stall, n, kind):
+    rng = np.random.default_rng(n)
+    S = np.exp(6 * rng.normal(size=n)) if kind == "spread" else rng.integers(0, 3, size=n).astype(np.float64)
+    d = torch.from_numpy(S).cuda()
+    order = np.lexsort((np.arange(n), -S))
+    for k in (1, 20, 1025, 4096):
+        for on in (False, True, False):
+            if on:
+                stall()
+            idx, val = B.topk(d, k)
+            B.cb_debug_stall_barrier(0)
+            assert np.array_equal(idx.cpu().numpy().astype(np.int64), order[:k])
+            assert np.array_equal(val.cpu().numpy(), S[order[:k]])
 
 
 @pytest.mark.parametrize("prec", ["fp32", "fp64 reorthogonalised"])

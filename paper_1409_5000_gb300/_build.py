@@ -2,7 +2,8 @@
 
 * ``_lib/libcb.so``      -- the C-ABI library (CUDA, sm_103a only), built
   with nvcc from ``csrc/*.cu``; one object per translation unit, compiled
-  in parallel, then linked with ``-shared``.
+  in parallel, then linked with ``-shared`` and ``-z nodelete``: its helper threads
+  outlive a call by two seconds, so closing the library must not unmap it.
 * ``_lib/libcb_debug.so`` -- the same sources with ``-DCB_DEBUG``: every
   indexed access of the SpMV kernels checked on the device (a violation is
   counted and skipped, never trapped); loaded instead of libcb.so when the
@@ -99,7 +100,7 @@ def build_cb(verbose: bool = False, extra_flags=(), debug: bool = False) -> str:
         fd, tmp = tempfile.mkstemp(suffix=".so", dir=LIBDIR)
         os.close(fd)
         _run([nvcc, "-shared", "-o", tmp] + [o for o, _ in results] + ARCH
-             + ["-Xcompiler", "-fPIC", "-cudart", "static"])
+             + ["-Xcompiler", "-fPIC", "-Xlinker", "-z,nodelete", "-cudart", "static"])
         _atomic_move(tmp, cb_lib_path(debug))
     finally:
         shutil.rmtree(objdir, ignore_errors=True)

@@ -999,9 +999,9 @@ CB_API int cb_graph_set_path(cb_graph *h, int path) {
   if (!h) return set_error(CB_ERR_ARG, "cb_graph_set_path: null handle");
   if (path != CB_PATH_AUTO && path != CB_PATH_FORMATS && path != CB_PATH_CSR)
     return set_error(CB_ERR_ARG, "cb_graph_set_path: unknown path");
-  if (h->path != path || h->tuned_auto) {
+  if (h->path != path || h->tuned) {
     h->path = path;
-    h->tuned_auto = false;
+    h->tuned = false;
     drop_graphs(h);  // captured passes hold the old kernel choice
   }
   return CB_OK;
@@ -1022,12 +1022,14 @@ CB_API int cb_graph_tune(cb_graph *h, int prec, uint32_t *lanes_out, double *ms_
   static const uint32_t kCand[6] = {1, 2, 4, 8, 16, 32};
   for (int c = 0; ms_out && c < 8; ++c) ms_out[c] = -1.0;
   // the format path is a candidate in FP32 when a format was built; the
-  // single launch of all steps (the automatic path) when every realisation is
-  // small enough for it
+  // automatic path where it runs all steps in one launch, or every realisation is small
   const bool formats = prec == CB_FP32 && (h->total_btiles > 0 || h->total_ptiles > 0);
-  bool small = true;
-  for (uint32_t r = 0; r < h->n_inst && small; ++r)
-    small = h->inst[r].n <= kSmallN && h->inst[r].nnz <= kSmallNnz;
+  bool small = lanczos_one_launch(h, prec);
+  if (!small) {  // a small handle's automatic path is timed whatever it does
+    small = true;
+    for (uint32_t r = 0; r < h->n_inst && small; ++r)
+      small = h->inst[r].n <= kSmallN && h->inst[r].nnz <= kSmallNnz;
+  }
   constexpr uint32_t kProbe = 3;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   Workspace W;
@@ -1037,8 +1039,6 @@ CB_API int cb_graph_tune(cb_graph *h, int prec, uint32_t *lanes_out, double *ms_
   cudaError_t e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
   const int keep_lanes = h->lanes, keep_path = h->path;
-  const bool keep_auto = h->tuned_auto;
-  h->tuned_auto = false;
   int best_lanes = keep_lanes, best_path = keep_path;
   double best_ms = 1e300;
   auto time_one = [&](int lanes, int path, int slot) {
@@ -1053,7 +1053,7 @@ CB_API int cb_graph_tune(cb_graph *h, int prec, uint32_t *lanes_out, double *ms_
     float ms = 0.f;
     if (rc == CB_OK && e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
     if (rc == CB_OK && e == cudaSuccess) {
-      if (ms_out && slot >= 0) ms_out[slot] = ms / 2.0;
+      if (ms_out) ms_out[slot] = ms / 2.0;
       if (ms < best_ms) {
         best_ms = ms;
         best_lanes = lanes;
@@ -1067,27 +1067,20 @@ CB_API int cb_graph_tune(cb_graph *h, int prec, uint32_t *lanes_out, double *ms_
   if (small && e == cudaSuccess && rc == CB_OK) time_one(best_lanes, CB_PATH_AUTO, 7);
   // FP64 depends on the path only through the single launch
   if (prec == CB_FP64 && !small) best_path = keep_path;
-  // other handles may run as one launch too: the path kept stays a per-step
-  // one, and the automatic choice is taken beside it where it is faster
-  if (!small && e == cudaSuccess && rc == CB_OK) {
-    const double per_step = best_ms;
-    const int l = best_lanes, p = best_path;
-    time_one(best_lanes, CB_PATH_AUTO, -1);
-    h->tuned_auto = best_ms < per_step;
-    best_lanes = l;
-    best_path = p;
-  }
   h->lanes = best_lanes;
   h->path = best_path;
-  if (keep_auto != h->tuned_auto || best_lanes != keep_lanes || best_path != keep_path) drop_graphs(h);
+  if (best_lanes != keep_lanes || best_path != keep_path) drop_graphs(h);
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   free_workspace(W);
   if (rc != CB_OK || e != cudaSuccess) {
     h->lanes = keep_lanes;
     h->path = keep_path;
-    h->tuned_auto = keep_auto;
     return rc != CB_OK ? rc : cuda_error(e, "cb_graph_tune");
+  }
+  if ((prec == CB_FP32 || small) && !h->tuned) {  // otherwise FP64 keeps the path as it was
+    h->tuned = true;
+    drop_graphs(h);  // captured FP64 passes of a path set before
   }
   if (lanes_out) *lanes_out = (uint32_t)best_lanes;
   return CB_OK;

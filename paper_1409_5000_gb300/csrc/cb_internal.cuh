@@ -205,8 +205,8 @@ struct cb_graph {
   uint32_t total_slots = 0, total_groups = 0;
   int lanes = 8;  // lanes per row for short rows (1, 2, 4, 8, 16, 32)
   int path = CB_PATH_AUTO;  // FP32 SpMV path (cb_graph_set_path)
-  bool tuned_auto = false;  // the tuner found the automatic path fastest and kept a per-step one
-                            // beside it (cb_graph_tune)
+  bool tuned = false;  // `path` is what the tuner measured best without reorthogonalisation, not a
+                       // caller's choice: FP64 with it stays on the automatic path
   uint32_t n_sm = 1;        // SMs of the handle's device
   // a group handle of the budgeted adjoint plans its teams as part of the
   // whole handle, so that the groups' results are the whole's bit for bit
@@ -479,6 +479,8 @@ void free_backwork(BackWork &B);  // cb_adjoint.cu
 // (k entries), or with per_inst one start node per realisation (e_idx[r-r0]).
 // restart_scale (device, double[N]): a restarted cycle; W_0 already holds
 // the start vector with scale restart_scale[r] (0: nothing to do).
+// Whether the automatic path runs the handle's plain FP32 or FP64 recurrence in one launch.
+bool lanczos_one_launch(const cb_graph *h, int prec);
 int lanczos_run(cb_graph *h, Workspace &W, uint32_t r0, uint32_t r1, uint32_t m, int prec,
                 cudaStream_t s, const uint32_t *start_idx = nullptr, uint32_t k = 0,
                 bool per_inst = false, const double *restart_scale = nullptr);

@@ -1209,6 +1209,37 @@ static void launch_spmv_lanes(int lanes, const LArgs &a, uint32_t j, uint32_t co
   }
 }
 
+// The route of the recurrence over realisations [r0, r1) on the automatic path,
+// and the plan of the first: on-chip problems take one launch.  A team sums in an
+// order of its own: taken where that cannot show, FP64 with reorthogonalisation
+// and FP32 ensembles and small graphs without hubs.  One larger graph in FP32 keeps
+// the order of the per-step kernels (a planted clique's scores differ by less
+// than FP32 rounding), as does FP64 without it (T's trailing part).
+enum Route { kPerStep, kTeam, kOneCta };
+template <typename T>
+static Route one_launch_route(const cb_graph *h, uint32_t r0, uint32_t r1, bool reorth, TeamArgs *ta, uint32_t *grid,
+                              bool *cooperative) {
+  const cb_graph *hp = h->plan_of ? h->plan_of : h;  // a group handle decides as the whole one
+  const uint32_t p0 = h->plan_of ? 0u : r0, p1 = h->plan_of ? hp->n_inst : r1;
+  bool small = true, hubs = false;
+  for (uint32_t r = p0; r < p1; ++r) {
+    small &= hp->inst[r].n <= kSmallN && hp->inst[r].nnz <= kSmallNnz;
+    hubs |= hp->inst[r].hubs != 0;
+  }
+  if ((sizeof(T) == 8 ? reorth : !reorth && !hubs && (small || p1 - p0 > 1)) &&
+      team_plan(h, r0, r1, sizeof(T), reorth, ta, grid, cooperative))
+    return kTeam;
+  return small && !reorth && (sizeof(T) == 8 || hubs || small_launch_pays(hp, p0, p1)) ? kOneCta : kPerStep;
+}
+
+bool lanczos_one_launch(const cb_graph *h, int prec) {
+  TeamArgs ta;
+  uint32_t grid;
+  bool coop;
+  return (prec == CB_FP64 ? one_launch_route<double>(h, 0, h->n_inst, false, &ta, &grid, &coop)
+                          : one_launch_route<float>(h, 0, h->n_inst, false, &ta, &grid, &coop)) != kPerStep;
+}
+
 template <typename T>
 static int run_t(cb_graph *h, Workspace &W, uint32_t r0, uint32_t r1, uint32_t m, cudaStream_t s,
                  const uint32_t *start_idx, uint32_t k, bool per_inst, const double *rscale) {
@@ -1302,30 +1333,17 @@ static int run_t(cb_graph *h, Workspace &W, uint32_t r0, uint32_t r1, uint32_t m
         reinterpret_cast<T *>(a.V) + A0.node_base, init_n8, start_idx ? T(0) : T(1));
   if (start_idx && !rscale)
     init_indicator_kernel<T><<<r1 - r0, kThreads, 0, s>>>(a, r0, start_idx, k, per_inst);
-  // on-chip problems on the automatic path: the whole recurrence in one launch
   TeamArgs ta;
   uint32_t team_grid = 0;
   bool team_coop = false;
-  const bool one_launch = (h->path == CB_PATH_AUTO || h->tuned_auto) && h->stall_btile == UINT32_MAX;
-  const cb_graph *hp = h->plan_of ? h->plan_of : h;  // a group handle decides as the whole one
-  const uint32_t p0 = h->plan_of ? 0u : r0, p1 = h->plan_of ? hp->n_inst : r1;
-  bool small = true, hubs = false;
-  for (uint32_t r = p0; r < p1; ++r) {
-    small &= hp->inst[r].n <= kSmallN && hp->inst[r].nnz <= kSmallNnz;
-    hubs |= hp->inst[r].hubs != 0;
-  }
-  // a team sums in an order of its own: taken where that cannot show, FP64 with
-  // reorthogonalisation and FP32 ensembles and small graphs without hubs.  One larger graph in
-  // FP32 keeps the order of the per-step kernels (a planted clique's scores differ
-  // by less than FP32 rounding), as does FP64 without it (T's trailing part)
-  const bool team = one_launch &&
-                    (sizeof(T) == 8 ? h->reorth : !h->reorth && !hubs && (small || p1 - p0 > 1)) &&
-                    team_plan(h, r0, r1, sizeof(T), h->reorth, &ta, &team_grid, &team_coop);
+  Route route = kPerStep;
+  if ((h->path == CB_PATH_AUTO || (h->tuned && sizeof(T) == 8 && h->reorth)) && h->stall_btile == UINT32_MAX)
+    route = one_launch_route<T>(h, r0, r1, h->reorth, &ta, &team_grid, &team_coop);
   const uint64_t nsc = (uint64_t)(r1 - r0) * W.sc.ms;
   init_scalars_kernel<<<(uint32_t)((nsc + kThreads - 1) / kThreads), kThreads, 0, s>>>(
       a, r0, r1, m, start_idx, k, per_inst, rscale, W.tctr);
   prof_end(tok, s);
-  if (team) {
+  if (route == kTeam) {
     ta.parts = W.tparts;
     ta.ctr = W.tctr;
     ta.xd = W.xd;
@@ -1336,7 +1354,7 @@ static int run_t(cb_graph *h, Workspace &W, uint32_t r0, uint32_t r1, uint32_t m
     prof_end(tok, s);
     return rc;
   }
-  if (small && one_launch && !h->reorth && (sizeof(T) == 8 || hubs || small_launch_pays(hp, p0, p1))) {
+  if (route == kOneCta) {
     cudaFuncSetAttribute(lanczos_small_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(3 * kSmallN * sizeof(T)));
     tok = prof_begin(CB_K_SPMV, s);

@@ -100,3 +100,38 @@ def test_centrality_beside_a_heavy_row(B, k, links, copies, prec):
     ref = np.exp(th - top) * c0  # the hub's lambda is 95: no plain exponentials
     got = got * np.exp(float(ls.item()) - top)
     assert np.max(np.abs(got - ref)) <= (1e-11 if prec else 1e-4) * ref.max()
+
+
+def test_tuning_keeps_the_one_launch(B):
+    """Eight graphs of 30 000 nodes run fastest in one launch: the tuner times that
+    beside the per-step paths, keeps it, and the path read back and set on
+    another handle, as from a cache, is the same."""
+    sizes, target = [30_000] * 8, np.array([(0, 1)])
+    with B.GraphSet.generate_er(sizes, 12, 5, target) as gs:
+        lanes, ms = B.cb_graph_tune(gs.h, B.CB_FP32, 0)
+        assert all(x >= 0 for x in ms) and ms[7] == min(ms)
+        path = B.cb_graph_path(gs.h)
+        ls, S, launches = _pass(B, gs, 10, B.CB_FP32)
+        assert launches == 1 and path == B.CB_PATH_AUTO
+    with B.GraphSet.generate_er(sizes, 12, 5, target) as gs:
+        B.cb_graph_set_lanes(gs.h, lanes)
+        B.cb_graph_set_path(gs.h, path)
+        ls_2, S_2, launches = _pass(B, gs, 10, B.CB_FP32)
+    assert launches == 1 and ls_2 == ls and np.array_equal(S_2, S)
+
+
+def test_tuning_fp32_leaves_fp64_alone(B):
+    """One larger graph: FP32 keeps a per-step path, reorthogonalised FP64 its one
+    launch; a path that the caller sets holds for both."""
+    with B.GraphSet.generate_er([60_000], 10, 6, np.array([(0, 1)])) as gs:
+        p64 = B.CB_FP64 | B.CB_REORTH
+        ls, S, launches = _pass(B, gs, 10, p64)
+        assert launches == 1
+        for _ in range(3):
+            B.cb_graph_tune(gs.h, B.CB_FP32, 0)
+            assert B.cb_graph_path(gs.h) in (B.CB_PATH_FORMATS, B.CB_PATH_CSR)
+            assert _pass(B, gs, 10, B.CB_FP32)[2] == 10
+            ls_t, S_t, launches = _pass(B, gs, 10, p64)
+            assert launches == 1 and ls_t == ls and np.array_equal(S_t, S)
+        B.cb_graph_set_path(gs.h, B.CB_PATH_CSR)
+        assert _pass(B, gs, 10, p64)[2] == 10

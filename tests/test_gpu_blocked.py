@@ -55,3 +55,29 @@ def test_rows_as_long_as_their_stream(d):
     with B.GraphSet(graphs, path=B.CB_PATH_FORMATS) as gs:
         ls, S = B.ensemble_scores(gs, 15, B.CB_FP32)
         parity.assert_scores(float(ls.item()), S.cpu().numpy(), th_o, S_o, "fp32")
+
+
+@pytest.mark.parametrize("d", [64, 120, 250, 440])
+def test_long_runs_without_hubs(d):
+    """The same in graphs dense enough that rows of d entries are no hubs, so that
+    their streams are dealt out of lane order and ordered by bank: a row's run of
+    up to 511 entries goes on over lanes and rounds, and no step may add twice
+    into one sum.  FP32 parity bars against the oracle."""
+    from paper_1409_5000_gb300 import binding as B
+
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for -m gpu tests")
+    n, rng = 3000, np.random.default_rng(d)
+    base = synth.er(n, 60.0 / n, d)
+    src = np.repeat(np.arange(n), np.diff(base.row_ptr.astype(np.int64)))
+    e = [np.stack([src, base.col.astype(np.int64)], axis=1)]
+    e += [np.stack([np.full(d, h), rng.choice(np.arange(200, n), d, replace=False)], axis=1) for h in (3, 4, 40, 41, 77)]
+    e = np.concatenate(e)
+    g = synth.from_edges(n, e[e[:, 0] != e[:, 1]])
+    deg = np.diff(g.row_ptr.astype(np.int64))
+    assert deg.max() <= min(8 * (deg.sum() // n) + 64, 512)  # no hub, and none too long for the streams
+    graphs = [g, synth.er(20_000, 70.0 / 20_000, d + 1)]
+    th_o, S_o = oc.ensemble_scores([(q.n, q.row_ptr, q.col) for q in graphs], 15)
+    with B.GraphSet(graphs, path=B.CB_PATH_FORMATS) as gs:
+        ls, S = B.ensemble_scores(gs, 15, B.CB_FP32)
+        parity.assert_scores(float(ls.item()), S.cpu().numpy(), th_o, S_o, "fp32")

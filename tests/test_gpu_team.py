@@ -124,3 +124,46 @@ def test_small_ensembles_to_fp32_rounding():
             S = B.ensemble_scores(gs, 20, B.CB_FP32)[1].float().double().cpu().numpy()
         err.append(np.linalg.norm(S - S_o) / np.linalg.norm(S_o))
     assert np.mean(err) <= 1.2e-7, err
+
+
+def _is_hub(g):
+    deg = np.diff(g.row_ptr.astype(np.int64))
+    return deg.max() > 8 * (deg.sum() // g.n) + 64
+
+
+@pytest.mark.parametrize("name", ["warp rows", "cta rows"])
+def test_long_rows_in_fp32(name):
+    """FP32 graphs without hubs, which the team kernel takes, whose rows are still
+    too long for the lanes of a row: 1000 rows a CTA and one lane a row, some of
+    them above 32 entries (few enough for the list); a dense graph of teams with
+    rows above 1024 and above 2048."""
+    from paper_1409_5000_gb300 import binding as B
+
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for -m gpu tests")
+    if name == "warp rows":
+        graphs = [synth.er(1000, 24.0 / 999, 900 + q) for q in range(160)]  # more than SMs: a CTA each
+        over = [int((np.diff(g.row_ptr.astype(np.int64)) > 32).sum()) for g in graphs]
+        assert sum(0 < c <= 64 for c in over) > 100
+    else:
+        rng, n = np.random.default_rng(9), 3000
+        base = synth.er(n, 270.0 / n, 31)
+        src = np.repeat(np.arange(n), np.diff(base.row_ptr.astype(np.int64)))
+        e = [np.stack([src, base.col.astype(np.int64)], axis=1)]
+        e += [np.stack([np.full(d, h), rng.choice(np.arange(10, n), d, replace=False)], axis=1)
+              for h, d in ((3, 1400), (4, 2100))]
+        e = np.concatenate(e)
+        graphs = [synth.from_edges(n, e[e[:, 0] != e[:, 1]])]
+        deg = np.diff(graphs[0].row_ptr.astype(np.int64))
+        assert deg[3] > 1024 and deg[4] > 2048
+    assert not any(_is_hub(g) for g in graphs)
+    m = 12
+    th_o, S_o = oc.ensemble_scores([(g.n, g.row_ptr, g.col) for g in graphs], m)
+    with B.GraphSet(graphs) as gs:
+        B.cb_profile_enable(1)
+        ls, S = B.ensemble_scores(gs, m, B.CB_FP32)
+        torch.cuda.synchronize()
+        launches = B.cb_profile_read(B.CB_K_SPMV)[1]
+        B.cb_profile_enable(0)
+        assert launches == 1
+        parity.assert_scores(float(ls.item()), S.cpu().numpy(), th_o, S_o, "fp32")

@@ -371,13 +371,29 @@ def kernel_families(B, step, steps):
 
 
 def spmv_path(ens, csr_only=False):
-    """Which SpMV the workload runs under the automatic path: 'small' (every
-    realisation at most 8192 nodes and 2^20 entries: one launch of m steps),
-    'twophase' (a realisation above 2^19 nodes), 'blocked' (otherwise, when
-    the handle has at least one 16384-row blocked tile per SM) or 'csr'
-    (fewer tiles, or CB_CSR_ONLY)."""
+    """Which SpMV the sizes of a workload suggest under the automatic path:
+    'small' (every realisation at most 8192 nodes and 2^20 entries: one launch
+    of m steps), 'twophase' (a realisation above 2^19 nodes), 'blocked'
+    (otherwise, when the handle has at least one 16384-row blocked tile per SM)
+    or 'csr' (fewer tiles, or CB_CSR_ONLY).  The library's own rule also
+    weighs density, hubs and precision: path_run says what ran."""
     if all(g.n <= 8192 and g.nnz <= (1 << 20) for g in ens.graphs):
         return "small"
+    return per_step_path(ens, csr_only)
+
+
+def path_run(ens, fam, runs, prec=0, csr_only=False):
+    """The path a timed workload took: 'small' (the name of one launch for all m
+    steps, whatever the size: teams of CTAs, or one each) when the profile counted
+    a single launch of the SpMV family for each of its `runs` recurrences, else
+    the per-step path of the sizes."""
+    if fam["spmv"][1] <= runs:
+        return "small"
+    return "csr" if prec == 1 else per_step_path(ens, csr_only)
+
+
+def per_step_path(ens, csr_only=False):
+    """The FP32 path by sizes of a recurrence that runs step by step."""
     if csr_only:
         return "csr"
     if max(g.n for g in ens.graphs) > 32 * 16384:
@@ -388,7 +404,8 @@ def spmv_path(ens, csr_only=False):
     return "blocked" if tiles >= torch.cuda.get_device_properties(0).multi_processor_count else "csr"
 
 
-_KERNEL_NAMES = {"small": "team_lanczos_kernel (all m Lanczos steps of small realisations in one launch)",
+_KERNEL_NAMES = {"small": "team_lanczos_kernel, or lanczos_small_kernel in plain FP64 and with hubs (all m "
+                          "Lanczos steps in one launch)",
                  "blocked": "bspmv_kernel (column-blocked Lanczos SpMV step)",
                  "twophase": "pscatter_kernel + pgather_kernel (two-phase Lanczos SpMV step)",
                  "csr": "spmv_kernel (tiled-CSR Lanczos SpMV step)"}
@@ -538,9 +555,7 @@ def extra_leg(B, name, steps, warmup, dev, csr_only=False, precs=(0,), built=Non
             check_run(B, gs, m, prec)
             units = sum(g.nnz for g in ens.graphs) * m
             fam = kernel_families(B, step, steps)
-            path = spmv_path(ens, csr_only)
-            if path != "small" and prec == 1:
-                path = "csr"
+            path = path_run(ens, fam, (2 if with_grad else 1) * steps, prec, csr_only)
             leg = {"ms_per_step": ms, "value": units / (ms * 1e-3), "unit": UNIT,
                    "dtype": "f64" if prec == 1 else "f32", "roofline": roofline_for(ens, fam, path, m),
                    "gpu_launches_per_step": step_launches(m, path, with_grad)}
@@ -657,7 +672,7 @@ def main():
 
     # per-kernel times (CUDA events around each launch, same stream), separate pass
     fam = kernel_families(B, step, args.steps)
-    path_kind = spmv_path(ens, args.csr_only)
+    path_kind = path_run(ens, fam, (2 if with_grad else 1) * args.steps, csr_only=args.csr_only)
     roofline = roofline_for(ens, fam, path_kind, m)
     launches_per_step = step_launches(m, path_kind, with_grad)
 

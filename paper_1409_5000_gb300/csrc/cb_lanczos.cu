@@ -152,21 +152,23 @@ __device__ __forceinline__ double batch_sum(double (&v)[B]) {
 // with 8 short and 4 longer rows and five CTAs at every width, widths 1, 8, 16
 // and 32 spilled 260 to 340 bytes a thread.  m = 16, one row at a time / that /
 // now, ms: width 1, 8 graphs of 1.5e5 nodes, degree 2.5, 1.28 / 1.32 / 1.22; width 2,
-// degree 5, 1.68 / 1.54 / 1.43; width 4, degree 24, 3.38 / 3.28 / 3.05; width 8,
-// degree 60, 9.04 / 10.8 / 8.89, degree 40, 5.09 / 5.46 / 4.58; width 16, 6 of
-// 1e5, degree 120, 7.38 / 11.9 / 7.20; width 32, 6 of 3e4, degree 300, 5.38 / 5.65 /
-// 4.45.  (Width 4 as the others: 4% slower at degree 10; the others as width 4: 3%
-// slower than one row at a time at degree 40.)  FP32: five CTAs, six spill
-// 20 bytes, within 3% of each other at every width.
-template <typename T, int G>
+// degree 5, 1.68 / 1.54 / 1.43; width 8, degree 60, 9.04 / 10.8 / 8.89, degree 40,
+// 5.09 / 5.46 / 4.58; width 16, 6 of 1e5, degree 120, 7.38 / 11.9 / 7.20; width 32,
+// 6 of 3e4, degree 300, 5.38 / 5.65 / 4.45.  Width 4 has both (SIDE): few entries a
+// row gain from rows side by side, BA(1e5, 5) 0.76 / 0.65 / 0.63 (0.70 as the other
+// widths); from degree kSideDeg on from the sixth CTA, degree 20, one graph of
+// 2.3e5 nodes, m = 10, 0.53 / 0.56 / 0.49 (0.56 with rows side by side).  FP32: six
+// CTAs, one row at a time (five: up to 20% slower where six hold all tiles at once).
+constexpr uint32_t kSideDeg = 16;
+template <typename T, int G, bool SIDE>
 struct SpmvShape {
-  static constexpr int kCtas = sizeof(T) == 4 || G == 4 ? 5 : 6;
-  static constexpr int kSide = G == 4 ? 4 : G < 2 ? G : 2, kSideLong = G == 4 ? 2 : 1;
+  static constexpr int kCtas = SIDE ? 5 : 6;
+  static constexpr int kSide = SIDE ? 4 : G < 2 ? G : 2, kSideLong = SIDE ? 2 : 1;
 };
 // Blocks [0, n_chunks) are heavy-row chunks starting at chunk_off; blocks
 // [n_chunks, ...) are normal tiles starting at tile_off.
-template <typename T, int G>
-__global__ void __launch_bounds__(kThreads, SpmvShape<T, G>::kCtas)
+template <typename T, int G, bool SIDE>
+__global__ void __launch_bounds__(kThreads, SpmvShape<T, G, SIDE>::kCtas)
     spmv_kernel(LArgs a, uint32_t j, uint32_t chunk_off, uint32_t n_chunks, uint32_t tile_off) {
   __shared__ double s_red[32];
   __shared__ uint32_t s_rp[kTileRows + 1];
@@ -228,7 +230,7 @@ __global__ void __launch_bounds__(kThreads, SpmvShape<T, G>::kCtas)
   // so every lane of a warp runs every iteration and the full-mask group
   // shuffles are always converged.
   if constexpr (sizeof(T) == 8) {
-    constexpr int B = SpmvShape<T, G>::kSide, kDup = G / B;
+    constexpr int B = SpmvShape<T, G, SIDE>::kSide, kDup = G / B;
     for (uint32_t it0 = 0; it0 < (uint32_t)G && it0 * kGroups < nrows; it0 += B) {
       // this lane's row of the batch, its operands loaded before the sums
       const uint32_t mine = (it0 + lane_g / kDup) * kGroups + grp;
@@ -395,7 +397,7 @@ __global__ void __launch_bounds__(kThreads, SpmvShape<T, G>::kCtas)
 
   if constexpr (sizeof(T) == 8) {
     // medium rows: warp w takes list entries w, w+8, ..., kR at a time
-    constexpr int kR = SpmvShape<T, G>::kSideLong;
+    constexpr int kR = SpmvShape<T, G, SIDE>::kSideLong;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t nmed = s_nmed;
     for (uint32_t q0 = warp; q0 < nmed; q0 += kR * (kThreads / 32)) {
@@ -430,7 +432,7 @@ __global__ void __launch_bounds__(kThreads, SpmvShape<T, G>::kCtas)
       }
     }
     // long rows: the whole CTA, kL rows at a time, in row order
-    constexpr int kL = SpmvShape<T, G>::kSideLong;
+    constexpr int kL = SpmvShape<T, G, SIDE>::kSideLong;
     __shared__ double s_sums[kL][kThreads / 32];
     const uint32_t nlong = s_nlong;
     for (uint32_t q0 = 0; q0 < nlong; q0 += kL) {
@@ -1189,16 +1191,19 @@ __global__ void __launch_bounds__(kThreads) reorth_update_kernel(LArgs a, uint32
   }
 }
 
-template <typename T, int G>
+template <typename T, int G, bool SIDE = false>
 static void launch_spmv(const LArgs &a, uint32_t j, uint32_t chunk_off, uint32_t n_chunks,
                         uint32_t tile_off, uint32_t n_tiles, cudaStream_t s) {
   const uint32_t grid = n_chunks + n_tiles;
-  if (grid) launch_dep(spmv_kernel<T, G>, grid, kThreads, 0, s, a, j, chunk_off, n_chunks, tile_off);
+  if (grid) launch_dep(spmv_kernel<T, G, SIDE>, grid, kThreads, 0, s, a, j, chunk_off, n_chunks, tile_off);
 }
 
 template <typename T>
-static void launch_spmv_lanes(int lanes, const LArgs &a, uint32_t j, uint32_t co, uint32_t nc,
+static void launch_spmv_lanes(int lanes, bool side, const LArgs &a, uint32_t j, uint32_t co, uint32_t nc,
                               uint32_t to, uint32_t nt, cudaStream_t s) {
+  if constexpr (sizeof(T) == 8) {
+    if (lanes == 4 && side) return launch_spmv<T, 4, true>(a, j, co, nc, to, nt, s);
+  }
   switch (lanes) {
     case 1: launch_spmv<T, 1>(a, j, co, nc, to, nt, s); break;
     case 2: launch_spmv<T, 2>(a, j, co, nc, to, nt, s); break;
@@ -1362,9 +1367,10 @@ static int run_t(cb_graph *h, Workspace &W, uint32_t r0, uint32_t r1, uint32_t m
     prof_end(tok, s);
     return cuda_error(cudaGetLastError(), "lanczos launch");
   }
+  const bool side = h->total_nnz < kSideDeg * h->total_nodes_padded;
   for (uint32_t j = 0; j < m; ++j) {
     tok = prof_begin(CB_K_SPMV, s);
-    if (any_csr) launch_spmv_lanes<T>(h->lanes, a, j, chunk_off, n_chunks, tile_off, n_tiles, s);
+    if (any_csr) launch_spmv_lanes<T>(h->lanes, side, a, j, chunk_off, n_chunks, tile_off, n_tiles, s);
     if (n_btiles) launch_dep(bspmv_kernel, n_btiles, kBThreads, kBSmemBytes, s, a, j, btile_off);
     if (any_pb)
       launch_twophase(a, h->lanes, j, ptile_lo, ptile_hi, pg_lo, pg_hi, chunk_off, n_chunks,

@@ -13,5 +13,5 @@ def test_spmv_kernels_do_not_spill(tmp_path):
     log = _build._run(cmd + _build.nvcc_flags(["-Xptxas", "-v"]))
     names = re.findall(r"Function properties for (\S+)\n\s+\d+ bytes stack frame, (\d+) bytes spill stores", log)
     spills = {n: int(b) for n, b in names if re.search(r"\d+spmv_kernelI[fd]Li\d+E", n) and "bspmv" not in n}
-    assert len(spills) == 12, log[-2000:]
+    assert len(spills) == 13, log[-2000:]  # FP64 at width 4 in two shapes
     assert max(spills.values()) <= 32, spills

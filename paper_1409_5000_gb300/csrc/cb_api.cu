@@ -796,19 +796,20 @@ static int upload_impl(uint32_t n_inst, const uint32_t *n, const uint64_t *nnz,
   // with the fill last, 45 so).
   BlockedBuild bb;
   int rc = blocked_count(h, s, cp.groups, bb);
-  if (rc == CB_OK) {
+  const bool fill_first = dev && h->total_btiles > 0;
+  auto set_longest = [&](InstDesc &I, uint32_t most) {
+    I.longest = most;
+    I.hubs = (uint64_t)most > (uint64_t)kHubTimes * I.nnz / I.n + kHubRows;
+  };
+  if (rc == CB_OK && fill_first) {
     parallel_for(n_inst, node_off / 4, [&](uint32_t r) {  // a loop of maxima, a quarter of a scan
       const uint32_t *rp = rp_of(r);
-      InstDesc &I = h->inst[r];
       uint32_t most = 0;
-      for (uint32_t i = 0; i < I.n; ++i) most = std::max(most, rp[i + 1] - rp[i]);
-      I.longest = most;
-      I.hubs = (uint64_t)most > (uint64_t)kHubTimes * I.nnz / I.n + kHubRows;
+      for (uint32_t i = 0; i < h->inst[r].n; ++i) most = std::max(most, rp[i + 1] - rp[i]);
+      set_longest(h->inst[r], most);
     });
-    if (dev) {
-      chk(stage_h2d(h->d_inst, h->inst.data(), n_inst * sizeof(InstDesc), s));
-      rc = e == cudaSuccess ? blocked_fill(h, s, bb) : cuda_error(e, "cb_graph_upload: copy");
-    }
+    chk(stage_h2d(h->d_inst, h->inst.data(), n_inst * sizeof(InstDesc), s));
+    rc = e == cudaSuccess ? blocked_fill(h, s, bb) : cuda_error(e, "cb_graph_upload: copy");
   }
   if (rc != CB_OK) {
     cp.finish();
@@ -826,9 +827,10 @@ static int upload_impl(uint32_t n_inst, const uint32_t *n, const uint64_t *nnz,
   std::vector<std::vector<uint32_t>> heavy_rows(n_inst), tile_starts(n_inst);
   parallel_for(n_inst, node_off, [&](uint32_t r) {
     const uint32_t *rp = rp_of(r);
-    uint32_t rows = 0, acc = 0;
+    uint32_t rows = 0, acc = 0, most = 0;
     for (uint32_t i = 0; i < h->inst[r].n; ++i) {
       const uint32_t deg = rp[i + 1] - rp[i];
+      most = std::max(most, deg);
       if (deg > kHeavyDeg) heavy_rows[r].push_back(i);
       const uint32_t w = deg > kHeavyDeg ? 0u : deg;
       if (rows == 0 || rows == (uint32_t)kTileRows || (acc > 0 && acc + w > kTileNnz)) {
@@ -839,6 +841,7 @@ static int upload_impl(uint32_t n_inst, const uint32_t *n, const uint64_t *nnz,
       ++rows;
       acc += w;
     }
+    set_longest(h->inst[r], most);
   });
   for (uint32_t r = 0; r < n_inst; ++r) {
     h->inst[r].tile_base = tile_off;
@@ -938,7 +941,7 @@ static int upload_impl(uint32_t n_inst, const uint32_t *n, const uint64_t *nnz,
   std::vector<const uint32_t *> rpv(n_inst);
   for (uint32_t r = 0; r < n_inst; ++r) rpv[r] = rp_of(r);
   rc = blocked_long_rows(h, rpv, s);
-  if (rc == CB_OK && !dev) rc = blocked_fill(h, s, bb);
+  if (rc == CB_OK && !fill_first) rc = blocked_fill(h, s, bb);
   if (rc == CB_OK) rc = build_twophase(h, rpv, s, cp.groups, h->force_pb);
   if (rc == CB_OK) {  // every copy has landed before the handle is returned
     for (const CopyGroup &g : cp.groups) chk(cudaStreamWaitEvent(s, g.ev, 0));

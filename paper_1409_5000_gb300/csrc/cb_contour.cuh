@@ -47,13 +47,6 @@ __device__ __forceinline__ double rcp_nr(double r) {
   return fma(y, fma(-r, y, 1.0), y);
 }
 
-// 1 / sqrt(x) for x in the normal FP32 range, as rcp_nr: y <- y + y/2 (1 - x y^2).
-__device__ __forceinline__ double rsqrt_nr(double x) {
-  double y = (double)rsqrtf((float)x);
-  y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
-  return fma(0.5 * y, fma(-x * y, y, 1.0), y);
-}
-
 // FP32 Laguerre terms at x from f'/f and (f'/f)^2 - f''/f of f(x) = det(xI - T),
 // through the ratios r_k = p_k / p_{k-1} of the leading principal minors (one
 // reciprocal per k), which cannot overflow.  a: diagonal, b2: squared
@@ -101,7 +94,7 @@ struct Spectrum {
 //  1. FP32 multisection: x lies above the spectrum iff every pivot of xI - T
 //     is positive; the 32 lanes test 32 points of the bracket at once, so a
 //     round costs M dependent FP32 steps and gains a factor of 33; four
-//     rounds reach FP32 resolution, sigma just above lambda_max.
+//     rounds leave a bracket of 2e-6 lambda_max, sigma its upper end.
 //  2. two inverse iterations with sigma I - T (positive definite) in FP32.
 //  3. the Rayleigh quotient in FP64, as rho + v.(T - rho)v / v.v from rho =
 //     sigma, one correction of v from its FP64 residual by an FP32 solve, and
@@ -259,7 +252,7 @@ __device__ inline double lambda_max(const double *al, const double *be, int M, S
 // result: the convergence is cubic, so the FP32 estimate turns into an
 // FP64-accurate one.  Not always: where the FP32 iterate ends below lambda_max,
 // an FP64 step meets a pivot that is not positive and is left out, and theta
-// stays up to 4e-8 short (relative; 4 of 48 ER, WS and BA graphs of 900 to 8500
+// stays up to 4e-8 short (relative; 3 of 48 ER, WS and BA graphs of 900 to 8500
 // nodes at m = 30, the others within 6e-15); over copies of lambda_max (T without
 // reorthogonalisation) it stops up to 1.2e-7 above.  exp(theta) y does not depend
 // on it, but theta and y are results that callers compare and store to FP64
@@ -340,10 +333,14 @@ __device__ inline double lambda_max_laguerre(const double *al, const double *be,
   return x;
 }
 
-// The two differ where T carries copies of lambda_max, in FP32 recurrences by up
-// to 1.2e-7 lambda_max: 2e-5 of every score on a BA graph of 1e7 nodes
-// (lambda_max 158), which callers that compare or store FP32 scores would
-// see.  So above kCopiesShow Laguerre's value stays the result there too.
+// FP32 recurrences: lambda_max is the nearer of the two to the largest eigenvalue
+// of A's Krylov matrix (against a dense FP64 eigensolver on T of a fully
+// reorthogonalised FP64 run; 24 cliques in sparse graphs, ER and BA graphs of
+// lambda_max 19 to 201, m = 30 and 35: 7.3e-8 of lambda_max off on average, 2.4e-7 at
+// most; Laguerre's 4.4e-7 and 8.7e-7, from above, over the copies that T carries).
+// But every score is scaled by exp(-theta): above kCopiesShow the difference is
+// some 2e-5 of each, which callers that compare or store FP32 scores with earlier
+// ones would see, and Laguerre's value stays.  (FP64: its method alone.)
 constexpr double kCopiesShow = 48.0;
 
 __device__ inline double largest(const double *al, const double *be, int M, Spectrum &S, bool laguerre) {

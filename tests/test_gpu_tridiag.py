@@ -73,3 +73,24 @@ def test_shift_is_one_in_both_fp64_modes(graph):
     ls, ls_r, y, y_r = float(ls.item()), float(ls_r.item()), y.cpu().numpy(), y_r.cpu().numpy()
     assert abs(ls - ls_r) <= 1e-12 * ls
     assert np.max(np.abs(y - y_r)) <= 1e-12 * y.max()
+
+
+@pytest.mark.parametrize("q", [20, 30, 40, 47, 49, 50, 80, 120, 200])
+def test_fp32_shift_on_both_sides_of_the_methods(q):
+    """theta of FP32 recurrences against the oracle's (dense eigensolver on T of a
+    reorthogonalised FP64 run), T full of copies of it: within five units of FP32
+    roundoff (3e-7, T's own entries) by bracketing, below lambda_max = 48, and
+    within the relative step at which the other method's FP32 stage stops (1e-6)
+    above."""
+    from paper_1409_5000_gb300 import binding as B
+
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for -m gpu tests")
+    rng, n = np.random.default_rng(q), 2000
+    e = [rng.integers(0, n, (n, 2)), np.array([(a, b) for a in range(q) for b in range(a)])]
+    e = np.concatenate(e)
+    g = synth.from_edges(n, e[e[:, 0] != e[:, 1]])
+    th_o = oc.krylov_expv(g.n, g.row_ptr, g.col, 35)[0]
+    with B.GraphSet([g]) as gs:
+        th = float(B.communicability(gs, 0, 35, B.CB_FP32)[0].item())
+    assert abs(th - th_o) <= (3e-7 if th_o < 47.9 else 1e-6) * th_o

@@ -73,7 +73,8 @@ extern "C" {
                              stay on the chip and a cost model prefers it (FP64 with
                              reorthogonalisation; FP32 ensembles and realisations of n <= 8192,
                              without hubs or reorthogonalisation), or by one CTA each (n <= 8192
-                             and <= 2^20 entries: FP64, FP32 with hubs); otherwise, per step, the
+                             and <= 2^20 entries: FP64, FP32 with hubs or too dense for a team
+                             where the model prefers it); otherwise, per step, the
                              column-blocked kernel when the handle has >= one blocked tile per
                              SM, two-phase kernels where built, else tiled CSR */
 #define CB_PATH_FORMATS 1 /* column-blocked and two-phase kernels wherever their format was built */

@@ -26,7 +26,7 @@
 //
 // Measured, us per step before (one CTA with its rows' chains of global loads up
 // to 8192 nodes, three launches a step above) and now: 10 x 500 nodes FP32 7.0 ->
-// 3.5; 40 x 4000 36 -> 6.6; 8 x 30000 32 -> 12; FP64 with reorthogonalisation,
+// 3.8; 40 x 4000 36 -> 6.8; 8 x 30000 32 -> 12; FP64 with reorthogonalisation,
 // one graph of 1e5 nodes: 118 -> 43.  An FP64 instruction takes its sub-core 65
 // cycles per warp, so scalars and splits are formed by one warp.
 //
